@@ -363,9 +363,12 @@ def _plain_solve(A, b, iters):
     """Textbook Jacobi-preconditioned BiCGStab from zero, plain 64-bit arithmetic."""
     M = _plain(A)
     rows = torch.repeat_interleave(torch.arange(A.n, device=DEV), A.rowptr.diff())
-    d = torch.zeros(A.n, dtype=torch.float64, device=DEV)
     hit = A.col.to(torch.int64) == rows
-    d[rows[hit].flip(0)] = A.val[hit].flip(0)
+    at, diag = rows[hit], A.val[hit]
+    first = torch.ones_like(at, dtype=torch.bool)
+    first[1:] = at[1:] != at[:-1]  # the first stored (i, i) of a row with several
+    d = torch.zeros(A.n, dtype=torch.float64, device=DEV)
+    d[at[first]] = diag[first]
     x, r, r0, p = torch.zeros_like(b), b.clone(), b.clone(), b.clone()
     rho = torch.dot(r0, r)
     for _ in range(iters):
