@@ -248,16 +248,16 @@ Cfg grid_for(Workspace *w, int64_t items, int block, int per_sm) {
     return c;
 }
 
-// Exact-dot launch shape: a persistent grid of whole waves (blocks_per_sm
-// resident blocks on every SM), and never more than 2^20 products per thread
-// per launch (the register window's headroom).
-Cfg persistent_cfg(Workspace *w, int64_t n, int blocks_per_sm, int block) {
+// Exact-dot launch shape for each of k dots: together a persistent grid of whole
+// waves (blocks_per_sm resident blocks on every SM), and never more than 2^20
+// products per thread per launch (the windows' headroom).
+Cfg persistent_cfg(Workspace *w, int64_t n, int blocks_per_sm, int block, int k = 1) {
     Cfg c;
     c.block = block;
     int64_t g = p_exdot_grid.load();
     if (g <= 0) {
         int64_t need = (n + 2LL * c.block - 1) / (2LL * c.block);
-        int64_t cap = (int64_t)w->sms * blocks_per_sm;
+        int64_t cap = std::max<int64_t>((int64_t)w->sms * blocks_per_sm / k, 1);
         g = need < 1 ? 1 : (need < cap ? need : cap);
     }
     int64_t minimum = (n + ((int64_t)c.block << 20) - 1) / ((int64_t)c.block << 20);
@@ -268,7 +268,7 @@ Cfg persistent_cfg(Workspace *w, int64_t n, int blocks_per_sm, int block) {
 }
 Cfg exdot_cfg(Workspace *w, int64_t n, int k, int window) {
     const int block = block_of(p_exdot_block.load(), 256);
-    return persistent_cfg(w, n, exdot_blocks_per_sm(k, window, block, n), block);
+    return persistent_cfg(w, n, exdot_blocks_per_sm(window, block), block, k);
 }
 
 // Shared-memory carveout of the staging kernels. Measured on GB300 (Poisson
@@ -283,7 +283,7 @@ int carveout_param() {
 
 int window_param() {
     int64_t q = p_exdot_window.load();
-    return (q == 1 || q == 2 || q == 4) ? (int)q : 4;
+    return (q == 1 || q == 2) ? (int)q : 0;
 }
 
 // Per-kernel CUDA events. Kernels enqueued back to back share events: a
@@ -513,7 +513,7 @@ int rbs_exdot_partial(const double *x, const double *y, int64_t n, int64_t *limb
         CK(cudaMemsetAsync(flags, 0, sizeof(int32_t), w->stream));
         return RBS_OK;
     }
-    CK(launch_exdot_partial(x, y, n, w->g, limbs, flags, 4, exdot_cfg(w, n, 1, 4), w->stream));
+    CK(launch_exdot_partial(x, y, n, w->g, limbs, flags, exdot_cfg(w, n, 1, 0), w->stream));
     return RBS_OK;
 }
 

@@ -23,7 +23,7 @@ constexpr uint32_t F_NAN = 1u, F_PINF = 2u, F_NINF = 4u;
 struct DotScratch {
     unsigned long long limbs[KMAX][NL];
     unsigned int flags[KMAX];
-    unsigned int ticket;
+    unsigned int ticket[KMAX];
     unsigned int err;  // sticky workspace error word (bad CSR index seen)
 };
 

@@ -119,42 +119,6 @@ __device__ __forceinline__ void win_place_add(Win<Q> &W, const uint32_t (&u)[5],
     add8_carry(W.w, v, SIGNED ? (m & 1u) : 0u);
 }
 
-// win_place_add for windows anchored top-aligned (products of the anchor's
-// limb land at q = Q - 1): with Q = 4 the placements q = 2, 3 take the first
-// select level only and a branch picks the word layout, so the common case of
-// products within two limbs skips the second level (a branch that is uniform
-// across the warp on well-scaled data; divergent warps run both layouts, which
-// costs about what the second select level does).
-template <int Q>
-__device__ __forceinline__ void win_place_add_top(Win<Q> &W, const uint32_t (&u)[5], int q, uint32_t m) {
-    if (Q != 4) {
-        win_place_add<Q, true>(W, u, q, m);
-        return;
-    }
-    uint32_t x[5], t[6], v[8];
-#pragma unroll
-    for (int k = 0; k < 5; k++) x[k] = u[k] ^ m;
-    const bool b1 = (q & 1) != 0;
-    t[0] = b1 ? m : x[0];
-    t[1] = b1 ? x[0] : x[1];
-    t[2] = b1 ? x[1] : x[2];
-    t[3] = b1 ? x[2] : x[3];
-    t[4] = b1 ? x[3] : x[4];
-    t[5] = b1 ? x[4] : m;
-    if (q & 2) {
-        v[0] = m;
-        v[1] = m;
-#pragma unroll
-        for (int k = 0; k < 6; k++) v[k + 2] = t[k];
-    } else {
-#pragma unroll
-        for (int k = 0; k < 6; k++) v[k] = t[k];
-        v[6] = m;
-        v[7] = m;
-    }
-    add8_carry(W.w, v, m & 1u);
-}
-
 // Add a signed 64-bit value to a limb of a block accumulator in shared memory
 // with two 32-bit atomics: the low word's add returns the old low word, which
 // gives that add's carry into the high word. Measured on GB300 with four lanes
@@ -291,76 +255,6 @@ __device__ __forceinline__ bool prod_exact(double x, double y, uint32_t &flags, 
     L = pos >> 5;
     shift5((uint32_t)m00, (uint32_t)m10, (uint32_t)m11, (uint32_t)(m11 >> 32), (uint32_t)pos & 31u, u);
     return true;
-}
-
-// Two windows per thread: H takes the product if it fits; a product above H
-// re-anchors H at it and the old H becomes the low window L; a product below H
-// goes to L (anchoring or re-anchoring it when it is empty or lies between L and
-// H); only products below both go to shared memory. Wide-exponent sums (the
-// ill-conditioned dots) then rarely touch shared memory.
-template <int Q>
-__device__ __forceinline__ void exact_add2(Win<Q> &H, Win<Q> &Lw, uint32_t &flags, unsigned long long *sacc,
-                                           double x, double y) {
-    const uint32_t xh = (uint32_t)__double2hiint(x), xl = (uint32_t)__double2loint(x);
-    const uint32_t yh = (uint32_t)__double2hiint(y), yl = (uint32_t)__double2loint(y);
-    const uint32_t exm = xh & 0x7ff00000u, eym = yh & 0x7ff00000u;  // biased exponents << 20
-    uint32_t A1, B1;
-    int pos;
-    if (exm - 0x00100000u < 0x7fe00000u && eym - 0x00100000u < 0x7fe00000u) {
-        // both operands normal (the common case): implicit bit set, no zero
-        A1 = (xh & 0xfffffu) | 0x100000u;
-        B1 = (yh & 0xfffffu) | 0x100000u;
-        pos = (int)((exm >> 20) + (eym >> 20)) - 2;
-    } else {
-        const uint32_t ex = exm >> 20, ey = eym >> 20;
-        if (ex == 0x7ffu || ey == 0x7ffu) {
-            flags |= special_flags(xh, xl, yh, yl);
-            return;
-        }
-        A1 = (xh & 0xfffffu) | (ex ? 0x100000u : 0u);
-        B1 = (yh & 0xfffffu) | (ey ? 0x100000u : 0u);
-        if ((A1 | xl) == 0u || (B1 | yl) == 0u) return;
-        pos = (int)max(ex, 1u) + (int)max(ey, 1u) - 2;
-    }
-    const unsigned long long m00 = (unsigned long long)xl * yl;
-    const unsigned long long m01 = (unsigned long long)xl * B1 + (m00 >> 32);
-    const unsigned long long m10 = (unsigned long long)A1 * yl + (uint32_t)m01;
-    const unsigned long long m11 =
-        (unsigned long long)A1 * B1 + (unsigned long long)((uint32_t)(m01 >> 32) + (uint32_t)(m10 >> 32));
-    const uint32_t p0 = (uint32_t)m00, p1 = (uint32_t)m10, p2 = (uint32_t)m11, p3 = (uint32_t)(m11 >> 32);
-    const uint32_t m = (uint32_t)((int32_t)(xh ^ yh) >> 31);
-    const int L = pos >> 5;
-    uint32_t u[5];
-    shift5(p0, p1, p2, p3, (uint32_t)pos & 31u, u);
-    const int q = L - H.a;
-    if ((unsigned)q < (unsigned)Q) {
-        win_place_add_top<Q>(H, u, q, m);
-        return;
-    }
-    const int back = Q - 1;  // top-aligned: the anchoring product at q = Q - 1
-    if (q >= Q) {
-        if (H.a != WIN_EMPTY) {
-            win_flush<Q>(Lw, sacc);
-            Lw = H;
-        }
-#pragma unroll
-        for (int k = 0; k < 8; k++) H.w[k] = 0u;
-        H.a = L - back < 0 ? 0 : L - back;
-        win_place_add_top<Q>(H, u, L - H.a, m);
-        return;
-    }
-    const int ql = L - Lw.a;
-    if ((unsigned)ql < (unsigned)Q) {
-        win_place_add_top<Q>(Lw, u, ql, m);
-        return;
-    }
-    if (ql >= Q) {
-        win_flush<Q>(Lw, sacc);
-        Lw.a = L - back < 0 ? 0 : L - back;
-        win_place_add_top<Q>(Lw, u, L - Lw.a, m);
-        return;
-    }
-    smem_deposit(sacc, u, L, m);
 }
 
 // Warp-cooperative flush of every lane's window (all 32 lanes call it). The
@@ -516,12 +410,13 @@ static __device__ __noinline__ double round_limbs_thread(long long *G, uint32_t 
 // reduction (the whole grid unless given) calls it. Returns true in the block
 // that finishes last; there the rounded values are in vals[0..K-1] (shared
 // memory) after a barrier, or, with export_limbs, the partially normalised
-// limbs of the first reduction are in limbs_out.
+// limbs of the first reduction are in limbs_out. The reductions use g's
+// accumulators slot .. slot + K - 1 and ticket `slot`.
 template <int K>
 __device__ __forceinline__ bool block_grid_finish(const uint32_t (&flags)[K], unsigned long long (*sacc)[NL],
                                                   uint32_t *sflags, DotScratch *g, double *vals,
                                                   bool export_limbs = false, long long *limbs_out = nullptr,
-                                                  int32_t *flags_out = nullptr, unsigned nblk = 0u) {
+                                                  int32_t *flags_out = nullptr, unsigned nblk = 0u, int slot = 0) {
     // nonzero limb span of each reduction, found while the last block reads
     // the limbs back (so that its rounding need not scan all NL of them)
     __shared__ int s_span[K][2];
@@ -536,28 +431,28 @@ __device__ __forceinline__ bool block_grid_finish(const uint32_t (&flags)[K], un
     for (int idx = threadIdx.x; idx < K * NL; idx += blockDim.x) {
         const int k = idx / NL, j = idx - k * NL;
         const long long v = partial_norm(sacc[k], j);
-        if (v) atomicAdd(&g->limbs[k][j], (unsigned long long)v);
+        if (v) atomicAdd(&g->limbs[slot + k][j], (unsigned long long)v);
     }
-    if (threadIdx.x < K && sflags[threadIdx.x]) atomicOr(&g->flags[threadIdx.x], sflags[threadIdx.x]);
+    if (threadIdx.x < K && sflags[threadIdx.x]) atomicOr(&g->flags[slot + threadIdx.x], sflags[threadIdx.x]);
     __threadfence();
     __syncthreads();
     __shared__ bool s_last;
-    if (threadIdx.x == 0) s_last = (atomicAdd(&g->ticket, 1u) == (nblk ? nblk : gridDim.x) - 1);
+    if (threadIdx.x == 0) s_last = (atomicAdd(&g->ticket[slot], 1u) == (nblk ? nblk : gridDim.x) - 1);
     __syncthreads();
     if (!s_last) return false;
     __threadfence();
     // read back (and clear) the global accumulators into shared memory
     for (int idx = threadIdx.x; idx < K * NL; idx += blockDim.x) {
         const int k = idx / NL, j = idx - k * NL;
-        const unsigned long long v = atomicExch(&g->limbs[k][j], 0ull);
+        const unsigned long long v = atomicExch(&g->limbs[slot + k][j], 0ull);
         sacc[k][j] = v;
         if (v) {
             atomicMin(&s_span[k][0], j);
             atomicMax(&s_span[k][1], j);
         }
     }
-    if (threadIdx.x < K) sflags[threadIdx.x] = atomicExch(&g->flags[threadIdx.x], 0u);
-    if (threadIdx.x == 0) g->ticket = 0u;
+    if (threadIdx.x < K) sflags[threadIdx.x] = atomicExch(&g->flags[slot + threadIdx.x], 0u);
+    if (threadIdx.x == 0) g->ticket[slot] = 0u;
     __syncthreads();
     if (export_limbs) {
         for (int idx = threadIdx.x; idx < NL; idx += blockDim.x)

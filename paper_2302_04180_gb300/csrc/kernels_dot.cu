@@ -1,36 +1,153 @@
-// Standalone kernels: exact dot (single and multi-output; window size Q = 4
-// here, Q = 1 and 2 in kernels_exdot_w1.cu / _w2.cu), long-accumulator export
-// and rounding, the allocation-free exact dot, the FPE-8 dot.
+// Standalone kernels: exact dot (single and multi-output), long-accumulator
+// export and rounding, the allocation-free exact dot, the FPE-8 dot.
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <tuple>
-#include <type_traits>
 
-#include "exdot.cuh"
+#include "kernels.cuh"
+#include "launch.h"
 
 namespace rbs {
 
+struct DotArgs {
+    const double *x[KMAX];
+    const double *y[KMAX];
+};
+
+// Pairs of each operand that a thread loads at once, and blocks per SM to keep
+// registers for. The loads in flight set the rate: two pairs at three blocks
+// (80 registers) stream 2^27 products in 331 us, one pair at four blocks in 334,
+// two at four in 346 (64 registers spill).
+constexpr int EXDOT_PAIRS = 2, EXDOT_BLOCKS = 3;
+
+// U pairs into the windows.
+template <int U, class R>
+__device__ __forceinline__ void add_pairs(R &red, const double2 (&x)[U], const double2 (&y)[U]) {
+    double xv[2 * U], yv[2 * U];
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+        xv[2 * u] = x[u].x;
+        xv[2 * u + 1] = x[u].y;
+        yv[2 * u] = y[u].x;
+        yv[2 * u + 1] = y[u].y;
+    }
+    red.template add<2 * U>(xv, yv);
+}
+
+// Exact dots over the same length (Sec. 2 exdot; Sec. 4.1/4.2 merged
+// reductions): the blocks of row blockIdx.y take dot blockIdx.y, W the words
+// per sign of their windows. Aligned operands go through 16-byte loads, the
+// next pairs in flight while these are added, so that the stream does not stop
+// for the products.
+//
+// Several dots share the launch but not their blocks: five dots' windows in one
+// thread left two blocks per SM, and issue slots empty (2 million elements: 41
+// us against 30 now); an operand that several dots name comes from L2 for all
+// but the first of them, since their blocks walk the vectors together.
+// Bound by HBM once long (2^27: 331 us, 0.96 of the copy rate, cond 1; 378 with
+// 64-bit digits) and by the windows' set-up, flush and cross-block sum when
+// short (2^24: 49 us, 39.5 of them HBM's; cond 1e48: 54 against 73).
+template <int W, bool EXPORT>
+__global__ void __launch_bounds__(256, EXDOT_BLOCKS)
+    k_exdot(const __grid_constant__ DotArgs a, int64_t n, DotScratch *g, double *out, long long *limbs, int32_t *flags_out) {
+    using R = ExactW<W>;
+    R red;
+    const int slot = EXPORT ? 0 : blockIdx.y;
+    const double *__restrict__ xp = a.x[slot], *__restrict__ yp = a.y[slot];
+    const int64_t st = gstride();
+    if (((reinterpret_cast<uintptr_t>(xp) | reinterpret_cast<uintptr_t>(yp)) & 15) == 0) {
+        constexpr int U = EXDOT_PAIRS;
+        const double2 *x2 = reinterpret_cast<const double2 *>(xp), *y2 = reinterpret_cast<const double2 *>(yp);
+        const int64_t n2 = n >> 1;
+        int64_t j = gtid();
+        // the pair that opens the windows; a thread without one adds zeros
+        double2 x0[1] = {make_double2(0.0, 0.0)}, y0[1] = {make_double2(0.0, 0.0)};
+        if (j < n2) {
+            x0[0] = __ldcs(x2 + j);
+            y0[0] = __ldcs(y2 + j);
+        }
+        j += st;
+        // then `full` steps of U pairs per thread, two steps per turn of the
+        // loop with the loads of each ahead of the adds of the other
+        const int64_t full = n2 > st ? (n2 - st) / (U * st) : 0;
+        double2 xa[U], ya[U], xb[U], yb[U];
+        auto load = [&](double2 (&xv)[U], double2 (&yv)[U]) {
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                xv[u] = __ldcs(x2 + j);
+                yv[u] = __ldcs(y2 + j);
+                j += st;
+            }
+        };
+        if (full > 0) load(xa, ya);
+        red.init();
+        red.open(max(R::limb_of(x0[0].x, y0[0].x), R::limb_of(x0[0].y, y0[0].y)));
+        add_pairs<1>(red, x0, y0);
+        int64_t s = 0;
+        for (; s + 2 < full; s += 2) {
+            load(xb, yb);
+            add_pairs<U>(red, xa, ya);
+            load(xa, ya);
+            add_pairs<U>(red, xb, yb);
+        }
+        if (s + 1 < full) {
+            load(xb, yb);
+            add_pairs<U>(red, xa, ya);
+            add_pairs<U>(red, xb, yb);
+        } else if (s < full) {
+            add_pairs<U>(red, xa, ya);
+        }
+        for (; j < n2; j += st) {
+            x0[0] = __ldcs(x2 + j);
+            y0[0] = __ldcs(y2 + j);
+            add_pairs<1>(red, x0, y0);
+        }
+        if ((n & 1) && gtid() == 0) red.add_one(xp[n - 1], yp[n - 1]);
+    } else {
+        int64_t i = gtid();
+        red.init();
+        red.open(i < n ? R::limb_of(xp[i], yp[i]) : -1);
+        for (; i < n; i += st) red.add_one(xp[i], yp[i]);
+    }
+    __shared__ double val[1];
+    if (red.finish(g, slot, val, EXPORT, limbs, flags_out) && !EXPORT && threadIdx.x == 0) out[slot] = val[0];
+}
+
+// Words per sign for the "exdot.window" knob: 16 unless it asks for a small
+// window (1 or 2). 12 placements hold the products of 2^-128 .. 2^128 and more
+// around a block's first ones without re-anchoring.
+template <class F>
+static auto with_window(int window, F &&f) {
+    if (window == 1) return f(k_exdot<6, false>);
+    if (window == 2) return f(k_exdot<7, false>);
+    return f(k_exdot<16, false>);
+}
+
 // Cached per device and kernel variant: the query costs a few microseconds of
 // host time, which a short dot would otherwise pay on every call.
-int exdot_blocks_per_sm(int k, int window, int block, int64_t n) {
+int exdot_blocks_per_sm(int window, int block) {
     static std::mutex mu;
-    static std::map<std::tuple<int, int, int, int, bool>, int> cache;
-    const bool smem = k <= 2 && n >= EXDOT_SMEM_MIN_N;
+    static std::map<std::tuple<int, int, int>, int> cache;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) {
         cudaGetLastError();
         dev = -1;
     }
-    const auto key = std::make_tuple(dev, k, window, block, smem);
+    const auto key = std::make_tuple(dev, window, block);
     {
         std::lock_guard<std::mutex> lk(mu);
         const auto it = cache.find(key);
         if (it != cache.end()) return it->second;
     }
-    int nb;
-    if (window == 2) nb = exdot_occ_w2(k, block, smem);
-    else if (window == 1) nb = exdot_occ_w1(k, block, smem);
-    else nb = smem ? exdot_occ_q<4, true>(k, block) : exdot_occ_q<4, false>(k, block);
+    const int nb = with_window(window, [&](auto kern) {
+        int v = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, kern, block, 0) != cudaSuccess || v < 1) {
+            cudaGetLastError();
+            v = 1;
+        }
+        return v;
+    });
     std::lock_guard<std::mutex> lk(mu);
     cache[key] = nb;
     return nb;
@@ -38,24 +155,24 @@ int exdot_blocks_per_sm(int k, int window, int block, int64_t n) {
 
 cudaError_t launch_exdot(int k, const double *const *xs, const double *const *ys, int64_t n,
                          DotScratch *g, double *out, int window, Cfg cfg, cudaStream_t s) {
-    if (window == 2) return launch_exdot_w2(k, xs, ys, n, g, out, cfg, s);
-    if (window == 1) return launch_exdot_w1(k, xs, ys, n, g, out, cfg, s);
-    return exdot_q<4>(k, xs, ys, n, g, out, cfg, s);
+    if (k < 1 || k > KMAX) return cudaErrorInvalidValue;
+    DotArgs a{};
+    for (int j = 0; j < k; j++) {
+        a.x[j] = xs[j];
+        a.y[j] = ys[j];
+    }
+    return with_window(window, [&](auto kern) {
+        kern<<<dim3((unsigned)cfg.grid, (unsigned)k), cfg.block, 0, s>>>(a, n, g, out, nullptr, nullptr);
+        return cudaGetLastError();
+    });
 }
 
 cudaError_t launch_exdot_partial(const double *x, const double *y, int64_t n, DotScratch *g,
-                                 int64_t *limbs, int32_t *flags, int window, Cfg cfg, cudaStream_t s) {
-    (void)window;
-    DotArgs<1> a;
+                                 int64_t *limbs, int32_t *flags, Cfg cfg, cudaStream_t s) {
+    DotArgs a{};
     a.x[0] = x;
     a.y[0] = y;
-    const bool aligned = ((uintptr_t)x % 16 == 0) && ((uintptr_t)y % 16 == 0);
-    if (n >= EXDOT_SMEM_MIN_N)
-        k_exdot<1, 4, true, true><<<cfg.grid, cfg.block, 0, s>>>(a, n, aligned, g, nullptr, (long long *)limbs,
-                                                              flags);
-    else
-        k_exdot<1, 4, true, false><<<cfg.grid, cfg.block, 0, s>>>(a, n, aligned, g, nullptr, (long long *)limbs,
-                                                               flags);
+    k_exdot<16, true><<<cfg.grid, cfg.block, 0, s>>>(a, n, g, nullptr, (long long *)limbs, flags);
     return cudaGetLastError();
 }
 
@@ -167,12 +284,12 @@ extern "C" int rbs_exdot_noalloc(int k, const double *const *xs, const double *c
     Cfg c;
     c.block = 256;
     int64_t g = (n + 2LL * c.block - 1) / (2LL * c.block);
-    const int64_t cap = (int64_t)sms * exdot_blocks_per_sm(k, 4, c.block, n);  // whole waves
+    const int64_t cap = std::max<int64_t>((int64_t)sms * exdot_blocks_per_sm(0, c.block) / k, 1);  // whole waves
     g = g < 1 ? 1 : (g < cap ? g : cap);
     const int64_t minimum = (n + ((int64_t)c.block << 20) - 1) / ((int64_t)c.block << 20);
     if (g < minimum) g = minimum;
     c.grid = (int)(g > 0x7fffffff ? 0x7fffffff : g);
-    cudaError_t e = exdot_q<4>(k, xs, ys, n, reinterpret_cast<DotScratch *>(p), out, c, s);
+    cudaError_t e = launch_exdot(k, xs, ys, n, reinterpret_cast<DotScratch *>(p), out, 0, c, s);
     if (e != cudaSuccess) return set_error(RBS_ECUDA, "rbs_exdot_noalloc: kernel launch failed");
     return RBS_OK;
 }
