@@ -119,7 +119,8 @@ struct Workspace {
     double *h_out = nullptr;
     double *d_out = nullptr;
     unsigned *h_err = nullptr;
-    Buf vec, hist, stage[8];
+    DiagArgs *h_diag = nullptr;
+    Buf vec, hist, diag, stage[8];
     Buf batch_work, batch_hist, batch_sys, batch_order, batch_out, batch_queue;
     Buf step_ctx, step_state, step_scr, step_tasks;  // the stepped batch schedule
     std::vector<cudaEvent_t> evpool;
@@ -167,6 +168,7 @@ int ws_get(cudaStream_t s, Workspace **out) {
     if (e == cudaSuccess) e = cudaMallocHost(&w->h_flags, NFLAGS * sizeof(int32_t));
     if (e == cudaSuccess) e = cudaMallocHost(&w->h_out, KMAX * sizeof(double));
     if (e == cudaSuccess) e = cudaMallocHost(&w->h_err, sizeof(unsigned));
+    if (e == cudaSuccess) e = cudaMallocHost(&w->h_diag, sizeof(DiagArgs));
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         delete w;
@@ -189,7 +191,9 @@ void ws_free(Workspace *w) {
     cudaFreeHost(w->h_flags);
     cudaFreeHost(w->h_out);
     cudaFreeHost(w->h_err);
+    cudaFreeHost(w->h_diag);
     cudaFree(w->vec.p);
+    cudaFree(w->diag.p);
     cudaFree(w->hist.p);
     for (Buf *b : {&w->batch_work, &w->batch_hist, &w->batch_sys, &w->batch_order, &w->batch_out,
                    &w->batch_queue, &w->step_ctx, &w->step_state, &w->step_scr, &w->step_tasks})
@@ -670,27 +674,58 @@ int rbs_solve_ex(const rbs_csr *A, const double *b, const double *x0, const doub
     a.hist = (double *)w->hist.p;
     a.err = &w->g->err;
     a.dot_mode = o.dot_mode;
+    // structure check and Jacobi set-up (Sec. 4: M = diag(A)); rows that can be
+    // few diagonals are laid out by them in the same pass
+    const int carve = carveout_param();
+    int smode = spmv_mode_for(n, nnz);
+    const bool try_diags = p_spmv_mode.load() == 0 && nnz > 0 && nnz <= SPMV_DIAGS * n && ((uintptr_t)val & 15) == 0;
+    if (try_diags) {
+        const int64_t chunks = (n + 31) / 32;
+        const size_t mask_at = ((size_t)(chunks + 1) * 8 + sizeof(DiagArgs) + 255) / 256 * 256;
+        CK(ensure(w->diag, mask_at + (size_t)chunks * 32 * 4));
+        int64_t *base = (int64_t *)w->diag.p;
+        DiagArgs *dd = (DiagArgs *)(base + chunks + 1);
+        uint32_t *mask = (uint32_t *)((char *)w->diag.p + mask_at);
+        CK(launch_prepare(a.A, (const double *)ddiag, V.invd, dd, mask, base, &w->g->err, grid_for(w, n, 256, 8),
+                          w->stream));
+        CK(cudaMemcpyAsync(w->h_diag, dd, sizeof(DiagArgs), cudaMemcpyDeviceToHost, w->stream));
+        a.D.mask = mask;
+        a.D.base = base;
+    } else {
+        CK(launch_csr_check(a.A, &w->g->err, grid_for(w, nnz > n ? nnz : n, 256, 8), w->stream));
+        CK(launch_jacobi_invd(a.A, (const double *)ddiag, V.invd, &w->g->err, grid_for(w, n, 256, 8), w->stream));
+    }
+    unsigned err = 0;
+    if ((rc = read_err(w, &err))) return rc;
+    if (err & 1u) return fail(RBS_EINVAL, "invalid CSR structure");
+    if (err & 2u) return fail(RBS_EINVAL, "zero, NaN or missing diagonal entry");
+    if (try_diags && !(err & ERR_DIAGS)) {
+        a.D.m = w->h_diag->m;
+        memcpy(a.D.off, w->h_diag->off, (size_t)a.D.m * sizeof(int32_t));
+        smode = (a.D.m <= 7 ? SPMV_MODE_DIAG7 : SPMV_MODE_DIAG32) | (smode & ~SPMV_MODE_MASK);
+    } else {
+        a.D.mask = nullptr;
+        a.D.base = nullptr;
+    }
     {
         const int vb = block_of(p_vec_block.load(), 256);
-        const int carve = carveout_param();
-        const int smode = spmv_mode_for(n, nnz);
-        const int bps = solver_blocks_per_sm(variant, o.dot_mode, 1, vb, carve, smode & SPMV_MODE_MASK);
+        const int kind = smode & SPMV_MODE_MASK;
+        const int bps = solver_blocks_per_sm(variant, o.dot_mode, 1, vb, carve, kind);
         a.vec = grid_for(w, (n + 1) / 2, vb, bps);
         a.p3 = variant == RBS_PIPELINED
-                   ? grid_for(w, (n + 1) / 2, vb, solver_blocks_per_sm(variant, o.dot_mode, 2, vb, carve,
-                                                                       smode & SPMV_MODE_MASK))
+                   ? grid_for(w, (n + 1) / 2, vb, solver_blocks_per_sm(variant, o.dot_mode, 2, vb, carve, kind))
                    : a.vec;
         if (p_vec_grid.load() > 0) a.vec.grid = a.p3.grid = (int)p_vec_grid.load();
-        // long rows: the register-staged kernels' own block (the knob is for short rows)
-        const int sb = (smode & SPMV_MODE_MASK) == SPMV_MODE_LONG ? SPMV_REG_WARPS * 32
-                                                                  : block_of(p_spmv_block.load(), 256);
-        a.spmv = grid_for(w, n, sb, solver_blocks_per_sm(variant, o.dot_mode, 0, sb, carve, smode & SPMV_MODE_MASK));
+        // long rows: the kernels' own block of four warps (the knob is for short rows)
+        const int sb = kind == SPMV_MODE_LONG || kind == SPMV_MODE_DIAG32 ? SPMV_REG_WARPS * 32
+                                                                         : block_of(p_spmv_block.load(), 256);
+        a.spmv = grid_for(w, n, sb, solver_blocks_per_sm(variant, o.dot_mode, 0, sb, carve, kind));
         a.spmv.mode = smode;
         a.k3 = variant == RBS_CLASSIC
-                   ? grid_for(w, n, sb, solver_blocks_per_sm(variant, o.dot_mode, 3, sb, carve, smode & SPMV_MODE_MASK))
+                   ? grid_for(w, n, sb, solver_blocks_per_sm(variant, o.dot_mode, 3, sb, carve, kind))
                    : a.spmv;
         a.k3.mode = smode;
-        a.carveout = carveout_param();
+        a.carveout = carve;
         a.spmv.carveout = a.carveout;
         a.k3.carveout = a.carveout;
         // window headroom: at most 2^20 products per thread per launch
@@ -701,14 +736,6 @@ int rbs_solve_ex(const rbs_csr *A, const double *b, const double *x0, const doub
         if (a.spmv.grid < mins) a.spmv.grid = (int)mins;
         if (a.k3.grid < mins) a.k3.grid = (int)mins;
     }
-
-    // structure check and Jacobi set-up (Sec. 4: M = diag(A))
-    CK(launch_csr_check(a.A, &w->g->err, grid_for(w, nnz > n ? nnz : n, 256, 8), w->stream));
-    CK(launch_jacobi_invd(a.A, (const double *)ddiag, V.invd, &w->g->err, grid_for(w, n, 256, 8), w->stream));
-    unsigned err = 0;
-    if ((rc = read_err(w, &err))) return rc;
-    if (err & 1u) return fail(RBS_EINVAL, "invalid CSR structure");
-    if (err & 2u) return fail(RBS_EINVAL, "zero, NaN or missing diagonal entry");
 
     EventTimer timer(w);
     KernelTimer *tm = (o.profile && prof) ? &timer : nullptr;

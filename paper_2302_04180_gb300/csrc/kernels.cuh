@@ -531,6 +531,230 @@ stalled:
     __syncwarp();
 }
 
+// Matrices of few diagonals (stencils, bands): at most SPMV_DIAGS distinct
+// values of column - row, every row's columns ascending. The solvers' set-up
+// pass over the structure (k_prepare) writes one word per row saying which of
+// the diagonals it has, and the first nonzero of each chunk of 32 rows; the
+// product then needs neither the column indices nor the row pointers: 4.25
+// bytes per row instead of 4 per nonzero and 8 (7 points: 36). Rows read the
+// stored values and run the fma chain in stored order, as spmv_row does.
+//
+// With the columns out of the way the x gathers depend on nothing but the row's
+// word, so the next group of eight is in flight while this one's chain runs,
+// and only the values are staged. What bounds the product then is the FP64 pipe
+// (7 points at 256^3: 117 million fmas, 186 us at two per SM and clock) as much
+// as HBM (K1: 84 bytes per row, 207 us). @@MEASURED@@
+//
+// Warps take chunks in tiles: a block runs SPMV_TILE groups of consecutive
+// chunks, one chunk per warp, before it moves on, so that rows that gather the
+// same x lines follow each other on one SM while the grid as a whole sweeps the
+// rows in order (a contiguous share per block would have each x line fetched
+// from HBM again for every plane offset).
+//
+// N: most diagonals, in groups of up to eight (7: one group, the next chunk's
+// gathers ahead of this one's chain; 32: four, of which the unused are skipped).
+// Each warp's two staging buffers take 32 N values. Every value span is one bulk
+// copy of whole 16-byte units; the last value of an odd nnz is stored by a
+// lane. Waits are bounded, with the timeout fallback of spmv_rows.
+constexpr int SPMV_TILE = 4;
+template <int N>
+struct DiagLayout {
+    static constexpr int PER = N < 8 ? N : 8, G = N / PER;  // diagonals per group, groups
+    static_assert(G == 1 || G % 2 == 0, "groups in pairs");
+    static constexpr int WARPS = G == 1 ? MAX_WARPS : SPMV_REG_WARPS;
+    static constexpr int BUF = (32 * N + 2) * 8;
+    static constexpr int SCRATCH = 2 * BUF;  // per warp
+    static_assert(BUF % 16 == 0 && SCRATCH >= FLUSH_SCRATCH, "the flush reuses the staging buffers");
+};
+
+template <int N, class F>
+__device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const DiagArgs &D, const double *__restrict__ x,
+                                               const double *__restrict__ z, bool test_stall, unsigned &err, F &&fn) {
+    constexpr unsigned FULL = 0xffffffffu;
+    using L = DiagLayout<N>;
+    constexpr int G = L::G, PER = L::PER;
+    __shared__ __align__(8) unsigned long long s_bar[L::WARPS][2];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int n = (int)A.n, chunks = (n + 31) >> 5;
+    unsigned char *bufs = warp_scratch<L::SCRATCH, L::WARPS>();
+    unsigned long long *bars = s_bar[wid];
+    if (lane == 0) {
+        mbar_init(bars);
+        mbar_init(bars + 1);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    __syncwarp();
+    const long long wait_limit = test_stall ? SPMV_TEST_WAIT_LIMIT : SPMV_WAIT_LIMIT;
+    // This warp's chunks in turn: whole rounds of tiles, then chunk by chunk, so
+    // that the last round is even over the blocks. `left`: steps to go in the
+    // tile; c >= chunks: none.
+    const int round = gridDim.x * nw, tiled = chunks / (round * SPMV_TILE) * (round * SPMV_TILE);
+    struct Walk {
+        int c, left;
+    };
+    auto first = [&]() {
+        return tiled ? Walk{(int)blockIdx.x * (SPMV_TILE * nw) + wid, SPMV_TILE - 1}
+                     : Walk{(int)blockIdx.x * nw + wid, 0};
+    };
+    auto next = [&](Walk &w) {
+        if (w.left > 0) {
+            w.left--;
+            w.c += nw;
+        } else if (w.c < tiled) {
+            // the next round's tile, or the first chunk after the rounds
+            w.c += (round - nw) * SPMV_TILE + nw;
+            w.left = SPMV_TILE - 1;
+            if (w.c >= tiled) w = Walk{tiled + (int)blockIdx.x * nw + wid, 0};
+        } else {
+            w.c += round;
+        }
+    };
+    struct Head {
+        long long base;  // the chunk's first nonzero
+        uint32_t word;   // this lane's row: its diagonals (N = 7: and where its values start, at bit 8)
+    };
+    auto head = [&](int c) {
+        Head h{0, 0u};
+        if (c < chunks) {
+            h.base = D.base[c];
+            h.word = D.mask[c * 32 + lane];
+        }
+        return h;
+    };
+    auto diags_of = [](uint32_t word) { return N <= 8 ? word & ((1u << (N & 31)) - 1u) : word; };
+    // the chunk's values into buffer b, by one lane
+    auto stage = [&](const Head &h, int b) {
+        const int count = (int)__reduce_add_sync(FULL, (unsigned)__popc(diags_of(h.word)));
+        if (lane != 0) return;
+        const long long va = h.base & ~1LL, end = h.base + count;
+        long long ve = (end + 1) & ~1LL;
+        double *dst = reinterpret_cast<double *>(bufs + b * L::BUF);
+        if (ve > A.nnz) {
+            ve -= 2;
+            if (count > 0) dst[end - 1 - va] = A.val[end - 1];
+        }
+        const unsigned bytes = ve > va ? (unsigned)(ve - va) * 8u : 0u;
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+        mbar_arrive_expect_tx(bars + b, bytes);
+        if (bytes && !test_stall) bulk_copy_g2s(dst, A.val + va, bytes, bars + b);
+    };
+    auto gather = [&](int row, uint32_t word, int g, double (&xv)[PER]) {
+#pragma unroll
+        for (int j = 0; j < PER; j++)
+            if ((word >> (g * PER + j)) & 1u) xv[j] = __ldg(x + (row + D.off[g * PER + j]));
+    };
+    Walk w0 = first(), w1 = w0;  // w0: the chunk being computed, w1: the one after
+    next(w1);
+    Head h0 = head(w0.c), h1 = head(w1.c);
+    unsigned parity = 0u;  // bit b: phase of buffer b's barrier to wait for
+    double xa[PER], xb[PER], z0 = 0.0, z1 = 0.0;
+    int cur = 0;
+    if (w0.c < chunks) {
+        stage(h0, 0);
+        gather(w0.c * 32 + lane, h0.word, 0, xa);
+        if (z && w0.c * 32 + lane < n) z0 = __ldg(z + w0.c * 32 + lane);
+    }
+    // One chunk: stage the next one's values, then this one's chain. xc, zc hold
+    // its first gathers and companion; xn, zn get the next one's (G = 1). Returns
+    // false when the wait for the values ran out.
+    auto step = [&](int b, double (&xc)[PER], double (&xn)[PER], double &zc, double &zn) {
+        const int row = w0.c * 32 + lane, row1 = w1.c * 32 + lane;
+        if (w1.c < chunks) stage(h1, b ^ 1);
+        Walk w2 = w1;
+        next(w2);
+        const Head h2 = head(w2.c);
+        int at;  // this row's first value in the chunk
+        if (N <= 8) {
+            at = (int)(h0.word >> 8);
+        } else {
+            const int len = __popc(h0.word);
+            at = len;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(FULL, at, o);
+                if (lane >= o) at += v;
+            }
+            at -= len;
+        }
+        const double *val = reinterpret_cast<const double *>(bufs + b * L::BUF) + ((int)(h0.base & 1) + at);
+        auto next_gather = [&](double (&xv)[PER], double &zv) {
+            gather(row1, h1.word, 0, xv);
+            if (z && row1 < n) zv = __ldg(z + row1);
+        };
+        if (G == 1) next_gather(xn, zn);
+        {
+            long long spins = 0;
+            while (!mbar_try_wait(bars + b, (parity >> b) & 1u))
+                if (++spins > wait_limit) break;
+            if (__any_sync(FULL, spins > wait_limit)) return false;
+            parity ^= 1u << b;
+        }
+        __syncwarp();
+        double acc = 0.0;
+        auto chain = [&](int g, const double (&xv)[PER]) {
+#pragma unroll
+            for (int j = 0; j < PER; j++)
+                if ((h0.word >> (g * PER + j)) & 1u) acc = fma(*val++, xv[j], acc);
+        };
+        const double zr = zc;
+        if (G == 1) {
+            chain(0, xc);
+        } else {
+            // each group's gathers ahead of the chain of the one before, the
+            // next chunk's first ahead of this one's last
+#pragma unroll
+            for (int g = 0; g < G; g += 2) {
+                if (g * PER >= D.m) break;
+                gather(row, h0.word, g + 1, xn);
+                chain(g, xc);
+                if (g + 2 < G && (g + 2) * PER < D.m) gather(row, h0.word, g + 2, xc);
+                else next_gather(xc, zc);
+                if ((g + 1) * PER < D.m) chain(g + 1, xn);
+            }
+        }
+        if (row < n) fn((int64_t)row, acc, zr);
+        __syncwarp();  // buffer b is refilled in the next step
+        w0 = w1;
+        w1 = w2;
+        h0 = h1;
+        h1 = h2;
+        return true;
+    };
+    // two steps per turn (the buffers, and for one group the gathers, swap roles)
+    bool ok = true;
+    while (w0.c < chunks) {
+        cur = 0;
+        if (!(ok = step(0, xa, xb, z0, z1))) break;
+        if (w0.c >= chunks) break;
+        cur = 1;
+        if (!(ok = G == 1 ? step(1, xb, xa, z1, z0) : step(1, xa, xb, z0, z1))) break;
+    }
+    if (ok) return;
+    // A wait ran out (ERR_TIMEOUT): as in spmv_rows, stage nothing more, read
+    // this and every later row from global memory, then wait (bounded) for the
+    // copies in flight.
+    err |= ERR_TIMEOUT;
+    const bool more = w1.c < chunks;
+    for (; w0.c < chunks; next(w0)) {
+        const int row = w0.c * 32 + lane;
+        if (row < n) {
+            bool bad = false;
+            const double acc = spmv_row(A, row, x, bad);
+            if (bad) err |= ERR_INDEX;
+            fn((int64_t)row, acc, z ? z[row] : 0.0);
+        }
+    }
+    if (!test_stall && lane == 0) {
+        for (int k = 0; k < (more ? 2 : 1); k++) {
+            const int b = cur ^ k;
+            long long spins = 0;
+            while (!mbar_try_wait(bars + b, (parity >> b) & 1u) && ++spins <= wait_limit) {
+            }
+        }
+    }
+    __syncwarp();
+}
+
 // The whole matrix over the grid: every warp of every block.
 template <bool CHECKED, int CAP, class F>
 __device__ __forceinline__ void spmv_warp_rows(const CSRView &A, const double *__restrict__ x,

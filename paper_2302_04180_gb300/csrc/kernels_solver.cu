@@ -19,6 +19,7 @@
 //   P4  t = A what                                                  (S18)
 // Once the stop flag is set, every later kernel returns at once.
 #include <mutex>
+#include <type_traits>
 
 #include "kernels.cuh"
 
@@ -45,11 +46,13 @@ __global__ void __launch_bounds__(256) k_cls_setup(Ctx c) {
     if (red.finish(c.g, vals) && threadIdx.x == 0) tail_cls_setup(c.st, vals);
 }
 
-// SpMV rows of the fused K1/K3 with epilogue fn(row, y_row, z_row): short
-// rows warp-staged (or one thread per row, mode 1) in 256-thread blocks; long
-// rows (CAP = SPMV_CAP_LONG) register-staged in blocks of SPMV_REG_WARPS warps.
-// Finish the kernel's reducer with finish<FusedScratch<CAP>::BYTES,
-// FusedScratch<CAP>::WARPS>, so that its flush reuses the staging buffer.
+// SpMV rows of the fused K1/K3 with epilogue fn(row, y_row, z_row), by CAP:
+// matrices of few diagonals (CAP = -N, spmv_rows_diag); short rows warp-staged
+// (or one thread per row, mode 1) in 256-thread blocks; long rows (CAP =
+// SPMV_CAP_LONG) register-staged in blocks of SPMV_REG_WARPS warps. Finish the
+// kernel's reducer with finish<FusedScratch<CAP>::BYTES, FusedScratch<CAP>::WARPS>,
+// so that its flush reuses the staging buffer.
+constexpr int CAP_DIAG7 = -7, CAP_DIAG32 = -32;
 template <int CAP>
 struct FusedScratch {
     static constexpr bool REG = CAP > SPMV_CAP_SHORT;
@@ -57,9 +60,19 @@ struct FusedScratch {
     static constexpr int WARPS = REG ? SPMV_REG_WARPS : MAX_WARPS;
     static constexpr int THREADS = WARPS * 32;
 };
+template <int N>
+struct FusedDiag {
+    static constexpr int BYTES = DiagLayout<N>::SCRATCH;
+    static constexpr int WARPS = DiagLayout<N>::WARPS;
+    static constexpr int THREADS = WARPS * 32;
+};
+template <> struct FusedScratch<CAP_DIAG7> : FusedDiag<7> {};
+template <> struct FusedScratch<CAP_DIAG32> : FusedDiag<32> {};
 template <int CAP, class F>
 __device__ __forceinline__ void fused_spmv(const Ctx &c, const double *x, const double *z, unsigned &eb, F &&fn) {
-    if (FusedScratch<CAP>::REG)
+    if constexpr (CAP < 0)
+        spmv_rows_diag<-CAP>(c.A, c.D, x, z, (c.spmv_mode & SPMV_TEST_STALL) != 0, eb, fn);
+    else if constexpr (FusedScratch<CAP>::REG)
         spmv_rows_reg<false, CAP, false>(c.A, 0, c.A.n, (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5),
                                          (int64_t)gridDim.x * (blockDim.x >> 5), x, z, true,
                                          (c.spmv_mode & SPMV_TEST_STALL) != 0, eb, fn);
@@ -187,11 +200,11 @@ __global__ void __launch_bounds__(256) k_pipe_setup1(Ctx c) {
 
 // set-up 2: w = A rhat, what = w * invd, <r0,r>, <r0,w> -> alpha0
 template <class R, int CAP>
-__global__ void __launch_bounds__(256, CAP > SPMV_CAP_SHORT ? 1 : 3) k_pipe_setup2(Ctx c) {
+__global__ void __launch_bounds__(FusedScratch<CAP>::THREADS, 3) k_pipe_setup2(Ctx c) {
     R red;
     red.init();
     unsigned eb = 0u;
-    spmv_each<false, CAP>(c.A, c.rh, c.r0, c.spmv_mode, eb, [&](int64_t i, double wi, double r0) {
+    fused_spmv<CAP>(c, c.rh, c.r0, eb, [&](int64_t i, double wi, double r0) {
         c.w[i] = wi;
         c.wh[i] = __dmul_rn(wi, c.invd[i]);
         red.add_sq(0, r0);  // r = r0 at set-up
@@ -199,7 +212,9 @@ __global__ void __launch_bounds__(256, CAP > SPMV_CAP_SHORT ? 1 : 3) k_pipe_setu
     });
     if (eb) atomicOr(c.err, eb);
     __shared__ double vals[R::K];
-    if (red.template finish<SpmvLayout<CAP>::SCRATCH>(c.g, vals, 0u, !(eb & ERR_TIMEOUT)) && threadIdx.x == 0)
+    if (red.template finish<FusedScratch<CAP>::BYTES, FusedScratch<CAP>::WARPS>(c.g, vals, 0u,
+                                                                               !(eb & ERR_TIMEOUT)) &&
+        threadIdx.x == 0)
         tail_pipe_setup(c.st, vals);
 }
 
@@ -320,6 +335,7 @@ __global__ void __launch_bounds__(256, P3Cfg<R>::blocks) k_pipe_p3(Ctx c) {
 static Ctx make_ctx(const SolverArgs &a) {
     Ctx c;
     c.A = CSRView{a.A.n, a.A.nnz, a.A.rowptr, a.A.col, a.A.val};
+    c.D = a.D;
     c.n = a.A.n;
     c.x = a.v.x; c.r = a.v.r; c.r0 = a.v.r0; c.p = a.v.p; c.ph = a.v.ph; c.s = a.v.s;
     c.q = a.v.q; c.qh = a.v.qh; c.y = a.v.y; c.invd = a.v.invd;
@@ -337,6 +353,27 @@ static Ctx make_ctx(const SolverArgs &a) {
         if (tm) tm->after(kind);        \
     } while (0)
 
+// The compile-time schedule of a row schedule (mode), passed to f.
+template <class F>
+static void with_cap(int mode, F &&f) {
+    switch (mode & SPMV_MODE_MASK) {
+        case SPMV_MODE_DIAG7: f(std::integral_constant<int, CAP_DIAG7>()); break;
+        case SPMV_MODE_DIAG32: f(std::integral_constant<int, CAP_DIAG32>()); break;
+        case SPMV_MODE_LONG: f(std::integral_constant<int, SPMV_CAP_LONG>()); break;
+        default: f(std::integral_constant<int, SPMV_CAP_SHORT>()); break;
+    }
+}
+
+static bool diag_mode(int mode) {
+    return (mode & SPMV_MODE_MASK) == SPMV_MODE_DIAG7 || (mode & SPMV_MODE_MASK) == SPMV_MODE_DIAG32;
+}
+
+// y = A x without a dot (pipelined S10, S18 and set-up).
+static cudaError_t plain_spmv(const SolverArgs &a, const double *x, double *y, cudaStream_t s) {
+    if (diag_mode(a.spmv.mode)) return launch_spmv_diag(a.A, a.D, x, y, a.st, a.err, a.spmv, s);
+    return launch_spmv(a.A, x, y, a.st, a.err, a.spmv, s);
+}
+
 template <class R1, class R2, class R5>
 static cudaError_t setup_t(const SolverArgs &a, int variant, cudaStream_t s, KernelTimer *tm) {
     Ctx c = make_ctx(a);
@@ -344,11 +381,10 @@ static cudaError_t setup_t(const SolverArgs &a, int variant, cudaStream_t s, Ker
         TIMED(PK_SETUP, (k_cls_setup<R1><<<a.vec.grid, a.vec.block, 0, s>>>(c)));
     } else {
         TIMED(PK_SETUP, (k_pipe_setup1<<<a.vec.grid, a.vec.block, 0, s>>>(c)));
-        if ((a.spmv.mode & SPMV_MODE_MASK) == SPMV_MODE_LONG)
-            TIMED(PK_SETUP, (k_pipe_setup2<R2, SPMV_CAP_LONG><<<a.spmv.grid, a.spmv.block, 0, s>>>(c)));
-        else
-            TIMED(PK_SETUP, (k_pipe_setup2<R2, SPMV_CAP_SHORT><<<a.spmv.grid, a.spmv.block, 0, s>>>(c)));
-        TIMED(PK_SETUP, (launch_spmv(a.A, a.v.wh, a.v.t, a.st, a.err, a.spmv, s)));
+        with_cap(a.spmv.mode, [&](auto cap) {
+            TIMED(PK_SETUP, (k_pipe_setup2<R2, decltype(cap)::value><<<a.spmv.grid, a.spmv.block, 0, s>>>(c)));
+        });
+        TIMED(PK_SETUP, (plain_spmv(a, a.v.wh, a.v.t, s)));
     }
     return cudaGetLastError();
 }
@@ -357,19 +393,20 @@ template <class R1, class R2, class R5>
 static cudaError_t iter_t(const SolverArgs &a, int variant, cudaStream_t s, KernelTimer *tm) {
     Ctx c = make_ctx(a);
     if (variant == RBS_CLASSIC) {
-        const bool lng = (a.spmv.mode & SPMV_MODE_MASK) == SPMV_MODE_LONG;
-        if (lng) TIMED(PK_K1, (k_cls_k1<R1, SPMV_CAP_LONG><<<a.spmv.grid, a.spmv.block, 0, s>>>(c)));
-        else TIMED(PK_K1, (k_cls_k1<R1, SPMV_CAP_SHORT><<<a.spmv.grid, a.spmv.block, 0, s>>>(c)));
+        with_cap(a.spmv.mode, [&](auto cap) {
+            TIMED(PK_K1, (k_cls_k1<R1, decltype(cap)::value><<<a.spmv.grid, a.spmv.block, 0, s>>>(c)));
+        });
         TIMED(PK_VEC, (k_cls_k2<<<a.vec.grid, a.vec.block, 0, s>>>(c)));
-        if (lng) TIMED(PK_K3, (k_cls_k3<R2, SPMV_CAP_LONG><<<a.k3.grid, a.k3.block, 0, s>>>(c)));
-        else TIMED(PK_K3, (k_cls_k3<R2, SPMV_CAP_SHORT><<<a.k3.grid, a.k3.block, 0, s>>>(c)));
+        with_cap(a.spmv.mode, [&](auto cap) {
+            TIMED(PK_K3, (k_cls_k3<R2, decltype(cap)::value><<<a.k3.grid, a.k3.block, 0, s>>>(c)));
+        });
         TIMED(PK_K4, (k_cls_k4<R2><<<a.vec.grid, a.vec.block, 0, s>>>(c)));
         TIMED(PK_VEC, (k_cls_k5<<<a.vec.grid, a.vec.block, 0, s>>>(c)));
     } else {
         TIMED(PK_VEC_DOT, (k_pipe_p1<R2><<<a.vec.grid, a.vec.block, 0, s>>>(c)));
-        TIMED(PK_SPMV, (launch_spmv(a.A, a.v.zh, a.v.v, a.st, a.err, a.spmv, s)));
+        TIMED(PK_SPMV, (plain_spmv(a, a.v.zh, a.v.v, s)));
         TIMED(PK_VEC_DOT, (k_pipe_p3<R5><<<a.p3.grid, a.p3.block, 0, s>>>(c)));
-        TIMED(PK_SPMV, (launch_spmv(a.A, a.v.wh, a.v.t, a.st, a.err, a.spmv, s)));
+        TIMED(PK_SPMV, (plain_spmv(a, a.v.wh, a.v.t, s)));
     }
     return cudaGetLastError();
 }
@@ -379,15 +416,16 @@ static cudaError_t iter_t(const SolverArgs &a, int variant, cudaStream_t s, Kern
 // the SpMV live on L1 hits, so the split is a tuning knob, not a maximum.
 template <class R1, class R2, class R5>
 static void prefer_shared(int c) {
-    cudaFuncSetAttribute(k_cls_k1<R1, SPMV_CAP_SHORT>, cudaFuncAttributePreferredSharedMemoryCarveout, c);
-    cudaFuncSetAttribute(k_cls_k3<R2, SPMV_CAP_SHORT>, cudaFuncAttributePreferredSharedMemoryCarveout, c);
     cudaFuncSetAttribute(k_cls_k4<R2>, cudaFuncAttributePreferredSharedMemoryCarveout, c);
-    cudaFuncSetAttribute(k_pipe_setup2<R2, SPMV_CAP_SHORT>, cudaFuncAttributePreferredSharedMemoryCarveout, c);
-    // the long-row kernels need (nearly) all of it for their staging buffers
-    const int cl = c < 0 ? c : 100;
-    cudaFuncSetAttribute(k_cls_k1<R1, SPMV_CAP_LONG>, cudaFuncAttributePreferredSharedMemoryCarveout, cl);
-    cudaFuncSetAttribute(k_cls_k3<R2, SPMV_CAP_LONG>, cudaFuncAttributePreferredSharedMemoryCarveout, cl);
-    cudaFuncSetAttribute(k_pipe_setup2<R2, SPMV_CAP_LONG>, cudaFuncAttributePreferredSharedMemoryCarveout, cl);
+    for (int mode : {SPMV_MODE_SHORT, SPMV_MODE_LONG, SPMV_MODE_DIAG7, SPMV_MODE_DIAG32})
+        with_cap(mode, [&](auto cap) {
+            constexpr int CAP = decltype(cap)::value;
+            // the kernels of long rows need (nearly) all of it for their staging buffers
+            const int share = c < 0 || CAP == SPMV_CAP_SHORT || CAP == CAP_DIAG7 ? c : 100;
+            cudaFuncSetAttribute(k_cls_k1<R1, CAP>, cudaFuncAttributePreferredSharedMemoryCarveout, share);
+            cudaFuncSetAttribute(k_cls_k3<R2, CAP>, cudaFuncAttributePreferredSharedMemoryCarveout, share);
+            cudaFuncSetAttribute(k_pipe_setup2<R2, CAP>, cudaFuncAttributePreferredSharedMemoryCarveout, share);
+        });
     cudaFuncSetAttribute(k_pipe_p1<R2>, cudaFuncAttributePreferredSharedMemoryCarveout, c);
     cudaFuncSetAttribute(k_pipe_p3<R5>, cudaFuncAttributePreferredSharedMemoryCarveout, c);
     cudaGetLastError();
@@ -437,45 +475,31 @@ cudaError_t launch_set_cond(cudaGraphConditionalHandle h, SolverState *st, cudaS
     return cudaGetLastError();
 }
 
-int solver_blocks_per_sm(int variant, int dot_mode, int which, int block, int carveout, int spmv_mode) {
-    apply_carveout(dot_mode, carveout);
-    if (which == 0 && variant == RBS_PIPELINED) return spmv_blocks_per_sm(block, carveout, spmv_mode);
-    const bool lng = spmv_mode == SPMV_MODE_LONG;
+template <class R1, class R2, class R5>
+static int blocks_per_sm_t(int variant, int which, int block, int spmv_mode) {
     int nb = 0;
     cudaError_t e = cudaSuccess;
-    if (dot_mode == RBS_DOT_PLAIN) {
-        using R1 = PlainR<1>;
-        using R2 = PlainR<2>;
-        if (which == 0) {
-            e = lng ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_cls_k1<R1, SPMV_CAP_LONG>, block, 0)
-                    : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_cls_k1<R1, SPMV_CAP_SHORT>, block, 0);
-        } else if (which == 3) {
-            e = lng ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_cls_k3<R2, SPMV_CAP_LONG>, block, 0)
-                    : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_cls_k3<R2, SPMV_CAP_SHORT>, block, 0);
-        } else if (variant == RBS_PIPELINED) {
-            e = which == 2 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pipe_p3<PlainR<5>>, block, 0)
-                           : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pipe_p1<R2>, block, 0);
-        } else {
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_cls_k4<R2>, block, 0);
-        }
+    if (which == 0 || which == 3) {
+        with_cap(spmv_mode, [&](auto cap) {
+            constexpr int CAP = decltype(cap)::value;
+            e = which == 0 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_cls_k1<R1, CAP>, block, 0)
+                           : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_cls_k3<R2, CAP>, block, 0);
+        });
+    } else if (variant == RBS_PIPELINED) {
+        e = which == 2 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pipe_p3<R5>, block, 0)
+                       : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pipe_p1<R2>, block, 0);
     } else {
-        using R1 = ExactR<1, SQ>;
-        using R2 = ExactR<2, SQ>;
-        if (which == 0) {
-            e = lng ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_cls_k1<R1, SPMV_CAP_LONG>, block, 0)
-                    : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_cls_k1<R1, SPMV_CAP_SHORT>, block, 0);
-        } else if (which == 3) {
-            e = lng ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_cls_k3<R2, SPMV_CAP_LONG>, block, 0)
-                    : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_cls_k3<R2, SPMV_CAP_SHORT>, block, 0);
-        } else if (variant == RBS_PIPELINED) {
-            e = which == 2 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pipe_p3<ExactR<5, SQ>>, block, 0)
-                           : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pipe_p1<R2>, block, 0);
-        } else {
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_cls_k4<R2>, block, 0);
-        }
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_cls_k4<R2>, block, 0);
     }
     if (e != cudaSuccess || nb < 1) nb = 1;
     return nb;
+}
+
+int solver_blocks_per_sm(int variant, int dot_mode, int which, int block, int carveout, int spmv_mode) {
+    apply_carveout(dot_mode, carveout);
+    if (which == 0 && variant == RBS_PIPELINED) return spmv_blocks_per_sm(block, carveout, spmv_mode);
+    if (dot_mode == RBS_DOT_PLAIN) return blocks_per_sm_t<PlainR<1>, PlainR<2>, PlainR<5>>(variant, which, block, spmv_mode);
+    return blocks_per_sm_t<ExactR<1, SQ>, ExactR<2, SQ>, ExactR<5, SQ>>(variant, which, block, spmv_mode);
 }
 
 }  // namespace rbs

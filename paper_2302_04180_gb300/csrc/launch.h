@@ -19,11 +19,25 @@ struct CSRArgs {
     const double *val;
 };
 
+// A matrix of few diagonals as the solvers' set-up lays it out (kernels.cuh):
+// per row a word whose bit j says that the row has an entry at column
+// row + off[j] (off ascending, m of them; with at most 7, bits 8 and up hold the
+// row's first value within its 32 rows), and per 32 rows the first nonzero.
+constexpr int SPMV_DIAGS = 32;
+struct DiagArgs {
+    const uint32_t *mask;
+    const int64_t *base;
+    int32_t m, pad;
+    int32_t off[SPMV_DIAGS];
+};
+
 // SpMV row schedules (Cfg::mode): one thread per row, warp-staged chunks of
-// up to SPMV_CAP_SHORT or SPMV_CAP_LONG nonzeros.
+// up to SPMV_CAP_SHORT or SPMV_CAP_LONG nonzeros, rows of up to 7 or 32
+// diagonals.
 // Bit SPMV_TEST_STALL above the schedule bits selects the staged SpMV's test
 // mode of its bounded wait (kernels.cuh).
-enum : int { SPMV_MODE_ROW = 1, SPMV_MODE_SHORT = 2, SPMV_MODE_LONG = 3, SPMV_MODE_MASK = 0xff, SPMV_TEST_STALL = 0x100 };
+enum : int { SPMV_MODE_ROW = 1, SPMV_MODE_SHORT = 2, SPMV_MODE_LONG = 3, SPMV_MODE_DIAG7 = 4, SPMV_MODE_DIAG32 = 5,
+             SPMV_MODE_MASK = 0xff, SPMV_TEST_STALL = 0x100 };
 // Long rows run register-staged in blocks of SPMV_REG_WARPS warps: the
 // standalone SpMV, and the classic loop's fused K1/K3.
 constexpr int SPMV_REG_WARPS = 4;
@@ -59,11 +73,21 @@ cudaError_t launch_round_limbs(const int64_t *limbs, const int32_t *flags, doubl
 // the checks (and does nothing once the solver has stopped).
 cudaError_t launch_spmv(const CSRArgs &A, const double *x, double *y, const SolverState *st,
                         unsigned *err, Cfg cfg, cudaStream_t s);
+// The same product of a solver on a matrix laid out by its diagonals.
+cudaError_t launch_spmv_diag(const CSRArgs &A, const DiagArgs &D, const double *x, double *y, const SolverState *st,
+                             unsigned *err, Cfg cfg, cudaStream_t s);
 cudaError_t launch_jacobi_invd(const CSRArgs &A, const double *diag, double *invd, unsigned *err,
                                Cfg cfg, cudaStream_t s);
 cudaError_t launch_jacobi_apply(int64_t n, const double *invd, const double *p, double *phat, Cfg cfg,
                                 cudaStream_t s);
 cudaError_t launch_csr_check(const CSRArgs &A, unsigned *err, Cfg cfg, cudaStream_t s);
+// The structure check, the Jacobi inverse and the diagonal layout in one pass
+// over the rows. *diags (device): the diagonals of a sample of rows, m = 0 if
+// they are too many; mask and base are written for them, and a row that does
+// not fit them sets ERR_DIAGS in err (it is no error of the matrix).
+constexpr unsigned ERR_DIAGS = 16u;
+cudaError_t launch_prepare(const CSRArgs &A, const double *diag, double *invd, DiagArgs *diags, uint32_t *mask,
+                           int64_t *base, unsigned *err, Cfg cfg, cudaStream_t s);
 
 // ---- solver kernels (kernels_solver.cu) ----
 struct SolverVecs {
@@ -73,6 +97,7 @@ struct SolverVecs {
 
 struct SolverArgs {
     CSRArgs A;
+    DiagArgs D;  // with the SPMV_MODE_DIAG* schedules
     SolverVecs v;
     const double *b, *x0;
     SolverState *st;

@@ -13,6 +13,7 @@ constexpr int SQ = 4;  // window placements used by the solver kernels
 
 struct Ctx {
     CSRView A;
+    DiagArgs D;  // with the SPMV_MODE_DIAG* schedules
     int64_t n;
     double *x, *r, *r0, *p, *ph, *s, *q, *qh, *y, *invd;
     double *rh, *w, *wh, *t, *sh, *z, *zh, *v;
