@@ -209,9 +209,16 @@ __device__ __forceinline__ void exact_add(Win<Q> &W, uint32_t &flags, unsigned l
     }
     if (W.a < 0 || q >= Q) {
         // empty, or above the window: flush and re-anchor with the product at
-        // offset Q-2 (or 0), leaving room for somewhat larger products
+        // offset Q-2 (or 0), leaving room for somewhat larger products. Lanes that
+        // open their windows together take one anchor where their products are
+        // within two limbs, for the sake of warp_flush.
+        int top = L;
+        if (W.a < 0) {
+            const int m = (int)__reduce_max_sync(__activemask(), (unsigned)L);
+            if (m - L <= (Q >= 2 ? Q - 2 : 0)) top = m;
+        }
         win_flush<Q>(W, sacc);
-        int a = L - (Q >= 2 ? Q - 2 : 0);
+        int a = top - (Q >= 2 ? Q - 2 : 0);
         a = a < 0 ? 0 : a;
         W.a = a;
         win_place_add<Q, !SQUARE>(W, u, L - a, m);
@@ -289,6 +296,23 @@ __device__ __forceinline__ void warp_flush(Win<Q> &W, unsigned long long *sacc) 
     if (lo == 0x7fffffff) return;  // no lane holds a window
     if (hi - lo > 24) {
         win_flush<Q>(W, sacc);
+        return;
+    }
+    if (lo == hi) {
+        // one anchor (the usual case): every word summed over the warp in two
+        // 16-bit halves, the top word's upper half signed
+        long long mine = 0;
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            const uint32_t w = W.w[k];  // zero in lanes without a window
+            const long long low = (long long)__reduce_add_sync(FULL, w & 0xffffu);
+            const long long high = k < 7 ? (long long)__reduce_add_sync(FULL, w >> 16)
+                                         : (long long)__reduce_add_sync(FULL, (int)w >> 16);
+            if (lane == k) mine = low + high * 65536;
+            W.w[k] = 0u;
+        }
+        if (lane < 8 && mine && lo + lane < NL) sacc_add(&sacc[lo + lane], mine);
+        W.a = WIN_EMPTY;
         return;
     }
     __syncwarp();
@@ -404,6 +428,64 @@ static __device__ __noinline__ double round_limbs_thread(long long *G, uint32_t 
     return round_limbs_span(G, flags, lo, hi);
 }
 
+// round_limbs_span by a whole warp (all 32 lanes, same arguments; every lane
+// gets the value): one limb per lane, carries and borrows resolved over the
+// lanes with ballots instead of limb by limb (a chain of dependent shared-memory
+// reads and writes; the rounding is part of every reduction's latency). Spans
+// over 29 limbs, subnormal results and non-finite flags take the serial way.
+static __device__ __noinline__ double round_limbs_warp(long long *G, uint32_t flags, int lo, int hi) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    // carry into each bit of a ripple with generate mask g and propagate mask p
+    auto ripple = [](uint32_t g, uint32_t p) { return ((g | p) + g) ^ (g | p) ^ g; };
+    if (flags == 0u && (lo < 0 || lo > hi)) return 0.0;
+    if (flags == 0u && hi - lo <= 28) {
+        long long t = lane <= hi - lo ? G[lo + lane] : 0ll;
+        // two rounds leave -1 .. 2^32 in each lane
+#pragma unroll
+        for (int i = 0; i < 2; i++) {
+            const int up = __shfl_up_sync(FULL, (int)(t >> 32), 1);
+            t = (t & 0xffffffffll) + (lane ? up : 0);
+        }
+        const uint32_t n = t < 0 ? 1u : 0u;
+        uint32_t d = n ? 0u : (uint32_t)t;
+        const uint32_t cin =
+            ripple(__ballot_sync(FULL, t == 0x100000000ll), __ballot_sync(FULL, t == 0xffffffffll));
+        d += (cin >> lane) & 1u;
+        const uint32_t bin = ripple(__ballot_sync(FULL, n && d == 0u), __ballot_sync(FULL, d == n));
+        d -= n + ((bin >> lane) & 1u);
+        const bool neg = (__ballot_sync(FULL, (int)d < 0) >> 31) != 0u;  // lanes past the span hold the sign
+        uint32_t nz = __ballot_sync(FULL, d != 0u);
+        if (nz == 0u) return 0.0;
+        if (neg) {
+            const int z = __ffs(nz) - 1;
+            d = lane < z ? 0u : lane == z ? 0u - d : ~d;
+            nz = __ballot_sync(FULL, d != 0u);
+        }
+        const int tw = 31 - __clz(nz);
+        const uint32_t w2 = __shfl_sync(FULL, d, tw);
+        uint32_t w1 = __shfl_sync(FULL, d, tw >= 1 ? tw - 1 : 0), w0 = __shfl_sync(FULL, d, tw >= 2 ? tw - 2 : 0);
+        if (tw < 1) w1 = 0u;
+        if (tw < 2) w0 = 0u;
+        const int lead = __clz(w2);
+        const int lsb = 32 * (lo + tw) + 31 - lead - 52;  // of the 53-bit significand
+        if (lsb >= 1074) {
+            const uint32_t top = __funnelshift_l(w1, w2, lead), mid = __funnelshift_l(w0, w1, lead);
+            const unsigned long long v = ((unsigned long long)top << 32) | mid;
+            unsigned long long mant = v >> 11;
+            const bool sticky = (v & 0x3ffull) != 0ull || (w0 << lead) != 0u || (tw >= 3 && (nz & ((1u << (tw - 2)) - 1u)));
+            if (((v >> 10) & 1ull) && (sticky || (mant & 1ull))) mant += 1ull;
+            unsigned long long bits = ((unsigned long long)(lsb - 1074) << 52) + mant;
+            if (lsb - 1074 >= 2047 || bits >= 0x7ff0000000000000ull) bits = 0x7ff0000000000000ull;
+            if (neg) bits |= 0x8000000000000000ull;
+            return __longlong_as_double((long long)bits);
+        }
+    }
+    double v = 0.0;
+    if (lane == 0) v = round_limbs_span(G, flags, lo, hi);
+    return __shfl_sync(FULL, v, 0);
+}
+
 // Block- and grid-level finish of K exact reductions, once every thread's own
 // accumulators are in the block accumulators sacc (flags[k]: this thread's
 // non-finite flags). Every thread of each of the nblk blocks that share the
@@ -428,31 +510,42 @@ __device__ __forceinline__ bool block_grid_finish(const uint32_t (&flags)[K], un
     for (int k = 0; k < K; k++)
         if (flags[k]) atomicOr(&sflags[k], flags[k]);
     __syncthreads();
-    for (int idx = threadIdx.x; idx < K * NL; idx += blockDim.x) {
-        const int k = idx / NL, j = idx - k * NL;
-        const long long v = partial_norm(sacc[k], j);
-        if (v) atomicAdd(&g->limbs[slot + k][j], (unsigned long long)v);
-    }
-    if (threadIdx.x < K && sflags[threadIdx.x]) atomicOr(&g->flags[slot + threadIdx.x], sflags[threadIdx.x]);
-    __threadfence();
-    __syncthreads();
-    __shared__ bool s_last;
-    if (threadIdx.x == 0) s_last = (atomicAdd(&g->ticket[slot], 1u) == (nblk ? nblk : gridDim.x) - 1);
-    __syncthreads();
-    if (!s_last) return false;
-    __threadfence();
-    // read back (and clear) the global accumulators into shared memory
-    for (int idx = threadIdx.x; idx < K * NL; idx += blockDim.x) {
-        const int k = idx / NL, j = idx - k * NL;
-        const unsigned long long v = atomicExch(&g->limbs[slot + k][j], 0ull);
-        sacc[k][j] = v;
-        if (v) {
-            atomicMin(&s_span[k][0], j);
-            atomicMax(&s_span[k][1], j);
+    if ((nblk ? nblk : gridDim.x) == 1u) {
+        // a reduction of one block needs no other's part
+        for (int idx = threadIdx.x; idx < K * NL; idx += blockDim.x) {
+            const int k = idx / NL, j = idx - k * NL;
+            if (sacc[k][j]) {
+                atomicMin(&s_span[k][0], j);
+                atomicMax(&s_span[k][1], j);
+            }
         }
+    } else {
+        for (int idx = threadIdx.x; idx < K * NL; idx += blockDim.x) {
+            const int k = idx / NL, j = idx - k * NL;
+            const long long v = partial_norm(sacc[k], j);
+            if (v) atomicAdd(&g->limbs[slot + k][j], (unsigned long long)v);
+        }
+        if (threadIdx.x < K && sflags[threadIdx.x]) atomicOr(&g->flags[slot + threadIdx.x], sflags[threadIdx.x]);
+        __threadfence();
+        __syncthreads();
+        __shared__ bool s_last;
+        if (threadIdx.x == 0) s_last = (atomicAdd(&g->ticket[slot], 1u) == (nblk ? nblk : gridDim.x) - 1);
+        __syncthreads();
+        if (!s_last) return false;
+        __threadfence();
+        // read back (and clear) the global accumulators into shared memory
+        for (int idx = threadIdx.x; idx < K * NL; idx += blockDim.x) {
+            const int k = idx / NL, j = idx - k * NL;
+            const unsigned long long v = atomicExch(&g->limbs[slot + k][j], 0ull);
+            sacc[k][j] = v;
+            if (v) {
+                atomicMin(&s_span[k][0], j);
+                atomicMax(&s_span[k][1], j);
+            }
+        }
+        if (threadIdx.x < K) sflags[threadIdx.x] = atomicExch(&g->flags[slot + threadIdx.x], 0u);
+        if (threadIdx.x == 0) g->ticket[slot] = 0u;
     }
-    if (threadIdx.x < K) sflags[threadIdx.x] = atomicExch(&g->flags[slot + threadIdx.x], 0u);
-    if (threadIdx.x == 0) g->ticket[slot] = 0u;
     __syncthreads();
     if (export_limbs) {
         for (int idx = threadIdx.x; idx < NL; idx += blockDim.x)
@@ -460,9 +553,10 @@ __device__ __forceinline__ bool block_grid_finish(const uint32_t (&flags)[K], un
         if (threadIdx.x == 0) *flags_out = (int32_t)sflags[0];
         return true;
     }
-    if (threadIdx.x < K)
-        vals[threadIdx.x] = round_limbs_span((long long *)sacc[threadIdx.x], sflags[threadIdx.x],
-                                             s_span[threadIdx.x][0], s_span[threadIdx.x][1]);
+    for (int k = threadIdx.x >> 5; k < K; k += (int)(blockDim.x >> 5)) {
+        const double v = round_limbs_warp((long long *)sacc[k], sflags[k], s_span[k][0], s_span[k][1]);
+        if ((threadIdx.x & 31) == 0) vals[k] = v;
+    }
     __syncthreads();
     return true;
 }

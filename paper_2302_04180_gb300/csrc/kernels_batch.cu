@@ -62,6 +62,7 @@ struct ClusterRed {
     unsigned long long (*acc)[NL];  // this CTA's accumulators (shared)
     long long (*red)[NL];           // group sums (shared)
     uint32_t *flags, *rflags;
+    int (*span)[2];  // lowest and highest nonzero limb of each sum
     double *vals;
 };
 
@@ -86,6 +87,10 @@ __device__ __forceinline__ void group_reduce(const Grp &g, Win<BQ> (&win)[K], ui
         if (fl[k]) atomicOr(&R.flags[k], fl[k]);
         fl[k] = 0u;
     }
+    if (threadIdx.x < K) {
+        R.span[threadIdx.x][0] = NL;
+        R.span[threadIdx.x][1] = -1;
+    }
     g.sync();
     for (int idx = threadIdx.x; idx < K * NL; idx += blockDim.x) {
         long long sum = 0;
@@ -95,6 +100,10 @@ __device__ __forceinline__ void group_reduce(const Grp &g, Win<BQ> (&win)[K], ui
             sum = (long long)(&R.acc[0][0])[idx];
         }
         (&R.red[0][0])[idx] = sum;
+        if (sum) {
+            atomicMin(&R.span[idx / NL][0], idx % NL);
+            atomicMax(&R.span[idx / NL][1], idx % NL);
+        }
     }
     if (threadIdx.x < K) {
         uint32_t f = 0u;
@@ -107,9 +116,10 @@ __device__ __forceinline__ void group_reduce(const Grp &g, Win<BQ> (&win)[K], ui
     }
     g.sync();
     for (int idx = threadIdx.x; idx < K * NL; idx += blockDim.x) (&R.acc[0][0])[idx] = 0ull;
-    if (threadIdx.x < K) {
-        R.flags[threadIdx.x] = 0u;
-        R.vals[threadIdx.x] = round_limbs_thread(R.red[threadIdx.x], R.rflags[threadIdx.x]);
+    if (threadIdx.x < K) R.flags[threadIdx.x] = 0u;
+    for (int k = threadIdx.x >> 5; k < K; k += (int)(blockDim.x >> 5)) {
+        const double v = round_limbs_warp(R.red[k], R.rflags[k], R.span[k][0], R.span[k][1]);
+        if ((threadIdx.x & 31) == 0) R.vals[k] = v;
     }
     __syncthreads();
 }
@@ -435,11 +445,12 @@ __global__ void __launch_bounds__(256, 2)
     __shared__ unsigned long long s_acc[5][NL];
     __shared__ long long s_red[5][NL];
     __shared__ uint32_t s_flags[5], s_rflags[5];
+    __shared__ int s_span[5][2];
     __shared__ double s_vals[5];
     __shared__ int s_bad;
     for (int idx = threadIdx.x; idx < 5 * NL; idx += blockDim.x) (&s_acc[0][0])[idx] = 0ull;
     if (threadIdx.x < 5) s_flags[threadIdx.x] = 0u;
-    ClusterRed R{s_acc, s_red, s_flags, s_rflags, s_vals};
+    ClusterRed R{s_acc, s_red, s_flags, s_rflags, s_span, s_vals};
     cl.sync();  // every CTA of the cluster runs before any shared memory is touched remotely
     int first_small = -1;  // a small system the cluster pulled, solved by rank 0 alone
     if (csize > 1) {

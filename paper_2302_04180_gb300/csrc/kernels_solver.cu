@@ -34,8 +34,10 @@ namespace rbs {
 // set-up: r = b - A x0 (or b), x = x0 (or +0), r0 = p = r, phat = r*invd, <r0,r0>
 template <class R>
 __global__ void __launch_bounds__(256) k_cls_setup(Ctx c) {
+    StateCopy sc;
+    sc.load(c.st);
     R red;
-    red.init();
+    red.init();  // ends in a barrier
     bool bad = false;
     for (int64_t i = gtid(); i < c.n; i += gstride()) {
         const double ri = cls_setup_elem(c, i, bad);
@@ -43,7 +45,7 @@ __global__ void __launch_bounds__(256) k_cls_setup(Ctx c) {
     }
     if (bad) atomicOr(c.err, 1u);
     __shared__ double vals[R::K];
-    if (red.finish(c.g, vals) && threadIdx.x == 0) tail_cls_setup(c.st, vals);
+    if (red.finish(c.g, vals)) sc.tail([&](SolverState *st) { tail_cls_setup(st, vals); });
 }
 
 // SpMV rows of the fused K1/K3 with epilogue fn(row, y_row, z_row), by CAP:
@@ -83,9 +85,11 @@ __device__ __forceinline__ void fused_spmv(const Ctx &c, const double *x, const 
 // K1: s = A phat, <r0, s>
 template <class R, int CAP>
 __global__ void __launch_bounds__(FusedScratch<CAP>::THREADS, 3) k_cls_k1(Ctx c) {
-    if (c.st->done) return;
+    StateCopy sc;
+    sc.load(c.st);
     R red;
-    red.init();
+    red.init();  // ends in a barrier
+    if (sc.copy->done) return;
     unsigned eb = 0u;
     fused_spmv<CAP>(c, c.ph, c.r0, eb, [&](int64_t i, double si, double r0) {
         c.s[i] = si;
@@ -94,9 +98,8 @@ __global__ void __launch_bounds__(FusedScratch<CAP>::THREADS, 3) k_cls_k1(Ctx c)
     if (eb) atomicOr(c.err, eb);
     __shared__ double vals[R::K];
     if (red.template finish<FusedScratch<CAP>::BYTES, FusedScratch<CAP>::WARPS>(c.g, vals, 0u,
-                                                                               !(eb & ERR_TIMEOUT)) &&
-        threadIdx.x == 0)
-        tail_cls_alpha(c.st, vals);
+                                                                               !(eb & ERR_TIMEOUT)))
+        sc.tail([&](SolverState *st) { tail_cls_alpha(st, vals); });
 }
 
 // K2: q = fma(-alpha, s, r), qhat = q * invd. Four blocks per SM, like K4, whose
@@ -122,9 +125,11 @@ __global__ void __launch_bounds__(256, 4) k_cls_k2(Ctx c) {
 // K3: y = A qhat, <q, y>, <y, y>
 template <class R, int CAP>
 __global__ void __launch_bounds__(FusedScratch<CAP>::THREADS, 3) k_cls_k3(Ctx c) {
-    if (c.st->done) return;
+    StateCopy sc;
+    sc.load(c.st);
     R red;
-    red.init();
+    red.init();  // ends in a barrier
+    if (sc.copy->done) return;
     unsigned eb = 0u;
     fused_spmv<CAP>(c, c.qh, c.q, eb, [&](int64_t i, double yi, double qi) {
         c.y[i] = yi;
@@ -134,18 +139,19 @@ __global__ void __launch_bounds__(FusedScratch<CAP>::THREADS, 3) k_cls_k3(Ctx c)
     if (eb) atomicOr(c.err, eb);
     __shared__ double vals[R::K];
     if (red.template finish<FusedScratch<CAP>::BYTES, FusedScratch<CAP>::WARPS>(c.g, vals, 0u,
-                                                                               !(eb & ERR_TIMEOUT)) &&
-        threadIdx.x == 0)
-        tail_cls_omega(c.st, vals);
+                                                                               !(eb & ERR_TIMEOUT)))
+        sc.tail([&](SolverState *st) { tail_cls_omega(st, vals); });
 }
 
 // K4: x = fma(omega, qhat, fma(alpha, phat, x)), r = fma(-omega, y, q), <r0,r>, <r,r>
 template <class R>
 __global__ void __launch_bounds__(256) k_cls_k4(Ctx c) {
-    if (c.st->done) return;
+    StateCopy sc;
+    sc.load(c.st);
     R red;
-    red.init();
-    const double al = c.st->alpha, om = c.st->omega, nom = -om;
+    red.init();  // ends in a barrier
+    if (sc.copy->done) return;
+    const double al = sc.copy->alpha, om = sc.copy->omega, nom = -om;
     for_pairs(c.n, [&](int64_t i, bool pair) {
         if (pair) {
             const double2 qh = ld2(c.qh, i), ph = ld2(c.ph, i), y = ld2(c.y, i), q = ld2(c.q, i),
@@ -168,7 +174,7 @@ __global__ void __launch_bounds__(256) k_cls_k4(Ctx c) {
         }
     });
     __shared__ double vals[R::K];
-    if (red.finish(c.g, vals) && threadIdx.x == 0) tail_cls_beta(c.st, vals, c.hist);
+    if (red.finish(c.g, vals)) sc.tail([&](SolverState *st) { tail_cls_beta(st, vals, c.hist); });
 }
 
 // K5: p = fma(beta, fma(-omega, s, p), r), phat = p * invd
@@ -201,8 +207,10 @@ __global__ void __launch_bounds__(256) k_pipe_setup1(Ctx c) {
 // set-up 2: w = A rhat, what = w * invd, <r0,r>, <r0,w> -> alpha0
 template <class R, int CAP>
 __global__ void __launch_bounds__(FusedScratch<CAP>::THREADS, 3) k_pipe_setup2(Ctx c) {
+    StateCopy sc;
+    sc.load(c.st);
     R red;
-    red.init();
+    red.init();  // ends in a barrier
     unsigned eb = 0u;
     fused_spmv<CAP>(c, c.rh, c.r0, eb, [&](int64_t i, double wi, double r0) {
         c.w[i] = wi;
@@ -213,9 +221,8 @@ __global__ void __launch_bounds__(FusedScratch<CAP>::THREADS, 3) k_pipe_setup2(C
     if (eb) atomicOr(c.err, eb);
     __shared__ double vals[R::K];
     if (red.template finish<FusedScratch<CAP>::BYTES, FusedScratch<CAP>::WARPS>(c.g, vals, 0u,
-                                                                               !(eb & ERR_TIMEOUT)) &&
-        threadIdx.x == 0)
-        tail_pipe_setup(c.st, vals);
+                                                                               !(eb & ERR_TIMEOUT)))
+        sc.tail([&](SolverState *st) { tail_pipe_setup(st, vals); });
 }
 
 // Launch shape of P1 and P3 per reducer (blocks per SM; two elements per thread
@@ -231,11 +238,13 @@ template <int K> struct P1Cfg<PlainR<K>> { static constexpr int blocks = 4, pair
 // not restrict-qualified, so later loads could not be issued early).
 template <class R>
 __global__ void __launch_bounds__(256, P1Cfg<R>::blocks) k_pipe_p1(Ctx c) {
-    if (c.st->done) return;
+    StateCopy sc;
+    sc.load(c.st);
     R red;
-    red.init();
-    const double al = c.st->alpha, nal = -al, be = c.st->beta, nom = -c.st->omega;
-    const bool first = c.st->iter == 0;
+    red.init();  // ends in a barrier
+    if (sc.copy->done) return;
+    const double al = sc.copy->alpha, nal = -al, be = sc.copy->beta, nom = -sc.copy->omega;
+    const bool first = sc.copy->iter == 0;
     if (P1Cfg<R>::pairs) {
         for_pairs(c.n, [&](int64_t i, bool pair) {
             if (pair) {
@@ -271,7 +280,7 @@ __global__ void __launch_bounds__(256, P1Cfg<R>::blocks) k_pipe_p1(Ctx c) {
             p1_store(c, i, p1_elem(p1_load(c, i, first), first, nal, be, nom, red));
     }
     __shared__ double vals[R::K];
-    if (red.finish(c.g, vals) && threadIdx.x == 0) tail_pipe_omega(c.st, vals);
+    if (red.finish(c.g, vals)) sc.tail([&](SolverState *st) { tail_pipe_omega(st, vals); });
 }
 
 // (P3's launch shape: see P1Cfg.)
@@ -283,10 +292,12 @@ template <int K> struct P3Cfg<PlainR<K>> { static constexpr int blocks = 3, pair
 // not restrict-qualified, so later loads could not be issued early).
 template <class R>
 __global__ void __launch_bounds__(256, P3Cfg<R>::blocks) k_pipe_p3(Ctx c) {
-    if (c.st->done) return;
+    StateCopy sc;
+    sc.load(c.st);
     R red;
-    red.init();
-    const double al = c.st->alpha, nal = -al, om = c.st->omega, nom = -om;
+    red.init();  // ends in a barrier
+    if (sc.copy->done) return;
+    const double al = sc.copy->alpha, nal = -al, om = sc.copy->omega, nom = -om;
     if (P3Cfg<R>::pairs) {
         for_pairs(c.n, [&](int64_t i, bool pair) {
             if (pair) {
@@ -327,7 +338,7 @@ __global__ void __launch_bounds__(256, P3Cfg<R>::blocks) k_pipe_p3(Ctx c) {
         }
     }
     __shared__ double vals[R::K];
-    if (red.finish(c.g, vals) && threadIdx.x == 0) tail_pipe_beta(c.st, vals, c.hist);
+    if (red.finish(c.g, vals)) sc.tail([&](SolverState *st) { tail_pipe_beta(st, vals, c.hist); });
 }
 
 // ---- launch -----------------------------------------------------------------------

@@ -102,23 +102,27 @@ template <class R>
 __global__ void __launch_bounds__(256) k_step_cls_setup(const Ctx *ctxs, const StepTask *tasks) {
     const StepTask t = tasks[blockIdx.x];
     const Ctx c = ctxs[t.sys];
-    if (c.st->done) return;
+    StateCopy sc;
+    sc.load(c.st);
     R red;
-    red.init();
+    red.init();  // ends in a barrier
+    if (sc.copy->done) return;
     bool bad = false;
     for (int64_t i = t.lo + threadIdx.x; i < t.hi; i += blockDim.x) red.add_sq(0, cls_setup_elem(c, i, bad));
     if (bad) atomicOr(c.err, 1u);
     __shared__ double vals[R::K];
-    if (red.finish(c.g, vals, t.nblk) && threadIdx.x == 0) tail_cls_setup(c.st, vals);
+    if (red.finish(c.g, vals, t.nblk)) sc.tail([&](SolverState *st) { tail_cls_setup(st, vals); });
 }
 
 template <class R>
 __global__ void __launch_bounds__(256, 3) k_step_cls_k1(const Ctx *ctxs, const StepTask *tasks) {
     const StepTask t = tasks[blockIdx.x];
     const Ctx c = ctxs[t.sys];
-    if (c.st->done) return;
+    StateCopy sc;
+    sc.load(c.st);
     R red;
-    red.init();
+    red.init();  // ends in a barrier
+    if (sc.copy->done) return;
     unsigned eb = 0u;
     seg_spmv(c, t, c.ph, c.r0, eb, [&](int64_t i, double si, double r0) {
         c.s[i] = si;
@@ -126,7 +130,8 @@ __global__ void __launch_bounds__(256, 3) k_step_cls_k1(const Ctx *ctxs, const S
     });
     if (eb) atomicOr(c.err, eb);
     __shared__ double vals[R::K];
-    if (red.template finish<SCR>(c.g, vals, t.nblk, !(eb & ERR_TIMEOUT)) && threadIdx.x == 0) tail_cls_alpha(c.st, vals);
+    if (red.template finish<SCR>(c.g, vals, t.nblk, !(eb & ERR_TIMEOUT)))
+        sc.tail([&](SolverState *st) { tail_cls_alpha(st, vals); });
 }
 
 __global__ void __launch_bounds__(256) k_step_cls_k2(const Ctx *ctxs, const StepTask *tasks) {
@@ -152,9 +157,11 @@ template <class R>
 __global__ void __launch_bounds__(256, 3) k_step_cls_k3(const Ctx *ctxs, const StepTask *tasks) {
     const StepTask t = tasks[blockIdx.x];
     const Ctx c = ctxs[t.sys];
-    if (c.st->done) return;
+    StateCopy sc;
+    sc.load(c.st);
     R red;
-    red.init();
+    red.init();  // ends in a barrier
+    if (sc.copy->done) return;
     unsigned eb = 0u;
     seg_spmv(c, t, c.qh, c.q, eb, [&](int64_t i, double yi, double qi) {
         c.y[i] = yi;
@@ -163,17 +170,20 @@ __global__ void __launch_bounds__(256, 3) k_step_cls_k3(const Ctx *ctxs, const S
     });
     if (eb) atomicOr(c.err, eb);
     __shared__ double vals[R::K];
-    if (red.template finish<SCR>(c.g, vals, t.nblk, !(eb & ERR_TIMEOUT)) && threadIdx.x == 0) tail_cls_omega(c.st, vals);
+    if (red.template finish<SCR>(c.g, vals, t.nblk, !(eb & ERR_TIMEOUT)))
+        sc.tail([&](SolverState *st) { tail_cls_omega(st, vals); });
 }
 
 template <class R>
 __global__ void __launch_bounds__(256, 4) k_step_cls_k4(const Ctx *ctxs, const StepTask *tasks) {
     const StepTask t = tasks[blockIdx.x];
     const Ctx c = ctxs[t.sys];
-    if (c.st->done) return;
+    StateCopy sc;
+    sc.load(c.st);
     R red;
-    red.init();
-    const double al = c.st->alpha, om = c.st->omega, nom = -om;
+    red.init();  // ends in a barrier
+    if (sc.copy->done) return;
+    const double al = sc.copy->alpha, om = sc.copy->omega, nom = -om;
     seg_pairs(t.lo, t.hi, [&](int64_t i, bool pair) {
         if (pair) {
             const double2 qh = ld2(c.qh, i), ph = ld2(c.ph, i), y = ld2(c.y, i), q = ld2(c.q, i),
@@ -195,7 +205,7 @@ __global__ void __launch_bounds__(256, 4) k_step_cls_k4(const Ctx *ctxs, const S
         }
     });
     __shared__ double vals[R::K];
-    if (red.finish(c.g, vals, t.nblk) && threadIdx.x == 0) tail_cls_beta(c.st, vals, c.hist);
+    if (red.finish(c.g, vals, t.nblk)) sc.tail([&](SolverState *st) { tail_cls_beta(st, vals, c.hist); });
 }
 
 __global__ void __launch_bounds__(256) k_step_cls_k5(const Ctx *ctxs, const StepTask *tasks) {
@@ -232,9 +242,11 @@ template <class R>
 __global__ void __launch_bounds__(256, 3) k_step_pipe_setup2(const Ctx *ctxs, const StepTask *tasks) {
     const StepTask t = tasks[blockIdx.x];
     const Ctx c = ctxs[t.sys];
-    if (c.st->done) return;
+    StateCopy sc;
+    sc.load(c.st);
     R red;
-    red.init();
+    red.init();  // ends in a barrier
+    if (sc.copy->done) return;
     unsigned eb = 0u;
     seg_spmv(c, t, c.rh, c.r0, eb, [&](int64_t i, double wi, double r0) {
         c.w[i] = wi;
@@ -244,7 +256,8 @@ __global__ void __launch_bounds__(256, 3) k_step_pipe_setup2(const Ctx *ctxs, co
     });
     if (eb) atomicOr(c.err, eb);
     __shared__ double vals[R::K];
-    if (red.template finish<SCR>(c.g, vals, t.nblk, !(eb & ERR_TIMEOUT)) && threadIdx.x == 0) tail_pipe_setup(c.st, vals);
+    if (red.template finish<SCR>(c.g, vals, t.nblk, !(eb & ERR_TIMEOUT)))
+        sc.tail([&](SolverState *st) { tail_pipe_setup(st, vals); });
 }
 
 // y = A x without a dot: the pipelined S10 (v = A zhat) and S18 / set-up (t = A what)
@@ -263,25 +276,29 @@ template <class R>
 __global__ void __launch_bounds__(256, 3) k_step_pipe_p1(const Ctx *ctxs, const StepTask *tasks) {
     const StepTask t = tasks[blockIdx.x];
     const Ctx c = ctxs[t.sys];
-    if (c.st->done) return;
+    StateCopy sc;
+    sc.load(c.st);
     R red;
-    red.init();
-    const double al = c.st->alpha, nal = -al, be = c.st->beta, nom = -c.st->omega;
-    const bool first = c.st->iter == 0;
+    red.init();  // ends in a barrier
+    if (sc.copy->done) return;
+    const double al = sc.copy->alpha, nal = -al, be = sc.copy->beta, nom = -sc.copy->omega;
+    const bool first = sc.copy->iter == 0;
     for (int64_t i = t.lo + threadIdx.x; i < t.hi; i += blockDim.x)
         p1_store(c, i, p1_elem(p1_load(c, i, first), first, nal, be, nom, red));
     __shared__ double vals[R::K];
-    if (red.finish(c.g, vals, t.nblk) && threadIdx.x == 0) tail_pipe_omega(c.st, vals);
+    if (red.finish(c.g, vals, t.nblk)) sc.tail([&](SolverState *st) { tail_pipe_omega(st, vals); });
 }
 
 template <class R>
 __global__ void __launch_bounds__(256, 2) k_step_pipe_p3(const Ctx *ctxs, const StepTask *tasks) {
     const StepTask t = tasks[blockIdx.x];
     const Ctx c = ctxs[t.sys];
-    if (c.st->done) return;
+    StateCopy sc;
+    sc.load(c.st);
     R red;
-    red.init();
-    const double al = c.st->alpha, nal = -al, om = c.st->omega, nom = -om;
+    red.init();  // ends in a barrier
+    if (sc.copy->done) return;
+    const double al = sc.copy->alpha, nal = -al, om = sc.copy->omega, nom = -om;
     for (int64_t i = t.lo + threadIdx.x; i < t.hi; i += blockDim.x) {
         const P3Out o = p3_elem(P3In{c.qh[i], c.y[i], c.q[i], c.ph[i], c.x[i], c.zh[i], c.wh[i], c.v[i], c.t[i],
                                      c.invd[i], c.r0[i], c.s[i], c.z[i]},
@@ -293,7 +310,7 @@ __global__ void __launch_bounds__(256, 2) k_step_pipe_p3(const Ctx *ctxs, const 
         c.wh[i] = o.wh;
     }
     __shared__ double vals[R::K];
-    if (red.finish(c.g, vals, t.nblk) && threadIdx.x == 0) tail_pipe_beta(c.st, vals, c.hist);
+    if (red.finish(c.g, vals, t.nblk)) sc.tail([&](SolverState *st) { tail_pipe_beta(st, vals, c.hist); });
 }
 
 using R1 = ExactR<1, SQ>;

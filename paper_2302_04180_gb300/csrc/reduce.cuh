@@ -314,6 +314,7 @@ struct PlainR {
     __device__ __forceinline__ void init() {
 #pragma unroll
         for (int k = 0; k < K; k++) s[k] = 0.0;
+        __syncthreads();  // as the exact reducers' init
     }
     __device__ __forceinline__ void add(int k, double x, double y) { s[k] = fma(x, y, s[k]); }
     __device__ __forceinline__ void add_sq(int k, double x) { s[k] = fma(x, x, s[k]); }

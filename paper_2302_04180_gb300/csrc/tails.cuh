@@ -21,6 +21,28 @@ __device__ __forceinline__ void stop(SolverState *st, int status) {
     st->done = 1;
 }
 
+// A kernel's copy of the solver state in shared memory: load() at its start
+// (every thread; a barrier before the first use), tail() in the block that runs
+// the scalar recurrence, which then touches no global memory between its
+// dependent steps. Only that block writes the state during the kernel.
+struct StateCopy {
+    SolverState *st, *copy;
+    static constexpr int WORDS = (int)(sizeof(SolverState) / 4);
+    __device__ __forceinline__ void load(SolverState *from) {
+        __shared__ __align__(8) uint32_t s_state[WORDS];
+        st = from;
+        copy = reinterpret_cast<SolverState *>(s_state);
+        for (int j = threadIdx.x; j < WORDS; j += blockDim.x) s_state[j] = reinterpret_cast<const uint32_t *>(from)[j];
+    }
+    template <class F>
+    __device__ __forceinline__ void tail(F &&f) {
+        if (threadIdx.x == 0) f(copy);
+        __syncthreads();
+        for (int j = threadIdx.x; j < WORDS; j += blockDim.x)
+            reinterpret_cast<uint32_t *>(st)[j] = reinterpret_cast<const uint32_t *>(copy)[j];
+    }
+};
+
 // set-up, classic: rho = <r0,r0>, tau0 = sqrt(rho), tau_max = tol * tau0
 __device__ __forceinline__ void tail_cls_setup(SolverState *st, const double *v) {
     const double rho = v[0];
