@@ -120,6 +120,7 @@ struct Workspace {
     double *d_out = nullptr;
     unsigned *h_err = nullptr;
     DiagArgs *h_diag = nullptr;
+    BatchOut *h_small = nullptr;
     Buf vec, hist, diag, stage[8];
     Buf batch_work, batch_hist, batch_sys, batch_order, batch_out, batch_queue;
     Buf step_ctx, step_state, step_scr, step_tasks;  // the stepped batch schedule
@@ -169,6 +170,7 @@ int ws_get(cudaStream_t s, Workspace **out) {
     if (e == cudaSuccess) e = cudaMallocHost(&w->h_out, KMAX * sizeof(double));
     if (e == cudaSuccess) e = cudaMallocHost(&w->h_err, sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMallocHost(&w->h_diag, sizeof(DiagArgs));
+    if (e == cudaSuccess) e = cudaMallocHost(&w->h_small, sizeof(BatchOut));
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         delete w;
@@ -192,6 +194,7 @@ void ws_free(Workspace *w) {
     cudaFreeHost(w->h_out);
     cudaFreeHost(w->h_err);
     cudaFreeHost(w->h_diag);
+    cudaFreeHost(w->h_small);
     cudaFree(w->vec.p);
     cudaFree(w->diag.p);
     cudaFree(w->hist.p);
@@ -600,6 +603,12 @@ int rbs_solve(const rbs_csr *A, const double *b, const double *x0, const double 
                         stream);
 }
 
+// A solve's own outcome as the call's.
+static int solve_status(int status) {
+    if (status == RBS_OK) return RBS_OK;
+    return fail(status, status == RBS_EBREAKDOWN ? "breakdown: zero denominator" : "non-finite scalar");
+}
+
 int rbs_solve_ex(const rbs_csr *A, const double *b, const double *x0, const double *jacobi_diag,
                  double tol, int32_t maxit, int32_t variant, const rbs_opts *opts, double *x_out,
                  rbs_info *info, rbs_history *hist, rbs_prof *prof, void *stream) {
@@ -639,6 +648,54 @@ int rbs_solve_ex(const rbs_csr *A, const double *b, const double *x0, const doub
     if (x0 && (rc = to_device(w, 4, x0, (size_t)n * 8, &dx0))) return rc;
     if (jacobi_diag && (rc = to_device(w, 5, jacobi_diag, (size_t)n * 8, &ddiag))) return rc;
 
+    const int hcap = hist ? (hist->cap < maxit ? hist->cap : maxit) : 0;
+    CK(ensure(w->hist, (size_t)(hcap > 0 ? hcap : 1) * RBS_HIST_W * 8));
+
+    // a small system: one cluster, one launch (kernels_small.cu). The knobs and
+    // the loop drivers that shape the other path's launches, and profiles of its
+    // kernels, stay with it.
+    const bool knobs = p_spmv_mode.load() || p_spmv_block.load() || p_vec_grid.load() || p_vec_block.load() ||
+                       p_test_stall.load();
+    if (o.dot_mode == RBS_DOT_EXACT && o.loop_mode == RBS_LOOP_GRAPH && !(o.profile && prof) && !knobs &&
+        small_fits(n, nnz, variant)) {
+        double *dx = x_out;
+        if (!is_device_ptr(x_out)) {
+            CK(ensure(w->vec, (size_t)n * 8));
+            dx = (double *)w->vec.p;
+        }
+        CSRArgs A1{n, nnz, (const int64_t *)rowptr, (const int32_t *)col, (const double *)val};
+        CK(ensure(w->batch_out, sizeof(BatchOut)));
+        BatchOut *d_out = (BatchOut *)w->batch_out.p, O;
+        CK(cudaMemsetAsync(d_out, 0, sizeof(BatchOut), w->stream));
+        CK(launch_small(A1, (const double *)db, (const double *)dx0, (const double *)ddiag, dx, tol, maxit, variant,
+                        (double *)w->hist.p, hcap, d_out, w->stream));
+        CK(cudaMemcpyAsync(w->h_small, d_out, sizeof(BatchOut), cudaMemcpyDeviceToHost, w->stream));
+        CK(cudaStreamSynchronize(w->stream));
+        O = *w->h_small;
+        if (O.err & 1u) return fail(RBS_EINVAL, "invalid CSR structure");
+        if (!(O.err & SMALL_NO_ROOM)) {
+            if (O.err & 2u) return fail(RBS_EINVAL, "zero, NaN or missing diagonal entry");
+            info->iters = O.iters;
+            info->status = O.status;
+            info->tau0 = O.tau0;
+            info->tau_final = O.tau_final;
+            info->rho0 = O.rho0;
+            info->tau_max = O.tau_max;
+            info->alpha0 = variant == RBS_PIPELINED ? O.alpha0 : __builtin_nan("");
+            info->mu0 = variant == RBS_PIPELINED ? O.mu0 : 0.0;
+            info->converged = O.converged;
+            if (hist) {
+                hist->len = O.iters < hcap ? O.iters : hcap;
+                if (hist->len > 0)
+                    CK(cudaMemcpyAsync(hist->rec, w->hist.p, (size_t)hist->len * RBS_HIST_W * 8,
+                                       cudaMemcpyDeviceToHost, w->stream));
+            }
+            if (dx != x_out) CK(cudaMemcpyAsync(x_out, dx, (size_t)n * 8, cudaMemcpyDeviceToHost, w->stream));
+            if (dx != x_out || (hist && hist->len > 0)) CK(cudaStreamSynchronize(w->stream));
+            return solve_status(O.status);
+        }
+    }
+
     // solver vectors, 256-byte aligned each
     const size_t stride = ((size_t)n * 8 + 255) / 256 * 256;
     CK(ensure(w->vec, stride * NVEC));
@@ -650,9 +707,6 @@ int rbs_solve_ex(const rbs_csr *A, const double *b, const double *x0, const doub
     V.r = vp[1]; V.r0 = vp[2]; V.p = vp[3]; V.ph = vp[4]; V.s = vp[5]; V.q = vp[6]; V.qh = vp[7];
     V.y = vp[8]; V.invd = vp[9]; V.rh = vp[10]; V.w = vp[11]; V.wh = vp[12]; V.t = vp[13];
     V.sh = vp[14]; V.z = vp[15]; V.zh = vp[16]; V.v = vp[17];
-
-    const int hcap = hist ? (hist->cap < maxit ? hist->cap : maxit) : 0;
-    CK(ensure(w->hist, (size_t)(hcap > 0 ? hcap : 1) * RBS_HIST_W * 8));
 
     SolverState *h = w->h_st;
     memset(h, 0, sizeof *h);
@@ -827,10 +881,7 @@ int rbs_solve_ex(const rbs_csr *A, const double *b, const double *x0, const doub
             }
         }
     }
-    if (h->status != RBS_OK)
-        return fail(h->status, h->status == RBS_EBREAKDOWN ? "breakdown: zero denominator"
-                                                           : "non-finite scalar");
-    return RBS_OK;
+    return solve_status(h->status);
 }
 
 }  // extern "C"

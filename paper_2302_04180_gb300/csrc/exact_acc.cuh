@@ -285,6 +285,25 @@ __device__ __forceinline__ unsigned char *warp_scratch() {
     return buf + (threadIdx.x >> 5) * BYTES;
 }
 
+// Windows of one anchor (the usual case): every word summed over the warp in two
+// 16-bit halves, the top word's upper half signed, and one atomic per word.
+template <int Q>
+__device__ __forceinline__ void warp_sum_words(Win<Q> &W, unsigned long long *sacc, int lane, int anchor) {
+    constexpr unsigned FULL = 0xffffffffu;
+    long long mine = 0;
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
+        const uint32_t w = W.w[k];  // zero in lanes without a window
+        const long long low = (long long)__reduce_add_sync(FULL, w & 0xffffu);
+        const long long high =
+            k < 7 ? (long long)__reduce_add_sync(FULL, w >> 16) : (long long)__reduce_add_sync(FULL, (int)w >> 16);
+        if (lane == k) mine = low + high * 65536;
+        W.w[k] = 0u;
+    }
+    if (lane < 8 && mine && anchor + lane < NL) sacc_add(&sacc[anchor + lane], mine);
+    W.a = WIN_EMPTY;
+}
+
 template <int Q, int SCRATCH = FLUSH_SCRATCH, int WARPS = MAX_WARPS>
 __device__ __forceinline__ void warp_flush(Win<Q> &W, unsigned long long *sacc) {
     static_assert(SCRATCH >= FLUSH_SCRATCH, "flush staging");
@@ -299,20 +318,7 @@ __device__ __forceinline__ void warp_flush(Win<Q> &W, unsigned long long *sacc) 
         return;
     }
     if (lo == hi) {
-        // one anchor (the usual case): every word summed over the warp in two
-        // 16-bit halves, the top word's upper half signed
-        long long mine = 0;
-#pragma unroll
-        for (int k = 0; k < 8; k++) {
-            const uint32_t w = W.w[k];  // zero in lanes without a window
-            const long long low = (long long)__reduce_add_sync(FULL, w & 0xffffu);
-            const long long high = k < 7 ? (long long)__reduce_add_sync(FULL, w >> 16)
-                                         : (long long)__reduce_add_sync(FULL, (int)w >> 16);
-            if (lane == k) mine = low + high * 65536;
-            W.w[k] = 0u;
-        }
-        if (lane < 8 && mine && lo + lane < NL) sacc_add(&sacc[lo + lane], mine);
-        W.a = WIN_EMPTY;
+        warp_sum_words<Q>(W, sacc, lane, lo);
         return;
     }
     __syncwarp();
@@ -357,8 +363,8 @@ __device__ __forceinline__ long long partial_norm(const unsigned long long *L, i
 
 // Round an exact value given as carry-save signed limbs (|limb| < 2^62) once
 // to nearest even, given its lowest and highest nonzero limbs lo and hi (lo =
-// -1 or lo > hi: the value is zero). G is modified (normalised in place). One
-// thread.
+// -1 or lo > hi: the value is zero; the two limbs past hi are read and must be
+// zero). G is modified (normalised in place). One thread.
 static __device__ __noinline__ double round_limbs_span(long long *G, uint32_t flags, int lo, int hi) {
     if (flags & F_NAN) return qnan();
     if ((flags & F_PINF) && (flags & F_NINF)) return qnan();
@@ -428,62 +434,67 @@ static __device__ __noinline__ double round_limbs_thread(long long *G, uint32_t 
     return round_limbs_span(G, flags, lo, hi);
 }
 
-// round_limbs_span by a whole warp (all 32 lanes, same arguments; every lane
-// gets the value): one limb per lane, carries and borrows resolved over the
-// lanes with ballots instead of limb by limb (a chain of dependent shared-memory
-// reads and writes; the rounding is part of every reduction's latency). Spans
-// over 29 limbs, subnormal results and non-finite flags take the serial way.
-static __device__ __noinline__ double round_limbs_warp(long long *G, uint32_t flags, int lo, int hi) {
+// The rounding by a whole warp: lane l holds limb lo + l (carry-save, |t| < 2^62;
+// lanes 29 and up zero), carries and borrows are resolved over the lanes with
+// ballots instead of limb by limb (a chain of dependent shared-memory reads and
+// writes; the rounding is part of every reduction's latency). Every lane gets the
+// value; false for a subnormal result, which is left to round_limbs_span.
+__device__ __forceinline__ bool round_lanes(long long t, int lo, double &value) {
     constexpr unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     // carry into each bit of a ripple with generate mask g and propagate mask p
     auto ripple = [](uint32_t g, uint32_t p) { return ((g | p) + g) ^ (g | p) ^ g; };
-    if (flags == 0u && (lo < 0 || lo > hi)) return 0.0;
-    if (flags == 0u && hi - lo <= 28) {
-        long long t = lane <= hi - lo ? G[lo + lane] : 0ll;
-        // two rounds leave -1 .. 2^32 in each lane
+    // two rounds leave -1 .. 2^32 in each lane
 #pragma unroll
-        for (int i = 0; i < 2; i++) {
-            const int up = __shfl_up_sync(FULL, (int)(t >> 32), 1);
-            t = (t & 0xffffffffll) + (lane ? up : 0);
-        }
-        const uint32_t n = t < 0 ? 1u : 0u;
-        uint32_t d = n ? 0u : (uint32_t)t;
-        const uint32_t cin =
-            ripple(__ballot_sync(FULL, t == 0x100000000ll), __ballot_sync(FULL, t == 0xffffffffll));
-        d += (cin >> lane) & 1u;
-        const uint32_t bin = ripple(__ballot_sync(FULL, n && d == 0u), __ballot_sync(FULL, d == n));
-        d -= n + ((bin >> lane) & 1u);
-        const bool neg = (__ballot_sync(FULL, (int)d < 0) >> 31) != 0u;  // lanes past the span hold the sign
-        uint32_t nz = __ballot_sync(FULL, d != 0u);
-        if (nz == 0u) return 0.0;
-        if (neg) {
-            const int z = __ffs(nz) - 1;
-            d = lane < z ? 0u : lane == z ? 0u - d : ~d;
-            nz = __ballot_sync(FULL, d != 0u);
-        }
-        const int tw = 31 - __clz(nz);
-        const uint32_t w2 = __shfl_sync(FULL, d, tw);
-        uint32_t w1 = __shfl_sync(FULL, d, tw >= 1 ? tw - 1 : 0), w0 = __shfl_sync(FULL, d, tw >= 2 ? tw - 2 : 0);
-        if (tw < 1) w1 = 0u;
-        if (tw < 2) w0 = 0u;
-        const int lead = __clz(w2);
-        const int lsb = 32 * (lo + tw) + 31 - lead - 52;  // of the 53-bit significand
-        if (lsb >= 1074) {
-            const uint32_t top = __funnelshift_l(w1, w2, lead), mid = __funnelshift_l(w0, w1, lead);
-            const unsigned long long v = ((unsigned long long)top << 32) | mid;
-            unsigned long long mant = v >> 11;
-            const bool sticky = (v & 0x3ffull) != 0ull || (w0 << lead) != 0u || (tw >= 3 && (nz & ((1u << (tw - 2)) - 1u)));
-            if (((v >> 10) & 1ull) && (sticky || (mant & 1ull))) mant += 1ull;
-            unsigned long long bits = ((unsigned long long)(lsb - 1074) << 52) + mant;
-            if (lsb - 1074 >= 2047 || bits >= 0x7ff0000000000000ull) bits = 0x7ff0000000000000ull;
-            if (neg) bits |= 0x8000000000000000ull;
-            return __longlong_as_double((long long)bits);
-        }
+    for (int i = 0; i < 2; i++) {
+        const int up = __shfl_up_sync(FULL, (int)(t >> 32), 1);
+        t = (t & 0xffffffffll) + (lane ? up : 0);
     }
+    const uint32_t n = t < 0 ? 1u : 0u;
+    uint32_t d = n ? 0u : (uint32_t)t;
+    const uint32_t cin = ripple(__ballot_sync(FULL, t == 0x100000000ll), __ballot_sync(FULL, t == 0xffffffffll));
+    d += (cin >> lane) & 1u;
+    const uint32_t bin = ripple(__ballot_sync(FULL, n && d == 0u), __ballot_sync(FULL, d == n));
+    d -= n + ((bin >> lane) & 1u);
+    const bool neg = (__ballot_sync(FULL, (int)d < 0) >> 31) != 0u;  // lanes past the span hold the sign
+    uint32_t nz = __ballot_sync(FULL, d != 0u);
+    value = 0.0;
+    if (nz == 0u) return true;
+    if (neg) {
+        const int z = __ffs(nz) - 1;
+        d = lane < z ? 0u : lane == z ? 0u - d : ~d;
+        nz = __ballot_sync(FULL, d != 0u);
+    }
+    const int tw = 31 - __clz(nz);
+    const uint32_t w2 = __shfl_sync(FULL, d, tw);
+    uint32_t w1 = __shfl_sync(FULL, d, tw >= 1 ? tw - 1 : 0), w0 = __shfl_sync(FULL, d, tw >= 2 ? tw - 2 : 0);
+    if (tw < 1) w1 = 0u;
+    if (tw < 2) w0 = 0u;
+    const int lead = __clz(w2);
+    const int lsb = 32 * (lo + tw) + 31 - lead - 52;  // of the 53-bit significand
+    if (lsb < 1074) return false;
+    const uint32_t top = __funnelshift_l(w1, w2, lead), mid = __funnelshift_l(w0, w1, lead);
+    const unsigned long long v = ((unsigned long long)top << 32) | mid;
+    unsigned long long mant = v >> 11;
+    const bool sticky = (v & 0x3ffull) != 0ull || (w0 << lead) != 0u || (tw >= 3 && (nz & ((1u << (tw - 2)) - 1u)));
+    if (((v >> 10) & 1ull) && (sticky || (mant & 1ull))) mant += 1ull;
+    unsigned long long bits = ((unsigned long long)(lsb - 1074) << 52) + mant;
+    if (lsb - 1074 >= 2047 || bits >= 0x7ff0000000000000ull) bits = 0x7ff0000000000000ull;
+    if (neg) bits |= 0x8000000000000000ull;
+    value = __longlong_as_double((long long)bits);
+    return true;
+}
+
+// round_limbs_span by a whole warp (all 32 lanes, same arguments; every lane
+// gets the value). Spans over 29 limbs, subnormal results and non-finite flags
+// take the serial way.
+static __device__ __noinline__ double round_limbs_warp(long long *G, uint32_t flags, int lo, int hi) {
+    const int lane = threadIdx.x & 31;
     double v = 0.0;
+    if (flags == 0u && (lo < 0 || lo > hi)) return 0.0;
+    if (flags == 0u && hi - lo <= 28 && round_lanes(lane <= hi - lo ? G[lo + lane] : 0ll, lo, v)) return v;
     if (lane == 0) v = round_limbs_span(G, flags, lo, hi);
-    return __shfl_sync(FULL, v, 0);
+    return __shfl_sync(0xffffffffu, v, 0);
 }
 
 // Block- and grid-level finish of K exact reductions, once every thread's own

@@ -158,6 +158,18 @@ cudaError_t launch_batch(const BatchSys *d_sys, const int32_t *d_order, const in
 // Clusters of `csize` CTAs that fit on the device at once (0 if none).
 int batch_max_clusters(int csize);
 
+// ---- one small system in one cluster (kernels_small.cu) ----
+constexpr int SMALL_CTAS = 16;
+// Whether this device can run such a solve and the system fits, its nonzeros
+// spread evenly over the rows. A solve whose rows do not fit after all sets
+// bit 8 in d_out->err and leaves x alone.
+bool small_fits(int64_t n, int64_t nnz, int variant);
+constexpr unsigned SMALL_NO_ROOM = 8u;
+// Structure check, Jacobi (diag or the first stored (i, i)), set-up and loop;
+// *d_out zero before.
+cudaError_t launch_small(const CSRArgs &A, const double *b, const double *x0, const double *diag, double *x, double tol,
+                         int32_t maxit, int variant, double *hist, int32_t hist_cap, BatchOut *d_out, cudaStream_t s);
+
 // ---- per-step kernels of the serving engine (kernels_step.cu) ----
 // One block of a per-step launch: rows [lo, hi) of the system in slot `sys`
 // (lo even), which has nblk blocks in the launch.
