@@ -32,7 +32,7 @@ __device__ __forceinline__ void add_pairs(R &red, const double2 (&x)[U], const d
         yv[2 * u] = y[u].x;
         yv[2 * u + 1] = y[u].y;
     }
-    red.template add<2 * U>(xv, yv);
+    red.template add<2 * U>(0, xv, yv);
 }
 
 // Exact dots over the same length (Sec. 2 exdot; Sec. 4.1/4.2 merged
@@ -51,7 +51,7 @@ __device__ __forceinline__ void add_pairs(R &red, const double2 (&x)[U], const d
 template <int W, bool EXPORT>
 __global__ void __launch_bounds__(256, EXDOT_BLOCKS)
     k_exdot(const __grid_constant__ DotArgs a, int64_t n, DotScratch *g, double *out, long long *limbs, int32_t *flags_out) {
-    using R = ExactW<W>;
+    using R = ExactRows<1, W, true>;
     R red;
     const int slot = EXPORT ? 0 : blockIdx.y;
     const double *__restrict__ xp = a.x[slot], *__restrict__ yp = a.y[slot];
@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(256, EXDOT_BLOCKS)
         };
         if (full > 0) load(xa, ya);
         red.init();
-        red.open(max(R::limb_of(x0[0].x, y0[0].x), R::limb_of(x0[0].y, y0[0].y)));
+        red.open({max(R::limb_of(x0[0].x, y0[0].x), R::limb_of(x0[0].y, y0[0].y))});
         add_pairs<1>(red, x0, y0);
         int64_t s = 0;
         for (; s + 2 < full; s += 2) {
@@ -103,15 +103,15 @@ __global__ void __launch_bounds__(256, EXDOT_BLOCKS)
             y0[0] = __ldcs(y2 + j);
             add_pairs<1>(red, x0, y0);
         }
-        if ((n & 1) && gtid() == 0) red.add_one(xp[n - 1], yp[n - 1]);
+        if ((n & 1) && gtid() == 0) red.add(0, xp[n - 1], yp[n - 1]);
     } else {
         int64_t i = gtid();
         red.init();
-        red.open(i < n ? R::limb_of(xp[i], yp[i]) : -1);
-        for (; i < n; i += st) red.add_one(xp[i], yp[i]);
+        red.open({i < n ? R::limb_of(xp[i], yp[i]) : -1});
+        for (; i < n; i += st) red.add(0, xp[i], yp[i]);
     }
     __shared__ double val[1];
-    if (red.finish(g, slot, val, EXPORT, limbs, flags_out) && !EXPORT && threadIdx.x == 0) out[slot] = val[0];
+    if (red.finish(g, val, 0u, slot, EXPORT, limbs, flags_out) && !EXPORT && threadIdx.x == 0) out[slot] = val[0];
 }
 
 // Words per sign for the "exdot.window" knob: 16 unless it asks for a small

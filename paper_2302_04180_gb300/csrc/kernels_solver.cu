@@ -145,34 +145,14 @@ __global__ void __launch_bounds__(FusedScratch<CAP>::THREADS, 3) k_cls_k3(Ctx c)
 
 // K4: x = fma(omega, qhat, fma(alpha, phat, x)), r = fma(-omega, y, q), <r0,r>, <r,r>
 template <class R>
-__global__ void __launch_bounds__(256) k_cls_k4(Ctx c) {
+__global__ void __launch_bounds__(256, 4) k_cls_k4(Ctx c) {
     StateCopy sc;
     sc.load(c.st);
     R red;
     red.init();  // ends in a barrier
     if (sc.copy->done) return;
-    const double al = sc.copy->alpha, om = sc.copy->omega, nom = -om;
-    for_pairs(c.n, [&](int64_t i, bool pair) {
-        if (pair) {
-            const double2 qh = ld2(c.qh, i), ph = ld2(c.ph, i), y = ld2(c.y, i), q = ld2(c.q, i),
-                          r0 = ld2(c.r0, i);
-            const double2 x = ld2(c.x, i);
-            const VPair u0 = cls_k4(al, om, nom, qh.x, ph.x, x.x, y.x, q.x);
-            const VPair u1 = cls_k4(al, om, nom, qh.y, ph.y, x.y, y.y, q.y);
-            st2(c.x, i, make_double2(u0.a, u1.a));
-            st2(c.r, i, make_double2(u0.b, u1.b));
-            red.add(0, r0.x, u0.b);
-            red.add(0, r0.y, u1.b);
-            red.add_sq(1, u0.b);
-            red.add_sq(1, u1.b);
-        } else {
-            const VPair u = cls_k4(al, om, nom, c.qh[i], c.ph[i], c.x[i], c.y[i], c.q[i]);
-            c.x[i] = u.a;
-            c.r[i] = u.b;
-            red.add(0, c.r0[i], u.b);
-            red.add_sq(1, u.b);
-        }
-    });
+    cls_k4_pairs(c, red, sc.copy->alpha, sc.copy->omega, gtid(), c.n >> 1, gstride(),
+                 (c.n & 1) && gtid() == 0 ? c.n - 1 : -1);
     __shared__ double vals[R::K];
     if (red.finish(c.g, vals)) sc.tail([&](SolverState *st) { tail_cls_beta(st, vals, c.hist); });
 }
@@ -225,11 +205,12 @@ __global__ void __launch_bounds__(FusedScratch<CAP>::THREADS, 3) k_pipe_setup2(C
         sc.tail([&](SolverState *st) { tail_pipe_setup(st, vals); });
 }
 
-// Launch shape of P1 and P3 per reducer (blocks per SM; two elements per thread
-// with 16-byte accesses or one), the fastest measured on Poisson 256^3. With the
-// exact reducer, pairs issue twice the loads per thread and lower occupancy
-// keeps the dot windows in registers: P3 at two blocks uses 121 registers, no
-// spills, where four blocks spilled the five windows; P1 is best at three.
+// Launch shape of P1 and P3 per reducer (blocks per SM that registers are kept
+// for; two elements per thread with 16-byte accesses or one), the fastest measured
+// on Poisson 256^3. With the exact reducer P1 runs two of its three blocks
+// (P1_GRID): a third one's loads in flight overrun the L1 beside the windows
+// (192^3: 196 us against 184).
+constexpr int P1_GRID = 2;
 template <class R> struct P1Cfg { static constexpr int blocks = 3, pairs = 1; };
 template <int K> struct P1Cfg<PlainR<K>> { static constexpr int blocks = 4, pairs = 0; };
 
@@ -246,35 +227,8 @@ __global__ void __launch_bounds__(256, P1Cfg<R>::blocks) k_pipe_p1(Ctx c) {
     const double al = sc.copy->alpha, nal = -al, be = sc.copy->beta, nom = -sc.copy->omega;
     const bool first = sc.copy->iter == 0;
     if (P1Cfg<R>::pairs) {
-        for_pairs(c.n, [&](int64_t i, bool pair) {
-            if (pair) {
-                const double2 rh = ld2(c.rh, i), w = ld2(c.w, i), wh = ld2(c.wh, i), t = ld2(c.t, i),
-                              r = ld2(c.r, i), d = ld2(c.invd, i);
-                double2 ph{0.0, 0.0}, s{0.0, 0.0}, sh{0.0, 0.0}, z{0.0, 0.0}, zh{0.0, 0.0}, v{0.0, 0.0};
-                if (!first) {
-                    ph = ld2(c.ph, i);
-                    s = ld2(c.s, i);
-                    sh = ld2(c.sh, i);
-                    z = ld2(c.z, i);
-                    zh = ld2(c.zh, i);
-                    v = ld2(c.v, i);
-                }
-                const P1Out o0 = p1_elem(P1In{rh.x, w.x, wh.x, t.x, r.x, d.x, ph.x, s.x, sh.x, z.x, zh.x, v.x}, first,
-                                         nal, be, nom, red);
-                const P1Out o1 = p1_elem(P1In{rh.y, w.y, wh.y, t.y, r.y, d.y, ph.y, s.y, sh.y, z.y, zh.y, v.y}, first,
-                                         nal, be, nom, red);
-                st2(c.ph, i, make_double2(o0.ph, o1.ph));
-                st2(c.s, i, make_double2(o0.s, o1.s));
-                st2(c.sh, i, make_double2(o0.sh, o1.sh));
-                st2(c.z, i, make_double2(o0.z, o1.z));
-                st2(c.q, i, make_double2(o0.q, o1.q));
-                st2(c.qh, i, make_double2(o0.qh, o1.qh));
-                st2(c.y, i, make_double2(o0.y, o1.y));
-                st2(c.zh, i, make_double2(o0.zh, o1.zh));
-            } else {
-                p1_store(c, i, p1_elem(p1_load(c, i, first), first, nal, be, nom, red));
-            }
-        });
+        pipe_p1_pairs(c, red, first, nal, be, nom, gtid(), c.n >> 1, gstride(),
+                      (c.n & 1) && gtid() == 0 ? c.n - 1 : -1);
     } else {
         for (int64_t i = gtid(); i < c.n; i += gstride())
             p1_store(c, i, p1_elem(p1_load(c, i, first), first, nal, be, nom, red));
@@ -299,32 +253,7 @@ __global__ void __launch_bounds__(256, P3Cfg<R>::blocks) k_pipe_p3(Ctx c) {
     if (sc.copy->done) return;
     const double al = sc.copy->alpha, nal = -al, om = sc.copy->omega, nom = -om;
     if (P3Cfg<R>::pairs) {
-        for_pairs(c.n, [&](int64_t i, bool pair) {
-            if (pair) {
-                const double2 qh = ld2(c.qh, i), y = ld2(c.y, i), q = ld2(c.q, i), ph = ld2(c.ph, i),
-                              x = ld2(c.x, i), zh = ld2(c.zh, i), wh = ld2(c.wh, i), v = ld2(c.v, i),
-                              t = ld2(c.t, i), d = ld2(c.invd, i), r0 = ld2(c.r0, i), s = ld2(c.s, i),
-                              z = ld2(c.z, i);
-                const P3Out o0 = p3_elem(P3In{qh.x, y.x, q.x, ph.x, x.x, zh.x, wh.x, v.x, t.x, d.x, r0.x, s.x, z.x},
-                                         al, nal, om, nom, red);
-                const P3Out o1 = p3_elem(P3In{qh.y, y.y, q.y, ph.y, x.y, zh.y, wh.y, v.y, t.y, d.y, r0.y, s.y, z.y},
-                                         al, nal, om, nom, red);
-                st2(c.x, i, make_double2(o0.x, o1.x));
-                st2(c.r, i, make_double2(o0.r, o1.r));
-                st2(c.rh, i, make_double2(o0.rh, o1.rh));
-                st2(c.w, i, make_double2(o0.w, o1.w));
-                st2(c.wh, i, make_double2(o0.wh, o1.wh));
-            } else {
-                const P3Out o = p3_elem(P3In{c.qh[i], c.y[i], c.q[i], c.ph[i], c.x[i], c.zh[i], c.wh[i], c.v[i],
-                                             c.t[i], c.invd[i], c.r0[i], c.s[i], c.z[i]},
-                                        al, nal, om, nom, red);
-                c.x[i] = o.x;
-                c.r[i] = o.r;
-                c.rh[i] = o.rh;
-                c.w[i] = o.w;
-                c.wh[i] = o.wh;
-            }
-        });
+        pipe_p3_pairs(c, red, al, om, gtid(), c.n >> 1, gstride(), (c.n & 1) && gtid() == 0 ? c.n - 1 : -1);
     } else {
         for (int64_t i = gtid(); i < c.n; i += gstride()) {
             const P3Out o = p3_elem(P3In{c.qh[i], c.y[i], c.q[i], c.ph[i], c.x[i], c.zh[i], c.wh[i], c.v[i], c.t[i],
@@ -385,7 +314,7 @@ static cudaError_t plain_spmv(const SolverArgs &a, const double *x, double *y, c
     return launch_spmv(a.A, x, y, a.st, a.err, a.spmv, s);
 }
 
-template <class R1, class R2, class R5>
+template <class R1, class R2, class V2, class V5>
 static cudaError_t setup_t(const SolverArgs &a, int variant, cudaStream_t s, KernelTimer *tm) {
     Ctx c = make_ctx(a);
     if (variant == RBS_CLASSIC) {
@@ -400,7 +329,7 @@ static cudaError_t setup_t(const SolverArgs &a, int variant, cudaStream_t s, Ker
     return cudaGetLastError();
 }
 
-template <class R1, class R2, class R5>
+template <class R1, class R2, class V2, class V5>
 static cudaError_t iter_t(const SolverArgs &a, int variant, cudaStream_t s, KernelTimer *tm) {
     Ctx c = make_ctx(a);
     if (variant == RBS_CLASSIC) {
@@ -411,12 +340,12 @@ static cudaError_t iter_t(const SolverArgs &a, int variant, cudaStream_t s, Kern
         with_cap(a.spmv.mode, [&](auto cap) {
             TIMED(PK_K3, (k_cls_k3<R2, decltype(cap)::value><<<a.k3.grid, a.k3.block, 0, s>>>(c)));
         });
-        TIMED(PK_K4, (k_cls_k4<R2><<<a.vec.grid, a.vec.block, 0, s>>>(c)));
+        TIMED(PK_K4, (k_cls_k4<V2><<<a.vec.grid, a.vec.block, 0, s>>>(c)));
         TIMED(PK_VEC, (k_cls_k5<<<a.vec.grid, a.vec.block, 0, s>>>(c)));
     } else {
-        TIMED(PK_VEC_DOT, (k_pipe_p1<R2><<<a.vec.grid, a.vec.block, 0, s>>>(c)));
+        TIMED(PK_VEC_DOT, (k_pipe_p1<V2><<<a.vec.grid, a.vec.block, 0, s>>>(c)));
         TIMED(PK_SPMV, (plain_spmv(a, a.v.zh, a.v.v, s)));
-        TIMED(PK_VEC_DOT, (k_pipe_p3<R5><<<a.p3.grid, a.p3.block, 0, s>>>(c)));
+        TIMED(PK_VEC_DOT, (k_pipe_p3<V5><<<a.p3.grid, a.p3.block, 0, s>>>(c)));
         TIMED(PK_SPMV, (plain_spmv(a, a.v.wh, a.v.t, s)));
     }
     return cudaGetLastError();
@@ -425,9 +354,8 @@ static cudaError_t iter_t(const SolverArgs &a, int variant, cudaStream_t s, Kern
 // Shared-memory carveout (percent of the unified L1/shared storage, -1 = the
 // driver's choice) of the kernels that stage data per warp. The x gathers of
 // the SpMV live on L1 hits, so the split is a tuning knob, not a maximum.
-template <class R1, class R2, class R5>
+template <class R1, class R2, class V2, class V5>
 static void prefer_shared(int c) {
-    cudaFuncSetAttribute(k_cls_k4<R2>, cudaFuncAttributePreferredSharedMemoryCarveout, c);
     for (int mode : {SPMV_MODE_SHORT, SPMV_MODE_LONG, SPMV_MODE_DIAG7, SPMV_MODE_DIAG32})
         with_cap(mode, [&](auto cap) {
             constexpr int CAP = decltype(cap)::value;
@@ -437,8 +365,8 @@ static void prefer_shared(int c) {
             cudaFuncSetAttribute(k_cls_k3<R2, CAP>, cudaFuncAttributePreferredSharedMemoryCarveout, share);
             cudaFuncSetAttribute(k_pipe_setup2<R2, CAP>, cudaFuncAttributePreferredSharedMemoryCarveout, share);
         });
-    cudaFuncSetAttribute(k_pipe_p1<R2>, cudaFuncAttributePreferredSharedMemoryCarveout, c);
-    cudaFuncSetAttribute(k_pipe_p3<R5>, cudaFuncAttributePreferredSharedMemoryCarveout, c);
+    // (the vector kernels take the driver's: no more than their windows, since
+    // their loads in flight need the L1)
     cudaGetLastError();
 }
 
@@ -456,23 +384,23 @@ static void apply_carveout(int dot_mode, int c) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return;
     if (dot_mode == RBS_DOT_PLAIN && applied_plain[dev] != c) {
-        prefer_shared<PlainR<1>, PlainR<2>, PlainR<5>>(c);
+        prefer_shared<PlainR<1>, PlainR<2>, PlainR<2>, PlainR<5>>(c);
         applied_plain[dev] = c;
     } else if (dot_mode != RBS_DOT_PLAIN && applied_exact[dev] != c) {
-        prefer_shared<ExactR<1, SQ>, ExactR<2, SQ>, ExactR<5, SQ>>(c);
+        prefer_shared<ExactR<1, SQ>, ExactR<2, SQ>, RowsR2, RowsR5>(c);
         applied_exact[dev] = c;
     }
 }
 
 cudaError_t solver_setup(const SolverArgs &a, int variant, cudaStream_t s, KernelTimer *t) {
     apply_carveout(a.dot_mode, a.carveout);
-    if (a.dot_mode == RBS_DOT_PLAIN) return setup_t<PlainR<1>, PlainR<2>, PlainR<5>>(a, variant, s, t);
-    return setup_t<ExactR<1, SQ>, ExactR<2, SQ>, ExactR<5, SQ>>(a, variant, s, t);
+    if (a.dot_mode == RBS_DOT_PLAIN) return setup_t<PlainR<1>, PlainR<2>, PlainR<2>, PlainR<5>>(a, variant, s, t);
+    return setup_t<ExactR<1, SQ>, ExactR<2, SQ>, RowsR2, RowsR5>(a, variant, s, t);
 }
 
 cudaError_t solver_iteration(const SolverArgs &a, int variant, cudaStream_t s, KernelTimer *t) {
-    if (a.dot_mode == RBS_DOT_PLAIN) return iter_t<PlainR<1>, PlainR<2>, PlainR<5>>(a, variant, s, t);
-    return iter_t<ExactR<1, SQ>, ExactR<2, SQ>, ExactR<5, SQ>>(a, variant, s, t);
+    if (a.dot_mode == RBS_DOT_PLAIN) return iter_t<PlainR<1>, PlainR<2>, PlainR<2>, PlainR<5>>(a, variant, s, t);
+    return iter_t<ExactR<1, SQ>, ExactR<2, SQ>, RowsR2, RowsR5>(a, variant, s, t);
 }
 
 __global__ void k_set_cond(cudaGraphConditionalHandle h, SolverState *st) {
@@ -486,7 +414,7 @@ cudaError_t launch_set_cond(cudaGraphConditionalHandle h, SolverState *st, cudaS
     return cudaGetLastError();
 }
 
-template <class R1, class R2, class R5>
+template <class R1, class R2, class V2, class V5>
 static int blocks_per_sm_t(int variant, int which, int block, int spmv_mode) {
     int nb = 0;
     cudaError_t e = cudaSuccess;
@@ -497,10 +425,11 @@ static int blocks_per_sm_t(int variant, int which, int block, int spmv_mode) {
                            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_cls_k3<R2, CAP>, block, 0);
         });
     } else if (variant == RBS_PIPELINED) {
-        e = which == 2 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pipe_p3<R5>, block, 0)
-                       : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pipe_p1<R2>, block, 0);
+        e = which == 2 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pipe_p3<V5>, block, 0)
+                       : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_pipe_p1<V2>, block, 0);
+        if (which != 2 && V2::WINDOWS && block == 256 && nb > P1_GRID) nb = P1_GRID;
     } else {
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_cls_k4<R2>, block, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_cls_k4<V2>, block, 0);
     }
     if (e != cudaSuccess || nb < 1) nb = 1;
     return nb;
@@ -509,8 +438,8 @@ static int blocks_per_sm_t(int variant, int which, int block, int spmv_mode) {
 int solver_blocks_per_sm(int variant, int dot_mode, int which, int block, int carveout, int spmv_mode) {
     apply_carveout(dot_mode, carveout);
     if (which == 0 && variant == RBS_PIPELINED) return spmv_blocks_per_sm(block, carveout, spmv_mode);
-    if (dot_mode == RBS_DOT_PLAIN) return blocks_per_sm_t<PlainR<1>, PlainR<2>, PlainR<5>>(variant, which, block, spmv_mode);
-    return blocks_per_sm_t<ExactR<1, SQ>, ExactR<2, SQ>, ExactR<5, SQ>>(variant, which, block, spmv_mode);
+    if (dot_mode == RBS_DOT_PLAIN) return blocks_per_sm_t<PlainR<1>, PlainR<2>, PlainR<2>, PlainR<5>>(variant, which, block, spmv_mode);
+    return blocks_per_sm_t<ExactR<1, SQ>, ExactR<2, SQ>, RowsR2, RowsR5>(variant, which, block, spmv_mode);
 }
 
 }  // namespace rbs

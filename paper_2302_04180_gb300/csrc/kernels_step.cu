@@ -28,6 +28,11 @@ __device__ __forceinline__ void seg_pairs(int64_t lo, int64_t hi, F &&f) {
     if (((hi - lo) & 1) && threadIdx.x == 0) f(hi - 1, false);
 }
 
+// The odd last element of a segment (lo is even) in the thread that takes it.
+__device__ __forceinline__ int64_t seg_odd(const StepTask &t) {
+    return (t.hi & 1) && threadIdx.x == 0 ? t.hi - 1 : -1;
+}
+
 // y = A x over the block's segment with the warp-staged SpMV (structure
 // validated at admission), epilogue fn(row, y_row, z_row).
 template <class F>
@@ -183,27 +188,7 @@ __global__ void __launch_bounds__(256, 4) k_step_cls_k4(const Ctx *ctxs, const S
     R red;
     red.init();  // ends in a barrier
     if (sc.copy->done) return;
-    const double al = sc.copy->alpha, om = sc.copy->omega, nom = -om;
-    seg_pairs(t.lo, t.hi, [&](int64_t i, bool pair) {
-        if (pair) {
-            const double2 qh = ld2(c.qh, i), ph = ld2(c.ph, i), y = ld2(c.y, i), q = ld2(c.q, i),
-                          r0 = ld2(c.r0, i), x = ld2(c.x, i);
-            const VPair u0 = cls_k4(al, om, nom, qh.x, ph.x, x.x, y.x, q.x);
-            const VPair u1 = cls_k4(al, om, nom, qh.y, ph.y, x.y, y.y, q.y);
-            st2(c.x, i, make_double2(u0.a, u1.a));
-            st2(c.r, i, make_double2(u0.b, u1.b));
-            red.add(0, r0.x, u0.b);
-            red.add(0, r0.y, u1.b);
-            red.add_sq(1, u0.b);
-            red.add_sq(1, u1.b);
-        } else {
-            const VPair u = cls_k4(al, om, nom, c.qh[i], c.ph[i], c.x[i], c.y[i], c.q[i]);
-            c.x[i] = u.a;
-            c.r[i] = u.b;
-            red.add(0, c.r0[i], u.b);
-            red.add_sq(1, u.b);
-        }
-    });
+    cls_k4_pairs(c, red, sc.copy->alpha, sc.copy->omega, (t.lo >> 1) + threadIdx.x, t.hi >> 1, blockDim.x, seg_odd(t));
     __shared__ double vals[R::K];
     if (red.finish(c.g, vals, t.nblk)) sc.tail([&](SolverState *st) { tail_cls_beta(st, vals, c.hist); });
 }
@@ -281,10 +266,8 @@ __global__ void __launch_bounds__(256, 3) k_step_pipe_p1(const Ctx *ctxs, const 
     R red;
     red.init();  // ends in a barrier
     if (sc.copy->done) return;
-    const double al = sc.copy->alpha, nal = -al, be = sc.copy->beta, nom = -sc.copy->omega;
-    const bool first = sc.copy->iter == 0;
-    for (int64_t i = t.lo + threadIdx.x; i < t.hi; i += blockDim.x)
-        p1_store(c, i, p1_elem(p1_load(c, i, first), first, nal, be, nom, red));
+    pipe_p1_pairs(c, red, sc.copy->iter == 0, -sc.copy->alpha, sc.copy->beta, -sc.copy->omega,
+                  (t.lo >> 1) + threadIdx.x, t.hi >> 1, blockDim.x, seg_odd(t));
     __shared__ double vals[R::K];
     if (red.finish(c.g, vals, t.nblk)) sc.tail([&](SolverState *st) { tail_pipe_omega(st, vals); });
 }
@@ -298,24 +281,13 @@ __global__ void __launch_bounds__(256, 2) k_step_pipe_p3(const Ctx *ctxs, const 
     R red;
     red.init();  // ends in a barrier
     if (sc.copy->done) return;
-    const double al = sc.copy->alpha, nal = -al, om = sc.copy->omega, nom = -om;
-    for (int64_t i = t.lo + threadIdx.x; i < t.hi; i += blockDim.x) {
-        const P3Out o = p3_elem(P3In{c.qh[i], c.y[i], c.q[i], c.ph[i], c.x[i], c.zh[i], c.wh[i], c.v[i], c.t[i],
-                                     c.invd[i], c.r0[i], c.s[i], c.z[i]},
-                                al, nal, om, nom, red);
-        c.x[i] = o.x;
-        c.r[i] = o.r;
-        c.rh[i] = o.rh;
-        c.w[i] = o.w;
-        c.wh[i] = o.wh;
-    }
+    pipe_p3_pairs(c, red, sc.copy->alpha, sc.copy->omega, (t.lo >> 1) + threadIdx.x, t.hi >> 1, blockDim.x, seg_odd(t));
     __shared__ double vals[R::K];
     if (red.finish(c.g, vals, t.nblk)) sc.tail([&](SolverState *st) { tail_pipe_beta(st, vals, c.hist); });
 }
 
 using R1 = ExactR<1, SQ>;
 using R2 = ExactR<2, SQ>;
-using R5 = ExactR<5, SQ>;
 
 void step_carveout() {
     static std::once_flag once;
@@ -378,12 +350,12 @@ cudaError_t step_iteration(const void *ctxs, const StepTask *tasks, int ntasks, 
         k_step_cls_k1<R1><<<ntasks, 256, 0, s>>>(c, tasks);
         k_step_cls_k2<<<ntasks, 256, 0, s>>>(c, tasks);
         k_step_cls_k3<R2><<<ntasks, 256, 0, s>>>(c, tasks);
-        k_step_cls_k4<R2><<<ntasks, 256, 0, s>>>(c, tasks);
+        k_step_cls_k4<RowsR2><<<ntasks, 256, 0, s>>>(c, tasks);
         k_step_cls_k5<<<ntasks, 256, 0, s>>>(c, tasks);
     } else {
-        k_step_pipe_p1<R2><<<ntasks, 256, 0, s>>>(c, tasks);
+        k_step_pipe_p1<RowsR2><<<ntasks, 256, 0, s>>>(c, tasks);
         k_step_spmv<true><<<ntasks, 256, 0, s>>>(c, tasks);
-        k_step_pipe_p3<R5><<<ntasks, 256, 0, s>>>(c, tasks);
+        k_step_pipe_p3<RowsR5><<<ntasks, 256, 0, s>>>(c, tasks);
         k_step_spmv<false><<<ntasks, 256, 0, s>>>(c, tasks);
     }
     return cudaGetLastError();

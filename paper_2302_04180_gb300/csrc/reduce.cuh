@@ -48,14 +48,24 @@ struct ExactR {
     }
 };
 
-// Exact reducer of the standalone dots: per-thread windows in shared memory, W
-// 32-bit words per sign (positive and negative products kept apart, so a
-// product's five words are added to five words picked by address -- no word
-// selects, no two's complement) as one add-with-carry chain. A carry out of the
-// chain needs the sixth word to be all ones up to the product's top few bits,
-// so the ripple that continues it is a branch almost never taken. Layout
-// [sign][word][thread]: a thread's words share one bank, whatever their
-// placement, so every access is conflict-free.
+// Exact reducer with its per-thread windows in shared memory (the standalone dots
+// and the vector kernels): per dot W 32-bit words; a product's five words are
+// added to the five words at its placement, picked by address with no word
+// selects, as one add-with-carry chain. Layout [dot, sign, word][thread]: a
+// thread's words share one bank, whatever their placement, so every access is
+// conflict-free.
+//
+// SPLIT: W words per sign, positive and negative products kept apart (the
+// standalone dots: fewest instructions). Without it one set of words takes both,
+// a negative product as its complement with 1 carried in; the words start at
+// 2^31 and the flush takes that out again, so that a borrow, like a carry, leaves
+// the five words only when the fifth is within the product's top few bits of its
+// end: the ripple that continues it is a branch almost never taken. (Half the
+// shared memory: what the vector kernels' windows take comes out of the L1 that
+// their loads in flight need, and the registers that windows would take otherwise
+// cost more still. K4 at 256^3: 191 us with register windows, whose products
+// below the window go to atomics while the values still fall off steeply, 207
+// with 47 KB of windows a block, 162 with 35; HBM alone 158.)
 //
 // What bounds it: at the HBM rate an SM has 0.72 cycles per element pair. The
 // window update used to be five 64-bit carry-save digits, whose loads and
@@ -64,41 +74,47 @@ struct ExactR {
 // 64 bits bring a product to 62 instructions from 90 (2^24 products, cond 1e48:
 // 54 us from 73).
 //
-// The window covers W - 4 placements. All threads of a block start with one
+// A window covers W - 4 placements. All threads of a block start with one
 // anchor (open()): the block's largest first product lands at placement ANCHOR,
-// which leaves up to three placements (96 bits) above it. A product above the window
-// flushes and re-anchors its thread's own; one below goes straight into the
-// block accumulator. While a warp's anchors agree (they differ only after a
+// which leaves up to three placements (96 bits) above it. A product above the
+// window flushes and re-anchors its thread's own; one below goes straight into
+// the block accumulator. While a warp's anchors agree (they differ only after a
 // product above the window) the flush at the end sums each word over the warp
 // with one lane per word.
-template <int W_>
-struct ExactW {
+template <int K_, int W_, bool SPLIT>
+struct ExactRows {
+    static constexpr int K = K_;
     static constexpr int W = W_;
-    static constexpr int QMAX = W - 5;             // highest placement of a product's lowest word
+    static constexpr bool WINDOWS = true;  // open() before the first add
+    static constexpr int QMAX = W - 5;  // highest placement of a product's lowest word
     // placement of the product that (re)anchors the window: up to three above it
     static constexpr int ANCHOR = QMAX - (QMAX + 2) / 4;
-    static constexpr int NT = 256;                 // most threads per block (column stride)
-    static_assert(2 * W <= 32, "the warp flush gives each word of each sign a lane");
-    uint32_t *win;  // this thread's column: word j of sign s at win[(s * W + j) * NT]
-    int a;          // anchor limb, WIN_EMPTY when there is no window yet
+    static constexpr int NT = 256;  // most threads per block (column stride)
+    static constexpr int PER = SPLIT ? 2 * W : W, ROWS = K * PER;
+    static_assert(PER <= 32, "the warp flush gives each word a lane");
+    static constexpr uint32_t ZERO = SPLIT ? 0u : 0x80000000u;  // a word that holds nothing
+    static_assert(ROWS <= 255, "placements in bytes, the zero products' included");
+    uint32_t *win;  // this thread's column: word j of sign s of dot k at win[(k * PER + s * W + j) * NT]
+    int a[K];       // anchor limbs, WIN_EMPTY when there is no window yet
     unsigned long long (*sacc)[NL];
     uint32_t *sflags;
     int *amax;
 
     __device__ __forceinline__ void init() {
-        __shared__ uint32_t s_win[(2 * W + 5) * NT];  // the last five rows take zero products
-        __shared__ unsigned long long s_acc[1][NL];
-        __shared__ uint32_t s_flags[1];
-        __shared__ int s_amax;
+        __shared__ uint32_t s_win[(ROWS + 5) * NT];  // the last five rows take zero products
+        __shared__ unsigned long long s_acc[K][NL];
+        __shared__ uint32_t s_flags[K];
+        __shared__ int s_amax[K];
         win = s_win + threadIdx.x;
         sacc = s_acc;
         sflags = s_flags;
-        amax = &s_amax;
-        a = WIN_EMPTY;
+        amax = s_amax;
 #pragma unroll
-        for (int j = 0; j < 2 * W; j++) win[j * NT] = 0u;
-        if (threadIdx.x == 0) s_amax = -1;
-        sacc_zero<1>(sacc, sflags);
+        for (int k = 0; k < K; k++) a[k] = WIN_EMPTY;
+#pragma unroll
+        for (int j = 0; j < ROWS; j++) win[j * NT] = ZERO;
+        if (threadIdx.x < K) s_amax[threadIdx.x] = -1;
+        sacc_zero<K>(sacc, sflags);
     }
     // The limb of x*y's lowest bit, for the common start anchor (-1: no finite nonzero normal product).
     static __device__ __forceinline__ int limb_of(double x, double y) {
@@ -106,33 +122,38 @@ struct ExactW {
         if (ex - 0x00100000u >= 0x7fe00000u || ey - 0x00100000u >= 0x7fe00000u) return -1;
         return (int)((ex + ey - (2u << 20)) >> 25);
     }
-    // The common start anchor from every thread's first products (their highest
+    // The common start anchors from every thread's first products (their highest
     // limb, -1 for none). All threads call it, before the first add.
-    __device__ __forceinline__ void open(int limb) {
-        const int m = __reduce_max_sync(0xffffffffu, limb);
-        if ((threadIdx.x & 31) == 0) atomicMax(amax, m);
+    __device__ __forceinline__ void open(const int (&limb)[K]) {
+#pragma unroll
+        for (int k = 0; k < K; k++) {
+            const int m = __reduce_max_sync(0xffffffffu, limb[k]);
+            if ((threadIdx.x & 31) == 0) atomicMax(&amax[k], m);
+        }
         __syncthreads();
-        if (*amax >= 0) a = max(*amax - ANCHOR, 0);
+#pragma unroll
+        for (int k = 0; k < K; k++)
+            if (amax[k] >= 0) a[k] = max(amax[k] - ANCHOR, 0);
     }
-    // One thread's window (column w, anchor a) into the block
-    // accumulator sk, with its own atomics; words back to zero.
+    // One thread's window (column w, anchor a) into the block accumulator sk, with
+    // its own atomics; words back to nothing.
     static __device__ __forceinline__ void flush_column(uint32_t *w, unsigned long long *sk, int a) {
         for (int j = 0; j < W; j++) {
-            const long long d = (long long)w[j * NT] - (long long)w[(W + j) * NT];
-            w[j * NT] = 0u;
-            w[(W + j) * NT] = 0u;
+            const long long d = (long long)w[j * NT] - (SPLIT ? (long long)w[(W + j) * NT] : (long long)ZERO);
+            w[j * NT] = ZERO;
+            if (SPLIT) w[(W + j) * NT] = ZERO;
             if (d) sacc_add(&sk[a + j], d);
         }
     }
-    // +1 to word j of a sign's words p (a carry), or past the window's top into
-    // the block accumulator.
-    static __device__ __forceinline__ void ripple(uint32_t *p, unsigned long long *sk, int a, int j, bool neg) {
+    // A carry (or, with down, a borrow) into word j of a set of words p, or past
+    // the window's top into the block accumulator (neg: of the negative words).
+    static __device__ __forceinline__ void ripple(uint32_t *p, unsigned long long *sk, int a, int j, bool down, bool neg) {
         for (; j < W; j++) {
-            const uint32_t v = p[j * NT] + 1u;
-            p[j * NT] = v;
-            if (v) return;
+            const uint32_t v = p[j * NT];
+            p[j * NT] = down ? v - 1u : v + 1u;
+            if (v != (down ? 0u : 0xffffffffu)) return;
         }
-        if (a + W < NL) sacc_add(&sk[a + W], neg ? -1ll : 1ll);
+        if (a + W < NL) sacc_add(&sk[a + W], down || neg ? -1ll : 1ll);
     }
     // Products of any kind: zeros, subnormals and non-finite operands, products in
     // the window, below it (into the block accumulator) and above it (flush and
@@ -156,36 +177,36 @@ struct ExactW {
                 if (a >= 0) flush_column(w, sk, a);
                 a = L > ANCHOR ? L - ANCHOR : 0;
             }
-            uint32_t *p = w + (m ? W * NT : 0);
-            unsigned long long t = 0;
+            uint32_t *p = w + (SPLIT && m ? W * NT : 0);
+            const uint32_t inv = SPLIT ? 0u : m;
+            unsigned long long t = inv & 1u;
             for (int j = 0; j < 5; j++) {
-                t += (unsigned long long)p[(L - a + j) * NT] + u[j];
+                t += (unsigned long long)p[(L - a + j) * NT] + (u[j] ^ inv);
                 p[(L - a + j) * NT] = (uint32_t)t;
                 t >>= 32;
             }
-            if (t) ripple(p, sk, a, L - a + 5, m != 0u);
+            if ((uint32_t)t != (inv & 1u)) ripple(p, sk, a, L - a + 5, inv != 0u, m != 0u);
         }
         return a;
     }
-    // The carries out of the five words of add()'s products (rare): bit i of
-    // `carries` for product i, its sign at bit 16 + i, its placement in byte i
-    // of qs (at most four products).
-    static __device__ __noinline__ void carries_out(uint32_t *w, unsigned long long *sk, int a, uint32_t carries,
-                                                    uint32_t qs) {
+    // The carries and borrows out of the five words of add()'s products (rare):
+    // bit i of `out` for product i, its sign at bit 16 + i, its placement in byte
+    // i of qs (at most four products).
+    static __device__ __noinline__ void ripples(uint32_t *w, unsigned long long *sk, int a, uint32_t out, uint32_t qs) {
         for (int i = 0; i < 4; i++) {
             const int q = (int)(qs >> 8 * i) & 255;
-            const bool neg = ((carries >> (16 + i)) & 1u) != 0u;
-            if (((carries >> i) & 1u) && q <= QMAX) ripple(w + (neg ? W * NT : 0), sk, a, q + 5, neg);
+            const bool neg = ((out >> (16 + i)) & 1u) != 0u;
+            if (((out >> i) & 1u) && q <= QMAX) ripple(w + (SPLIT && neg ? W * NT : 0), sk, a, q + 5, !SPLIT && neg, neg);
         }
     }
-    static_assert(2 * W <= 255, "placements in bytes, the zero products' included");
-    // N products into the window. One branch for all of them: when every operand
+    // N products into window k. One branch for all of them: when every operand
     // is normal and every product lands in the window (nearly always), straight
     // code. Otherwise zero products are sent to five words that nobody reads, and
     // any other kind sends all N through add_any(). N is 1, 2 or 4.
-    template <int N>
-    __device__ __forceinline__ void add(const double (&x)[N], const double (&y)[N]) {
+    template <int N, bool SQ = false>
+    __device__ __forceinline__ void add(int k, const double (&x)[N], const double (&y)[N]) {
         uint32_t xh[N], yh[N], e[N], q[N], odd = 0u, far = 0u;
+        uint32_t *wk = win + k * PER * NT;
 #pragma unroll
         for (int i = 0; i < N; i++) {
             xh[i] = (uint32_t)__double2hiint(x[i]);
@@ -193,19 +214,19 @@ struct ExactW {
             const uint32_t ex = xh[i] & 0x7ff00000u, ey = yh[i] & 0x7ff00000u;
             odd = max(max(odd, ex - 0x00100000u), ey - 0x00100000u);
             e[i] = ex + ey - (2u << 20);  // bit position << 20; garbage for an odd operand
-            q[i] = (e[i] >> 25) - (uint32_t)a;
+            q[i] = (e[i] >> 25) - (uint32_t)a[k];
             far = max(far, q[i]);
         }
         bool go = true;
         if (!(odd < 0x7fe00000u && far <= (uint32_t)QMAX)) {
-            go = a >= 0;
+            go = a[k] >= 0;
 #pragma unroll
             for (int i = 0; i < N; i++) {
                 const uint32_t ex = xh[i] & 0x7ff00000u, ey = yh[i] & 0x7ff00000u;
                 const uint32_t zx = (xh[i] & 0x7fffffffu) | (uint32_t)__double2loint(x[i]);
                 const uint32_t zy = (yh[i] & 0x7fffffffu) | (uint32_t)__double2loint(y[i]);
                 if (min(zx, zy) == 0u && max(ex, ey) < 0x7ff00000u) {
-                    q[i] = (uint32_t)(2 * W);
+                    q[i] = (uint32_t)(ROWS - k * PER);
                     xh[i] = yh[i];
                 } else {
                     go = go && max(ex - 0x00100000u, ey - 0x00100000u) < 0x7fe00000u && q[i] <= (uint32_t)QMAX;
@@ -213,15 +234,15 @@ struct ExactW {
             }
             if (!go) {
                 if constexpr (N == 1)
-                    a = add_any(win, sacc[0], sflags, a, x[0], y[0]);
+                    a[k] = add_any(wk, sacc[k], &sflags[k], a[k], x[0], y[0]);
                 else if constexpr (N == 2)
-                    a = add_any(win, sacc[0], sflags, a, x[0], y[0], x[1], y[1]);
+                    a[k] = add_any(wk, sacc[k], &sflags[k], a[k], x[0], y[0], x[1], y[1]);
                 else
-                    a = add_any(win, sacc[0], sflags, a, x[0], y[0], x[1], y[1], x[2], y[2], x[3], y[3]);
+                    a[k] = add_any(wk, sacc[k], &sflags[k], a[k], x[0], y[0], x[1], y[1], x[2], y[2], x[3], y[3]);
             }
         }
         if (go) {
-            uint32_t carries = 0u;
+            uint32_t out = 0u;
 #pragma unroll
             for (int i = 0; i < N; i++) {
                 const uint32_t xl = (uint32_t)__double2loint(x[i]), yl = (uint32_t)__double2loint(y[i]);
@@ -229,86 +250,124 @@ struct ExactW {
                 // 106-bit significand product: the two middle terms share one 64-bit sum (< 2^54)
                 const unsigned long long lo = (unsigned long long)xl * yl, hi = (unsigned long long)A1 * B1;
                 const unsigned long long mid = (unsigned long long)xl * B1 + (unsigned long long)A1 * yl;
-                uint32_t p1, p2, p3, u[5], c;
+                uint32_t p0 = (uint32_t)lo, p1, p2, p3, u[5], c;
                 asm("add.cc.u32 %0, %3, %4;\n\t"
                     "addc.cc.u32 %1, %5, %6;\n\t"
                     "addc.u32 %2, %7, 0;"
                     : "=&r"(p1), "=&r"(p2), "=r"(p3)
                     : "r"((uint32_t)(lo >> 32)), "r"((uint32_t)mid), "r"((uint32_t)hi), "r"((uint32_t)(mid >> 32)),
                       "r"((uint32_t)(hi >> 32)));
+                // complement of a negative product (before the shift, which fills with it)
+                const uint32_t m = SPLIT || SQ ? 0u : (uint32_t)((int32_t)(xh[i] ^ yh[i]) >> 31);
+                if (!SPLIT && !SQ) {
+                    p0 ^= m;
+                    p1 ^= m;
+                    p2 ^= m;
+                    p3 ^= m;
+                }
                 const uint32_t r = e[i] >> 20;  // the funnel shifts take it modulo 32
-                u[0] = __funnelshift_l(0u, (uint32_t)lo, r);
-                u[1] = __funnelshift_l((uint32_t)lo, p1, r);
+                u[0] = __funnelshift_l(m, p0, r);
+                u[1] = __funnelshift_l(p0, p1, r);
                 u[2] = __funnelshift_l(p1, p2, r);
                 u[3] = __funnelshift_l(p2, p3, r);
-                u[4] = __funnelshift_l(p3, 0u, r);
-                uint32_t *p = win + q[i] * NT + ((xh[i] ^ yh[i]) >> 31) * (W * NT);
+                u[4] = __funnelshift_l(p3, m, r);
+                uint32_t *p = wk + q[i] * NT + (SPLIT && !SQ ? ((xh[i] ^ yh[i]) >> 31) * (W * NT) : 0u);
                 uint32_t w0 = p[0], w1 = p[NT], w2 = p[2 * NT], w3 = p[3 * NT], w4 = p[4 * NT];
-                asm("add.cc.u32 %0, %0, %6;\n\t"
-                    "addc.cc.u32 %1, %1, %7;\n\t"
-                    "addc.cc.u32 %2, %2, %8;\n\t"
-                    "addc.cc.u32 %3, %3, %9;\n\t"
-                    "addc.cc.u32 %4, %4, %10;\n\t"
-                    "addc.u32 %5, 0, 0;"
-                    : "+r"(w0), "+r"(w1), "+r"(w2), "+r"(w3), "+r"(w4), "=r"(c)
-                    : "r"(u[0]), "r"(u[1]), "r"(u[2]), "r"(u[3]), "r"(u[4]));
+                if (SPLIT || SQ) {
+                    asm("add.cc.u32 %0, %0, %6;\n\t"
+                        "addc.cc.u32 %1, %1, %7;\n\t"
+                        "addc.cc.u32 %2, %2, %8;\n\t"
+                        "addc.cc.u32 %3, %3, %9;\n\t"
+                        "addc.cc.u32 %4, %4, %10;\n\t"
+                        "addc.u32 %5, 0, 0;"
+                        : "+r"(w0), "+r"(w1), "+r"(w2), "+r"(w3), "+r"(w4), "=r"(c)
+                        : "r"(u[0]), "r"(u[1]), "r"(u[2]), "r"(u[3]), "r"(u[4]));
+                } else {
+                    // 1 carried in with a complement; out: 1 if a carry (positive) or a
+                    // borrow (negative: no carry) leaves the five words
+                    asm("{\n\t.reg .u32 t;\n\t"
+                        "add.cc.u32 t, %11, %11;\n\t"
+                        "addc.cc.u32 %0, %0, %6;\n\t"
+                        "addc.cc.u32 %1, %1, %7;\n\t"
+                        "addc.cc.u32 %2, %2, %8;\n\t"
+                        "addc.cc.u32 %3, %3, %9;\n\t"
+                        "addc.cc.u32 %4, %4, %10;\n\t"
+                        "addc.u32 %5, %11, 0;\n\t}"
+                        : "+r"(w0), "+r"(w1), "+r"(w2), "+r"(w3), "+r"(w4), "=&r"(c)
+                        : "r"(u[0]), "r"(u[1]), "r"(u[2]), "r"(u[3]), "r"(u[4]), "r"(m));
+                    // m + carry: 0 or 1 for a positive product, -1 (borrow) or 0 for a negative one
+                    c &= 1u;
+                }
                 p[0] = w0;
                 p[NT] = w1;
                 p[2 * NT] = w2;
                 p[3 * NT] = w3;
                 p[4 * NT] = w4;
-                carries += c << i;
+                out += c << i;
             }
-            if (carries) {
+            if (out) {
                 uint32_t qs = 0u;
 #pragma unroll
                 for (int i = 0; i < N; i++) {
                     qs |= q[i] << 8 * i;
-                    carries |= ((xh[i] ^ yh[i]) >> 31) << (16 + i);
+                    out |= (SQ ? 0u : (xh[i] ^ yh[i]) >> 31) << (16 + i);
                 }
-                carries_out(win, sacc[0], a, carries, qs);
+                ripples(wk, sacc[k], a[k], out, qs);
             }
         }
     }
-    __device__ __forceinline__ void add_one(double x, double y) {
-        const double xv[1] = {x}, yv[1] = {y};
-        add<1>(xv, yv);
+    template <int N>
+    __device__ __forceinline__ void add_sq(int k, const double (&x)[N]) {
+        add<N, true>(k, x, x);
     }
-    // Flush of every lane's window at the end of the kernel (all 32 lanes call
-    // it). With one anchor in the warp, lane r sums word r of the W positive and
-    // W negative words over the warp's columns, each lane starting at its own
-    // column (32 banks, no conflicts); else every lane flushes its own.
-    __device__ __forceinline__ void flush_warp() {
+    __device__ __forceinline__ void add(int k, double x, double y) {
+        const double xv[1] = {x}, yv[1] = {y};
+        add<1>(k, xv, yv);
+    }
+    __device__ __forceinline__ void add_sq(int k, double x) {
+        const double xv[1] = {x};
+        add_sq<1>(k, xv);
+    }
+    // Flush of every lane's window k at the end of the kernel (all 32 lanes call
+    // it). With one anchor in the warp, lane r sums word r over the warp's
+    // columns, each lane starting at its own column (32 banks, no conflicts); else
+    // every lane flushes its own.
+    __device__ __forceinline__ void flush_warp(int k) {
         constexpr unsigned FULL = 0xffffffffu;
         const int lane = threadIdx.x & 31;
-        const int a0 = __shfl_sync(FULL, a, 0);
-        if (!__all_sync(FULL, a == a0)) {
-            if (a >= 0) flush_column(win, sacc[0], a);
+        const int a0 = __shfl_sync(FULL, a[k], 0);
+        uint32_t *wk = win + k * PER * NT;
+        if (!__all_sync(FULL, a[k] == a0)) {
+            if (a[k] >= 0) flush_column(wk, sacc[k], a[k]);
             return;
         }
         if (a0 < 0) return;
         __syncwarp();
-        long long sum = 0;
-        if (lane < 2 * W) {
-            const uint32_t *row = win - lane + lane * NT;
+        long long sum = SPLIT ? 0 : -32ll * ZERO;
+        if (lane < PER) {
+            const uint32_t *r = wk - lane + lane * NT;
 #pragma unroll 8
-            for (int i = 0; i < 32; i++) sum += (long long)row[(i + lane) & 31];
+            for (int i = 0; i < 32; i++) sum += (long long)r[(i + lane) & 31];
         }
-        sum -= __shfl_down_sync(FULL, sum, W);
-        if (lane < W && sum && a0 + lane < NL) sacc_add(&sacc[0][a0 + lane], sum);
+        if (SPLIT) sum -= __shfl_down_sync(FULL, sum, W);
+        if (lane < W && sum && a0 + lane < NL) sacc_add(&sacc[k][a0 + lane], sum);
     }
-    // Reduction `slot` of g, over gridDim.x blocks (block_grid_finish).
-    __device__ __forceinline__ bool finish(DotScratch *g, int slot, double *val, bool export_limbs = false,
-                                           long long *limbs = nullptr, int32_t *fl = nullptr) {
-        flush_warp();
-        const uint32_t none[1] = {0u};  // add_any() has set the block's flags itself
-        return block_grid_finish<1>(none, sacc, sflags, g, val, export_limbs, limbs, fl, gridDim.x, slot);
+    // The K reductions from `slot` of g on, over nblk blocks (0: the grid); see
+    // block_grid_finish.
+    __device__ __forceinline__ bool finish(DotScratch *g, double *vals, unsigned nblk = 0u, int slot = 0,
+                                           bool export_limbs = false, long long *limbs = nullptr,
+                                           int32_t *fl = nullptr) {
+#pragma unroll
+        for (int k = 0; k < K; k++) flush_warp(k);
+        const uint32_t none[K] = {};  // add_any() has set the block's flags itself
+        return block_grid_finish<K>(none, sacc, sflags, g, vals, export_limbs, limbs, fl, nblk, slot);
     }
 };
 
 template <int K_>
 struct PlainR {
     static constexpr int K = K_;
+    static constexpr bool WINDOWS = false;
     double s[K];
 
     __device__ __forceinline__ void init() {
@@ -318,6 +377,18 @@ struct PlainR {
     }
     __device__ __forceinline__ void add(int k, double x, double y) { s[k] = fma(x, y, s[k]); }
     __device__ __forceinline__ void add_sq(int k, double x) { s[k] = fma(x, x, s[k]); }
+    template <int N>
+    __device__ __forceinline__ void add(int k, const double (&x)[N], const double (&y)[N]) {
+#pragma unroll
+        for (int i = 0; i < N; i++) add(k, x[i], y[i]);
+    }
+    template <int N>
+    __device__ __forceinline__ void add_sq(int k, const double (&x)[N]) {
+#pragma unroll
+        for (int i = 0; i < N; i++) add_sq(k, x[i]);
+    }
+    static __device__ __forceinline__ int limb_of(double, double) { return -1; }
+    __device__ __forceinline__ void open(const int (&)[K]) {}
     template <int SCRATCH = 0, int WARPS = MAX_WARPS>
     __device__ __forceinline__ bool finish(DotScratch *g, double *vals, unsigned nblk = 0u, bool coop = true) {
         (void)coop;  // its partials live in their own shared array
