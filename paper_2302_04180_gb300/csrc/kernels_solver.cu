@@ -403,6 +403,7 @@ cudaError_t solver_iteration(const SolverArgs &a, int variant, cudaStream_t s, K
     return iter_t<ExactR<1, SQ>, ExactR<2, SQ>, RowsR2, RowsR5>(a, variant, s, t);
 }
 
+// (a body holds one iteration or more, so maxit + 1 bodies are enough)
 __global__ void k_set_cond(cudaGraphConditionalHandle h, SolverState *st) {
     const int loops = st->loops + 1;
     st->loops = loops;
