@@ -51,9 +51,8 @@ __global__ void __launch_bounds__(256) k_cls_setup(Ctx c) {
 // SpMV rows of the fused K1/K3 with epilogue fn(row, y_row, z_row), by CAP:
 // matrices of few diagonals (CAP = -N, spmv_rows_diag); short rows warp-staged
 // (or one thread per row, mode 1) in 256-thread blocks; long rows (CAP =
-// SPMV_CAP_LONG) register-staged in blocks of SPMV_REG_WARPS warps. Finish the
-// kernel's reducer with finish<FusedScratch<CAP>::BYTES, FusedScratch<CAP>::WARPS>,
-// so that its flush reuses the staging buffer.
+// SPMV_CAP_LONG) register-staged in blocks of SPMV_REG_WARPS warps. finish_fused
+// lets the flush of register windows reuse the staging buffer.
 constexpr int CAP_DIAG7 = -7, CAP_DIAG32 = -32;
 template <int CAP>
 struct FusedScratch {
@@ -70,6 +69,29 @@ struct FusedDiag {
 };
 template <> struct FusedScratch<CAP_DIAG7> : FusedDiag<7> {};
 template <> struct FusedScratch<CAP_DIAG32> : FusedDiag<32> {};
+// The reducer R as K1, K3 and the pipelined set-up carry it: the kernels of few
+// diagonals, whose smaller staging leaves the shared memory, keep the exact
+// windows there (256^3, first hundred iterations: K3 320 -> 275 us, K1 249 -> 244;
+// 283 with 10 words and 314 with 8, since products below the window go to
+// atomics while the vectors fall off steeply).
+template <class R, int CAP>
+struct FusedDot {
+    using type = R;
+};
+template <int K>
+struct FusedDot<ExactR<K, SQ>, CAP_DIAG7> {
+    using type = ExactRows<K, 12, false>;
+};
+// finish() of either; coop = false after a timed-out staged copy
+template <int CAP, class R>
+__device__ __forceinline__ bool finish_fused(R &red, DotScratch *g, double *vals, bool coop) {
+    return red.template finish<FusedScratch<CAP>::BYTES, FusedScratch<CAP>::WARPS>(g, vals, 0u, coop);
+}
+template <int CAP, int K, int W>
+__device__ __forceinline__ bool finish_fused(ExactRows<K, W, false> &red, DotScratch *g, double *vals, bool) {
+    return red.finish(g, vals);
+}
+
 template <int CAP, class F>
 __device__ __forceinline__ void fused_spmv(const Ctx &c, const double *x, const double *z, unsigned &eb, F &&fn) {
     if constexpr (CAP < 0)
@@ -87,7 +109,7 @@ template <class R, int CAP>
 __global__ void __launch_bounds__(FusedScratch<CAP>::THREADS, 3) k_cls_k1(Ctx c) {
     StateCopy sc;
     sc.load(c.st);
-    R red;
+    typename FusedDot<R, CAP>::type red;
     red.init();  // ends in a barrier
     if (sc.copy->done) return;
     unsigned eb = 0u;
@@ -97,8 +119,7 @@ __global__ void __launch_bounds__(FusedScratch<CAP>::THREADS, 3) k_cls_k1(Ctx c)
     });
     if (eb) atomicOr(c.err, eb);
     __shared__ double vals[R::K];
-    if (red.template finish<FusedScratch<CAP>::BYTES, FusedScratch<CAP>::WARPS>(c.g, vals, 0u,
-                                                                               !(eb & ERR_TIMEOUT)))
+    if (finish_fused<CAP>(red, c.g, vals, !(eb & ERR_TIMEOUT)))
         sc.tail([&](SolverState *st) { tail_cls_alpha(st, vals); });
 }
 
@@ -127,7 +148,7 @@ template <class R, int CAP>
 __global__ void __launch_bounds__(FusedScratch<CAP>::THREADS, 3) k_cls_k3(Ctx c) {
     StateCopy sc;
     sc.load(c.st);
-    R red;
+    typename FusedDot<R, CAP>::type red;
     red.init();  // ends in a barrier
     if (sc.copy->done) return;
     unsigned eb = 0u;
@@ -138,8 +159,7 @@ __global__ void __launch_bounds__(FusedScratch<CAP>::THREADS, 3) k_cls_k3(Ctx c)
     });
     if (eb) atomicOr(c.err, eb);
     __shared__ double vals[R::K];
-    if (red.template finish<FusedScratch<CAP>::BYTES, FusedScratch<CAP>::WARPS>(c.g, vals, 0u,
-                                                                               !(eb & ERR_TIMEOUT)))
+    if (finish_fused<CAP>(red, c.g, vals, !(eb & ERR_TIMEOUT)))
         sc.tail([&](SolverState *st) { tail_cls_omega(st, vals); });
 }
 
@@ -189,7 +209,7 @@ template <class R, int CAP>
 __global__ void __launch_bounds__(FusedScratch<CAP>::THREADS, 3) k_pipe_setup2(Ctx c) {
     StateCopy sc;
     sc.load(c.st);
-    R red;
+    typename FusedDot<R, CAP>::type red;
     red.init();  // ends in a barrier
     unsigned eb = 0u;
     fused_spmv<CAP>(c, c.rh, c.r0, eb, [&](int64_t i, double wi, double r0) {
@@ -200,8 +220,7 @@ __global__ void __launch_bounds__(FusedScratch<CAP>::THREADS, 3) k_pipe_setup2(C
     });
     if (eb) atomicOr(c.err, eb);
     __shared__ double vals[R::K];
-    if (red.template finish<FusedScratch<CAP>::BYTES, FusedScratch<CAP>::WARPS>(c.g, vals, 0u,
-                                                                               !(eb & ERR_TIMEOUT)))
+    if (finish_fused<CAP>(red, c.g, vals, !(eb & ERR_TIMEOUT)))
         sc.tail([&](SolverState *st) { tail_pipe_setup(st, vals); });
 }
 

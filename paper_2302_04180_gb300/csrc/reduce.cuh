@@ -74,13 +74,15 @@ struct ExactR {
 // 64 bits bring a product to 62 instructions from 90 (2^24 products, cond 1e48:
 // 54 us from 73).
 //
-// A window covers W - 4 placements. All threads of a block start with one
-// anchor (open()): the block's largest first product lands at placement ANCHOR,
-// which leaves up to three placements (96 bits) above it. A product above the
-// window flushes and re-anchors its thread's own; one below goes straight into
-// the block accumulator. While a warp's anchors agree (they differ only after a
-// product above the window) the flush at the end sums each word over the warp
-// with one lane per word.
+// A window covers W - 4 placements. Where a kernel has every thread's first
+// products before it adds any, all threads of a block start with one anchor
+// (open()): the block's largest first product lands at placement ANCHOR, which
+// leaves up to three placements (96 bits) above it. Elsewhere a thread's first
+// product opens its window, lanes that do so together with one anchor where their
+// products all fit (a call and a divergent branch per thread: 1.5 us on a short
+// dot). A product above the window flushes and re-anchors its thread's own; one
+// below goes straight into the block accumulator. While a warp's anchors agree
+// the flush at the end sums each word over the warp with one lane per word.
 template <int K_, int W_, bool SPLIT>
 struct ExactRows {
     static constexpr int K = K_;
@@ -174,8 +176,14 @@ struct ExactRows {
                 continue;
             }
             if (L - a > QMAX) {
-                if (a >= 0) flush_column(w, sk, a);
-                a = L > ANCHOR ? L - ANCHOR : 0;
+                int top = L;
+                if (a >= 0) {
+                    flush_column(w, sk, a);
+                } else {
+                    const int m = (int)__reduce_max_sync(__activemask(), (unsigned)L);
+                    if (m - L <= ANCHOR) top = m;
+                }
+                a = top > ANCHOR ? top - ANCHOR : 0;
             }
             uint32_t *p = w + (SPLIT && m ? W * NT : 0);
             const uint32_t inv = SPLIT ? 0u : m;
@@ -219,7 +227,6 @@ struct ExactRows {
         }
         bool go = true;
         if (!(odd < 0x7fe00000u && far <= (uint32_t)QMAX)) {
-            go = a[k] >= 0;
 #pragma unroll
             for (int i = 0; i < N; i++) {
                 const uint32_t ex = xh[i] & 0x7ff00000u, ey = yh[i] & 0x7ff00000u;
