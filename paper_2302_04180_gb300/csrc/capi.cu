@@ -123,7 +123,7 @@ struct Workspace {
     BatchOut *h_small = nullptr;
     Buf vec, hist, diag, stage[8];
     Buf batch_work, batch_hist, batch_sys, batch_order, batch_out, batch_queue;
-    Buf step_ctx, step_state, step_scr, step_tasks;  // the stepped batch schedule
+    Buf step_ctx, step_state, step_scr, step_tasks, step_diag;  // the stepped batch schedule
     std::vector<cudaEvent_t> evpool;
     std::vector<cudaEvent_t> ev_chunk;
     // graph loop: one iteration captured as the body of a conditional WHILE node
@@ -199,7 +199,7 @@ void ws_free(Workspace *w) {
     cudaFree(w->diag.p);
     cudaFree(w->hist.p);
     for (Buf *b : {&w->batch_work, &w->batch_hist, &w->batch_sys, &w->batch_order, &w->batch_out,
-                   &w->batch_queue, &w->step_ctx, &w->step_state, &w->step_scr, &w->step_tasks})
+                   &w->batch_queue, &w->step_ctx, &w->step_state, &w->step_scr, &w->step_tasks, &w->step_diag})
         cudaFree(b->p);
     for (auto &b : w->stage) cudaFree(b.p);
     for (auto e : w->evpool) cudaEventDestroy(e);
@@ -939,7 +939,14 @@ int batch_stepped(Workspace *w, int32_t nsys, const rbs_system *systems, rbs_inf
     };
     std::vector<char> valid((size_t)nsys, 1);
     std::vector<int32_t> maxit((size_t)nsys, 0);
-    size_t work_elems = 0, hist_recs = 0;
+    size_t work_elems = 0, hist_recs = 0, layout_bytes = 0;
+    // room for a system's layout by diagonals: one word per row, one int64 per 32
+    auto layout_of = [&](const rbs_system &S) -> size_t {
+        const CSRArgs A{S.A.n, S.A.nnz, S.A.rowptr, S.A.col, S.A.val};
+        if (p_spmv_mode.load() != 0 || !step_wants_layout(A)) return 0;
+        const size_t chunks = (size_t)(S.A.n + 31) / 32;
+        return chunks * (32 * sizeof(uint32_t) + sizeof(int64_t));
+    };
     for (int i = 0; i < nsys; i++) {
         const rbs_system &S = systems[i];
         memset(&infos[i], 0, sizeof infos[i]);
@@ -956,12 +963,14 @@ int batch_stepped(Workspace *w, int32_t nsys, const rbs_system *systems, rbs_inf
         maxit[(size_t)i] = proxy ? std::min(S.maxit, std::max(proxy_maxit[i], 1)) : S.maxit;
         const int64_t stride = (S.A.n + 31) / 32 * 32;
         work_elems += (size_t)stride * ((S.variant == RBS_PIPELINED ? 16 : 9) + (proxy ? 1 : 0));
+        layout_bytes += layout_of(S);
         const int cap = hists ? std::min(hists[i].cap, S.maxit) : 0;
         hist_recs += (size_t)(cap > 0 ? cap : 0);
     }
     const size_t cb = step_ctx_bytes();
     CK(ensure(w->batch_work, work_elems * 8));
     CK(ensure(w->batch_hist, (hist_recs > 0 ? hist_recs : 1) * RBS_HIST_W * 8));
+    CK(ensure(w->step_diag, layout_bytes));
     CK(ensure(w->step_ctx, (size_t)nsys * cb));
     CK(ensure(w->step_state, (size_t)nsys * sizeof(SolverState)));
     CK(ensure(w->step_scr, (size_t)nsys * sizeof(DotScratch)));
@@ -971,7 +980,7 @@ int batch_stepped(Workspace *w, int32_t nsys, const rbs_system *systems, rbs_inf
     std::vector<int32_t> hist_cap((size_t)nsys, 0);
     SolverState *dst = (SolverState *)w->step_state.p;
     DotScratch *dscr = (DotScratch *)w->step_scr.p;
-    size_t woff = 0, hoff = 0;
+    size_t woff = 0, hoff = 0, loff = 0;
     for (int i = 0; i < nsys; i++) {
         SolverState &h = hst[(size_t)i];
         memset(&h, 0, sizeof h);
@@ -1010,8 +1019,15 @@ int batch_stepped(Workspace *w, int32_t nsys, const rbs_system *systems, rbs_inf
         h.variant = S.variant;
         h.hist_cap = hist_cap[(size_t)i];
         CSRArgs A{S.A.n, S.A.nnz, S.A.rowptr, S.A.col, S.A.val};
+        int64_t *base = nullptr;
+        uint32_t *mask = nullptr;
+        if (const size_t bytes = layout_of(S)) {
+            base = (int64_t *)((char *)w->step_diag.p + loff);
+            mask = (uint32_t *)(base + (S.A.n + 31) / 32);
+            loff += bytes;
+        }
         step_ctx_make(hctx.data() + (size_t)i * cb, A, V, S.b, S.x0, S.jacobi_diag, dst + i, dscr + i,
-                      hist_dev[(size_t)i]);
+                      hist_dev[(size_t)i], mask, base);
     }
     // tasks of a set of systems of one variant, appended to `out`
     auto tasks_of = [&](const std::vector<int> &ids, std::vector<StepTask> &out) {
@@ -1050,6 +1066,9 @@ int batch_stepped(Workspace *w, int32_t nsys, const rbs_system *systems, rbs_inf
     CK(step_admit(w->step_ctx.p, dtask, (int)ncls, RBS_CLASSIC, w->stream));
     CK(step_admit(w->step_ctx.p, dtask + ncls, (int)(tasks.size() - ncls), RBS_PIPELINED, w->stream));
     CK(cudaMemcpyAsync(hst.data(), dst, (size_t)nsys * sizeof(SolverState), cudaMemcpyDeviceToHost, w->stream));
+    std::vector<int32_t> diags((size_t)nsys, 0);
+    CK(cudaMemcpy2DAsync(diags.data(), sizeof(int32_t), (const char *)w->step_ctx.p + step_ctx_diags_offset(), cb,
+                         sizeof(int32_t), (size_t)nsys, cudaMemcpyDeviceToHost, w->stream));
     CK(cudaStreamSynchronize(w->stream));
     std::vector<int32_t> ran((size_t)nsys, 0);
     auto live = [&](int i) { return !hst[(size_t)i].done && ran[(size_t)i] < maxit[(size_t)i]; };
@@ -1060,6 +1079,8 @@ int batch_stepped(Workspace *w, int32_t nsys, const rbs_system *systems, rbs_inf
     if (!w->ev_join) CK(cudaEventCreateWithFlags(&w->ev_join, cudaEventDisableTiming));
     CK(ensure_host(w->h_states, (size_t)nsys * sizeof(SolverState)));
     SolverState *pst = (SolverState *)w->h_states.p;
+    // systems laid out by their diagonals step in launches of their own
+    const auto laid = [&](int i) { return diags[(size_t)i] > 0; };
     for (;;) {
         std::vector<int> c2, p2;
         int32_t chunk = 8;
@@ -1073,22 +1094,32 @@ int batch_stepped(Workspace *w, int32_t nsys, const rbs_system *systems, rbs_inf
         if (c2.empty() && p2.empty()) break;
         rows = pick_rows(live_rows);
         tasks.clear();
-        tasks_of(c2, tasks);
-        const size_t nc = tasks.size();
-        tasks_of(p2, tasks);
+        size_t at[5] = {0};  // tasks of the classic systems, laid out and not, then the pipelined ones
+        const auto append = [&](const std::vector<int> &ids, bool with, size_t &end) {
+            std::vector<int> of;
+            for (int i : ids)
+                if (laid(i) == with) of.push_back(i);
+            tasks_of(of, tasks);
+            end = tasks.size();
+        };
+        append(c2, true, at[1]);
+        append(c2, false, at[2]);
+        append(p2, true, at[3]);
+        append(p2, false, at[4]);
         // the pinned task list is rewritten only after the previous chunk's
         // copy from it has completed (the stream was synchronised)
         CK(ensure_host(w->h_tasks, tasks.size() * sizeof(StepTask)));
         memcpy(w->h_tasks.p, tasks.data(), tasks.size() * sizeof(StepTask));
         CK(cudaMemcpyAsync(dtask, w->h_tasks.p, tasks.size() * sizeof(StepTask), cudaMemcpyHostToDevice, w->stream));
-        const int np = (int)(tasks.size() - nc);
+        const int np = (int)(at[4] - at[2]);
         if (np > 0) {
             CK(cudaEventRecord(w->ev_fork, w->stream));
             CK(cudaStreamWaitEvent(w->side, w->ev_fork, 0));
         }
         for (int k = 0; k < chunk; k++) {
-            CK(step_iteration(w->step_ctx.p, dtask, (int)nc, RBS_CLASSIC, w->stream));
-            CK(step_iteration(w->step_ctx.p, dtask + nc, np, RBS_PIPELINED, w->side));
+            for (int g = 0; g < 4; g++)
+                CK(step_iteration(w->step_ctx.p, dtask + at[g], (int)(at[g + 1] - at[g]), g < 2 ? RBS_CLASSIC : RBS_PIPELINED,
+                                  g % 2 == 0, g < 2 ? w->stream : w->side));
         }
         if (np > 0) {
             CK(cudaEventRecord(w->ev_join, w->side));

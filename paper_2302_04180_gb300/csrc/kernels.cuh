@@ -569,15 +569,20 @@ struct DiagLayout {
     static_assert(BUF % 16 == 0 && SCRATCH >= FLUSH_SCRATCH, "the flush reuses the staging buffers");
 };
 
-template <int N, class F>
-__device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const DiagArgs &D, const double *__restrict__ x,
+//
+// Rows [32 c_begin, n_end) of the chunks [c_begin, c_end), blocks 0 .. nblk - 1
+// (this one is blk) together; off(j): the j-th diagonal, m of them.
+template <int N, class Off, class F>
+__device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const uint32_t *__restrict__ mask,
+                                               const int64_t *__restrict__ base, int m, Off &&off, int c_begin,
+                                               int c_end, int n_end, int blk, int nblk, const double *__restrict__ x,
                                                const double *__restrict__ z, bool test_stall, unsigned &err, F &&fn) {
     constexpr unsigned FULL = 0xffffffffu;
     using L = DiagLayout<N>;
     constexpr int G = L::G, PER = L::PER;
     __shared__ __align__(8) unsigned long long s_bar[L::WARPS][2];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int n = (int)A.n, chunks = (n + 31) >> 5;
+    const int n = n_end;
     unsigned char *bufs = warp_scratch<L::SCRATCH, L::WARPS>();
     unsigned long long *bars = s_bar[wid];
     if (lane == 0) {
@@ -587,16 +592,16 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const DiagArgs 
     }
     __syncwarp();
     const long long wait_limit = test_stall ? SPMV_TEST_WAIT_LIMIT : SPMV_WAIT_LIMIT;
-    // This warp's chunks in turn: whole rounds of tiles, then chunk by chunk, so
+    // This warp's c_end in turn: whole rounds of tiles, then chunk by chunk, so
     // that the last round is even over the blocks. `left`: steps to go in the
-    // tile; c >= chunks: none.
-    const int round = gridDim.x * nw, tiled = chunks / (round * SPMV_TILE) * (round * SPMV_TILE);
+    // tile; c >= c_end: none.
+    const int round = nblk * nw, tiled = c_begin + (c_end - c_begin) / (round * SPMV_TILE) * (round * SPMV_TILE);
     struct Walk {
         int c, left;
     };
     auto first = [&]() {
-        return tiled ? Walk{(int)blockIdx.x * (SPMV_TILE * nw) + wid, SPMV_TILE - 1}
-                     : Walk{(int)blockIdx.x * nw + wid, 0};
+        return tiled > c_begin ? Walk{c_begin + blk * (SPMV_TILE * nw) + wid, SPMV_TILE - 1}
+                               : Walk{c_begin + blk * nw + wid, 0};
     };
     auto next = [&](Walk &w) {
         if (w.left > 0) {
@@ -606,7 +611,7 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const DiagArgs 
             // the next round's tile, or the first chunk after the rounds
             w.c += (round - nw) * SPMV_TILE + nw;
             w.left = SPMV_TILE - 1;
-            if (w.c >= tiled) w = Walk{tiled + (int)blockIdx.x * nw + wid, 0};
+            if (w.c >= tiled) w = Walk{tiled + blk * nw + wid, 0};
         } else {
             w.c += round;
         }
@@ -617,9 +622,9 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const DiagArgs 
     };
     auto head = [&](int c) {
         Head h{0, 0u};
-        if (c < chunks) {
-            h.base = D.base[c];
-            h.word = D.mask[c * 32 + lane];
+        if (c < c_end) {
+            h.base = base[c];
+            h.word = mask[c * 32 + lane];
         }
         return h;
     };
@@ -643,7 +648,7 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const DiagArgs 
     auto gather = [&](int row, uint32_t word, int g, double (&xv)[PER]) {
 #pragma unroll
         for (int j = 0; j < PER; j++)
-            if ((word >> (g * PER + j)) & 1u) xv[j] = __ldg(x + (row + D.off[g * PER + j]));
+            if ((word >> (g * PER + j)) & 1u) xv[j] = __ldg(x + (row + off(g * PER + j)));
     };
     Walk w0 = first(), w1 = w0;  // w0: the chunk being computed, w1: the one after
     next(w1);
@@ -651,7 +656,7 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const DiagArgs 
     unsigned parity = 0u;  // bit b: phase of buffer b's barrier to wait for
     double xa[PER], xb[PER], z0 = 0.0, z1 = 0.0;
     int cur = 0;
-    if (w0.c < chunks) {
+    if (w0.c < c_end) {
         stage(h0, 0);
         gather(w0.c * 32 + lane, h0.word, 0, xa);
         if (z && w0.c * 32 + lane < n) z0 = __ldg(z + w0.c * 32 + lane);
@@ -661,7 +666,7 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const DiagArgs 
     // false when the wait for the values ran out.
     auto step = [&](int b, double (&xc)[PER], double (&xn)[PER], double &zc, double &zn) {
         const int row = w0.c * 32 + lane, row1 = w1.c * 32 + lane;
-        if (w1.c < chunks) stage(h1, b ^ 1);
+        if (w1.c < c_end) stage(h1, b ^ 1);
         Walk w2 = w1;
         next(w2);
         const Head h2 = head(w2.c);
@@ -706,12 +711,12 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const DiagArgs 
             // next chunk's first ahead of this one's last
 #pragma unroll
             for (int g = 0; g < G; g += 2) {
-                if (g * PER >= D.m) break;
+                if (g * PER >= m) break;
                 gather(row, h0.word, g + 1, xn);
                 chain(g, xc);
-                if (g + 2 < G && (g + 2) * PER < D.m) gather(row, h0.word, g + 2, xc);
+                if (g + 2 < G && (g + 2) * PER < m) gather(row, h0.word, g + 2, xc);
                 else next_gather(xc, zc);
-                if ((g + 1) * PER < D.m) chain(g + 1, xn);
+                if ((g + 1) * PER < m) chain(g + 1, xn);
             }
         }
         if (row < n) fn((int64_t)row, acc, zr);
@@ -724,10 +729,10 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const DiagArgs 
     };
     // two steps per turn (the buffers, and for one group the gathers, swap roles)
     bool ok = true;
-    while (w0.c < chunks) {
+    while (w0.c < c_end) {
         cur = 0;
         if (!(ok = step(0, xa, xb, z0, z1))) break;
-        if (w0.c >= chunks) break;
+        if (w0.c >= c_end) break;
         cur = 1;
         if (!(ok = G == 1 ? step(1, xb, xa, z1, z0) : step(1, xa, xb, z0, z1))) break;
     }
@@ -736,8 +741,8 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const DiagArgs 
     // this and every later row from global memory, then wait (bounded) for the
     // copies in flight.
     err |= ERR_TIMEOUT;
-    const bool more = w1.c < chunks;
-    for (; w0.c < chunks; next(w0)) {
+    const bool more = w1.c < c_end;
+    for (; w0.c < c_end; next(w0)) {
         const int row = w0.c * 32 + lane;
         if (row < n) {
             bool bad = false;
@@ -755,6 +760,112 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const DiagArgs 
         }
     }
     __syncwarp();
+}
+
+// The same over a whole matrix and grid.
+template <int N, class F>
+__device__ __forceinline__ void spmv_grid_diag(const CSRView &A, const DiagArgs &D, const double *__restrict__ x,
+                                               const double *__restrict__ z, bool test_stall, unsigned &err, F &&fn) {
+    spmv_rows_diag<N>(
+        A, D.mask, D.base, D.m, [&](int j) { return D.off[j]; }, 0, (int)((A.n + 31) >> 5), (int)A.n, (int)blockIdx.x,
+        (int)gridDim.x, x, z, test_stall, err, fn);
+}
+
+// ---- set-up: structure check, Jacobi, diagonal layout -----------------------------
+
+// The distinct values of column - row in 256 rows (every row of a small matrix,
+// else rows at scattered places), ascending, into off; returns their number, 0 if
+// there are more than `most`. One block of 256 threads; all get the number. A
+// diagonal that the sample misses is found out by check_row.
+__device__ __forceinline__ int sample_diags(const CSRView &A, int most, int32_t *off) {
+    constexpr int SLOTS = 64, EMPTY = 0x7fffffff;
+    __shared__ int slot[SLOTS];
+    __shared__ int count;
+    if (threadIdx.x < SLOTS) slot[threadIdx.x] = EMPTY;
+    if (threadIdx.x == 0) count = 0;
+    __syncthreads();
+    // a multiplicative hash of the thread number spreads the rows, whatever the grid sides
+    const int64_t i = A.n <= 256 ? (int64_t)threadIdx.x
+                                 : (int64_t)(((unsigned long long)(threadIdx.x * 2654435769u) * (unsigned long long)A.n) >> 32);
+    if (i < A.n) {
+        const int64_t b = A.rowptr[i], e = A.rowptr[i + 1];
+        if (b < 0 || e < b || e > A.nnz || e - b > most) {
+            atomicAdd(&count, most + 1);
+        } else {
+            for (int64_t k = b; k < e && *(volatile int *)&count <= most; k++) {
+                const int o = (int)((int64_t)A.col[k] - i);
+                unsigned h = ((unsigned)o * 2654435769u) >> 26;
+                for (int t = 0; t < SLOTS; t++, h = (h + 1) & (SLOTS - 1)) {
+                    const int was = atomicCAS(&slot[h], EMPTY, o);
+                    if (was == EMPTY) atomicAdd(&count, 1);
+                    if (was == EMPTY || was == o) break;
+                }
+            }
+        }
+    }
+    __syncthreads();
+    const int m = count <= most ? count : 0;
+    if (threadIdx.x < SLOTS && m > 0) {
+        const int o = slot[threadIdx.x];
+        int rank = 0;
+        for (int t = 0; t < SLOTS; t++) rank += slot[t] < o;
+        if (o != EMPTY) off[rank] = o;
+    }
+    return m;
+}
+
+// One row of the set-up: rowptr within [0, nnz] and non-decreasing, columns in
+// [0, n) (error bit 1); inv = RN(1 / d) with d the given diagonal or the first
+// stored (i, i) entry, a zero, NaN or missing one sets bit 2 and inv = 0; word:
+// which of the m diagonals s_off (ascending, then 0x7fffffff) the row has, or
+// ERR_DIAGS if its columns do not ascend along them. Eight columns are loaded at a
+// time.
+struct RowSetup {
+    uint32_t word;
+    unsigned err;
+    double inv;
+    int64_t first;  // rowptr[i]
+};
+__device__ __forceinline__ RowSetup check_row(const CSRView &A, int64_t i, const double *diag, const int *s_off, int m) {
+    const int64_t b = A.rowptr[i], e = A.rowptr[i + 1];
+    RowSetup o{0u, 0u, 0.0, b};
+    double d = 0.0;
+    bool found = false, fits = m > 0;
+    if (b < 0 || e < b || e > A.nnz) {
+        o.err |= 1u;
+    } else {
+        int j = 0;
+        for (int64_t k0 = b; k0 < e; k0 += 8) {
+            int32_t c[8];
+#pragma unroll
+            for (int t = 0; t < 8; t++) c[t] = k0 + t < e ? A.col[k0 + t] : 0;
+#pragma unroll
+            for (int t = 0; t < 8; t++) {
+                if (k0 + t >= e) break;
+                if ((uint64_t)(int64_t)c[t] >= (uint64_t)A.n) o.err |= 1u;
+                if (!found && (int64_t)c[t] == i) {
+                    d = A.val[k0 + t];
+                    found = true;
+                }
+                if (fits) {
+                    // columns ascend, so the diagonals are met in order; the list
+                    // ends with a value that no difference reaches
+                    const int w = (int)((int64_t)c[t] - i);
+                    while (s_off[j] < w) j++;
+                    if (s_off[j] == w && j < m) o.word |= 1u << j++;
+                    else fits = false;
+                }
+            }
+        }
+    }
+    if (!fits) o.err |= ERR_DIAGS;
+    if (diag) {
+        d = diag[i];
+        found = true;
+    }
+    if (!found || d == 0.0 || d != d) o.err |= 2u;
+    else o.inv = __ddiv_rn(1.0, d);
+    return o;
 }
 
 // The whole matrix over the grid: every warp of every block.

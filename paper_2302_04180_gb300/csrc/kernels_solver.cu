@@ -95,7 +95,7 @@ __device__ __forceinline__ bool finish_fused(ExactRows<K, W, false> &red, DotScr
 template <int CAP, class F>
 __device__ __forceinline__ void fused_spmv(const Ctx &c, const double *x, const double *z, unsigned &eb, F &&fn) {
     if constexpr (CAP < 0)
-        spmv_rows_diag<-CAP>(c.A, c.D, x, z, (c.spmv_mode & SPMV_TEST_STALL) != 0, eb, fn);
+        spmv_grid_diag<-CAP>(c.A, c.D, x, z, (c.spmv_mode & SPMV_TEST_STALL) != 0, eb, fn);
     else if constexpr (FusedScratch<CAP>::REG)
         spmv_rows_reg<false, CAP, false>(c.A, 0, c.A.n, (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5),
                                          (int64_t)gridDim.x * (blockDim.x >> 5), x, z, true,

@@ -8,8 +8,10 @@
 // last block runs the scalar tail on the system's own device state. Every
 // system therefore gets the bits a solve of it alone gives, whatever else
 // shares the launch, and a system that has stopped skips every later phase.
+#include <cstddef>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 
 #include "kernels.cuh"
 #include "launch.h"
@@ -44,57 +46,91 @@ __device__ __forceinline__ void seg_spmv(const Ctx &c, const StepTask &t, const 
 
 constexpr int SCR = SpmvLayout<SPMV_CAP_SHORT>::SCRATCH;
 
-// ---- admission ------------------------------------------------------------------
-
-// Structure check and Jacobi set-up of the segment's rows: rowptr within
-// [0, nnz] and non-decreasing, rowptr[0] = 0 and rowptr[n] = nnz, columns in
-// [0, n) (error bit 1); invd_i = RN(1 / d_i) with d the given diagonal or the
-// first stored (i, i) entry, a zero, NaN or missing one sets error bit 2 (the
-// checks of the per-solve path).
-__global__ void __launch_bounds__(256) k_step_prepare(const Ctx *ctxs, const StepTask *tasks) {
-    const StepTask t = tasks[blockIdx.x];
-    const Ctx c = ctxs[t.sys];
-    const CSRView A = c.A;
-    bool bad = false, bad_diag = false;
-    if (threadIdx.x == 0 && t.lo == 0 && A.rowptr[0] != 0) bad = true;
-    if (threadIdx.x == 0 && t.hi == A.n && A.rowptr[A.n] != A.nnz) bad = true;
-    for (int64_t i = t.lo + threadIdx.x; i < t.hi; i += blockDim.x) {
-        const int64_t b = A.rowptr[i], e = A.rowptr[i + 1];
-        double d = 0.0;
-        bool found = false;
-        if (b < 0 || e < b || e > A.nnz) {
-            bad = true;
-        } else {
-            for (int64_t k = b; k < e; k++) {
-                const int32_t col = A.col[k];
-                if ((uint64_t)(int64_t)col >= (uint64_t)A.n) bad = true;
-                else if (!found && col == i) {
-                    d = A.val[k];
-                    found = true;
-                }
-            }
-        }
-        if (c.diag) {
-            d = c.diag[i];
-            found = true;
-        }
-        if (!found || d == 0.0 || d != d) {
-            bad_diag = true;
-            c.invd[i] = 0.0;
-        } else {
-            c.invd[i] = __ddiv_rn(1.0, d);
-        }
-    }
-    if (bad) atomicOr(c.err, 1u);
-    if (bad_diag) atomicOr(c.err, 2u);
+// The same for a system laid out by its diagonals (segments start at multiples of
+// 64 rows). Every thread of the block calls it.
+constexpr int STEP_DIAGS = 7;
+template <class F>
+__device__ __forceinline__ void seg_spmv_diag(const Ctx &c, const int32_t *off, const StepTask &t, const double *x,
+                                              const double *z, unsigned &err, F &&fn) {
+    __shared__ int s_off[STEP_DIAGS];
+    if (threadIdx.x < STEP_DIAGS) s_off[threadIdx.x] = off[threadIdx.x];
+    __syncthreads();
+    spmv_rows_diag<STEP_DIAGS>(
+        c.A, c.D.mask, c.D.base, c.D.m, [&](int j) { return s_off[j]; }, (int)(t.lo >> 5), (int)((t.hi + 31) >> 5),
+        (int)t.hi, 0, 1, x, z, false, err, fn);
+}
+template <bool DIAG, class F>
+__device__ __forceinline__ void step_spmv(const Ctx *ctxs, const Ctx &c, const StepTask &t, const double *x,
+                                          const double *z, unsigned &err, F &&fn) {
+    if constexpr (DIAG) seg_spmv_diag(c, ctxs[t.sys].D.off, t, x, z, err, fn);
+    else seg_spmv(c, t, x, z, err, fn);
+}
+// K dots beside either product: windows in shared memory where the staging leaves
+// it, as in the per-solve kernels.
+template <int K, bool DIAG>
+using StepDot = typename std::conditional<DIAG, ExactRows<K, 12, false>, ExactR<K, SQ>>::type;
+template <int K>
+__device__ __forceinline__ bool finish_step(ExactR<K, SQ> &red, DotScratch *g, double *vals, unsigned nblk, bool coop) {
+    return red.template finish<SCR>(g, vals, nblk, coop);
+}
+template <int K, int W>
+__device__ __forceinline__ bool finish_step(ExactRows<K, W, false> &red, DotScratch *g, double *vals, unsigned nblk, bool) {
+    return red.finish(g, vals, nblk);
 }
 
-// A system that failed its checks stops before its set-up (one thread per
-// system: the one of its first task).
-__global__ void k_step_validate(const Ctx *ctxs, const StepTask *tasks, int ntasks) {
+// ---- admission ------------------------------------------------------------------
+
+// The diagonals of every system that has room for a layout by them (its first
+// task's block).
+__global__ void __launch_bounds__(256) k_step_sample(Ctx *ctxs, const StepTask *tasks) {
+    const StepTask t = tasks[blockIdx.x];
+    Ctx &c = ctxs[t.sys];
+    if (t.lo != 0 || !c.D.mask) return;
+    const int m = sample_diags(c.A, STEP_DIAGS, c.D.off);
+    if (threadIdx.x == 0) c.D.m = m;
+}
+
+// Structure check, Jacobi set-up and layout by diagonals of the segment's rows
+// (check_row; the checks of the per-solve path). Segments start at multiples of
+// 64 rows.
+__global__ void __launch_bounds__(256) k_step_prepare(const Ctx *ctxs, const StepTask *tasks) {
+    __shared__ int s_off[STEP_DIAGS + 1];
+    const StepTask t = tasks[blockIdx.x];
+    const Ctx &c = ctxs[t.sys];
+    const CSRView A = c.A;
+    const int m = c.D.mask ? c.D.m : 0;
+    if (threadIdx.x <= STEP_DIAGS) s_off[threadIdx.x] = (int)threadIdx.x < m ? c.D.off[threadIdx.x] : 0x7fffffff;
+    __syncthreads();
+    unsigned eb = 0u;
+    if (threadIdx.x == 0 && t.lo == 0 && A.rowptr[0] != 0) eb |= 1u;
+    if (threadIdx.x == 0 && t.hi == A.n && A.rowptr[A.n] != A.nnz) eb |= 1u;
+    uint32_t *mask = const_cast<uint32_t *>(c.D.mask);
+    int64_t *base = const_cast<int64_t *>(c.D.base);
+    const int64_t end = t.hi == A.n ? (A.n + 31) / 32 * 32 : t.hi;
+    for (int64_t i = t.lo + threadIdx.x; i < end; i += blockDim.x) {
+        uint32_t word = 0u;
+        if (i < A.n) {
+            const RowSetup r = check_row(A, i, c.diag, s_off, m);
+            eb |= m > 0 ? r.err : r.err & ~ERR_DIAGS;
+            c.invd[i] = r.inv;
+            if (m > 0 && (i & 31) == 0) base[i >> 5] = r.first;
+            word = r.word | (uint32_t)(r.first - A.rowptr[i & ~31LL]) << 8;
+        }
+        if (m > 0) mask[i] = word;
+    }
+    eb = __reduce_or_sync(__activemask(), eb);
+    if (eb && (*(volatile unsigned *)c.err & eb) != eb) atomicOr(c.err, eb);
+}
+
+// A system that failed its checks stops before its set-up, one whose rows do not
+// lie on its sampled diagonals has no layout (one thread per system: the one of
+// its first task).
+__global__ void k_step_validate(Ctx *ctxs, const StepTask *tasks, int ntasks) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= ntasks || tasks[j].lo != 0) return;
-    const Ctx c = ctxs[tasks[j].sys];
+    Ctx &c = ctxs[tasks[j].sys];
+    if (!c.D.mask || (*c.err & ERR_DIAGS)) c.D.m = 0;
+    *c.err &= ~ERR_DIAGS;
     if (*c.err) {
         c.st->status = RBS_EINVAL;
         c.st->done = 1;
@@ -119,25 +155,28 @@ __global__ void __launch_bounds__(256) k_step_cls_setup(const Ctx *ctxs, const S
     if (red.finish(c.g, vals, t.nblk)) sc.tail([&](SolverState *st) { tail_cls_setup(st, vals); });
 }
 
-template <class R>
-__global__ void __launch_bounds__(256, 3) k_step_cls_k1(const Ctx *ctxs, const StepTask *tasks) {
+template <bool DIAG>
+__device__ __forceinline__ void step_k1(const Ctx *ctxs, const StepTask *tasks) {
     const StepTask t = tasks[blockIdx.x];
     const Ctx c = ctxs[t.sys];
     StateCopy sc;
     sc.load(c.st);
-    R red;
+    StepDot<1, DIAG> red;
     red.init();  // ends in a barrier
     if (sc.copy->done) return;
     unsigned eb = 0u;
-    seg_spmv(c, t, c.ph, c.r0, eb, [&](int64_t i, double si, double r0) {
+    step_spmv<DIAG>(ctxs, c, t, c.ph, c.r0, eb, [&](int64_t i, double si, double r0) {
         c.s[i] = si;
         red.add(0, r0, si);
     });
     if (eb) atomicOr(c.err, eb);
-    __shared__ double vals[R::K];
-    if (red.template finish<SCR>(c.g, vals, t.nblk, !(eb & ERR_TIMEOUT)))
+    __shared__ double vals[1];
+    if (finish_step(red, c.g, vals, t.nblk, !(eb & ERR_TIMEOUT)))
         sc.tail([&](SolverState *st) { tail_cls_alpha(st, vals); });
 }
+__global__ void __launch_bounds__(256, 3) k_step_cls_k1(const Ctx *ctxs, const StepTask *tasks) { step_k1<false>(ctxs, tasks); }
+// (systems laid out by their diagonals)
+__global__ void __launch_bounds__(256, 3) k_step_diag_k1(const Ctx *ctxs, const StepTask *tasks) { step_k1<true>(ctxs, tasks); }
 
 __global__ void __launch_bounds__(256) k_step_cls_k2(const Ctx *ctxs, const StepTask *tasks) {
     const StepTask t = tasks[blockIdx.x];
@@ -158,26 +197,29 @@ __global__ void __launch_bounds__(256) k_step_cls_k2(const Ctx *ctxs, const Step
     });
 }
 
-template <class R>
-__global__ void __launch_bounds__(256, 3) k_step_cls_k3(const Ctx *ctxs, const StepTask *tasks) {
+template <bool DIAG>
+__device__ __forceinline__ void step_k3(const Ctx *ctxs, const StepTask *tasks) {
     const StepTask t = tasks[blockIdx.x];
     const Ctx c = ctxs[t.sys];
     StateCopy sc;
     sc.load(c.st);
-    R red;
+    StepDot<2, DIAG> red;
     red.init();  // ends in a barrier
     if (sc.copy->done) return;
     unsigned eb = 0u;
-    seg_spmv(c, t, c.qh, c.q, eb, [&](int64_t i, double yi, double qi) {
+    step_spmv<DIAG>(ctxs, c, t, c.qh, c.q, eb, [&](int64_t i, double yi, double qi) {
         c.y[i] = yi;
         red.add(0, qi, yi);
         red.add_sq(1, yi);
     });
     if (eb) atomicOr(c.err, eb);
-    __shared__ double vals[R::K];
-    if (red.template finish<SCR>(c.g, vals, t.nblk, !(eb & ERR_TIMEOUT)))
+    __shared__ double vals[2];
+    if (finish_step(red, c.g, vals, t.nblk, !(eb & ERR_TIMEOUT)))
         sc.tail([&](SolverState *st) { tail_cls_omega(st, vals); });
 }
+__global__ void __launch_bounds__(256, 3) k_step_cls_k3(const Ctx *ctxs, const StepTask *tasks) { step_k3<false>(ctxs, tasks); }
+// (systems laid out by their diagonals)
+__global__ void __launch_bounds__(256, 3) k_step_diag_k3(const Ctx *ctxs, const StepTask *tasks) { step_k3<true>(ctxs, tasks); }
 
 template <class R>
 __global__ void __launch_bounds__(256, 4) k_step_cls_k4(const Ctx *ctxs, const StepTask *tasks) {
@@ -246,14 +288,14 @@ __global__ void __launch_bounds__(256, 3) k_step_pipe_setup2(const Ctx *ctxs, co
 }
 
 // y = A x without a dot: the pipelined S10 (v = A zhat) and S18 / set-up (t = A what)
-template <bool TO_V>
+template <bool TO_V, bool DIAG>
 __global__ void __launch_bounds__(256, 3) k_step_spmv(const Ctx *ctxs, const StepTask *tasks) {
     const StepTask t = tasks[blockIdx.x];
     const Ctx c = ctxs[t.sys];
     if (c.st->done) return;
     unsigned eb = 0u;
     double *y = TO_V ? c.v : c.t;
-    seg_spmv(c, t, TO_V ? c.zh : c.wh, nullptr, eb, [&](int64_t i, double yi, double) { y[i] = yi; });
+    step_spmv<DIAG>(ctxs, c, t, TO_V ? c.zh : c.wh, nullptr, eb, [&](int64_t i, double yi, double) { y[i] = yi; });
     if (eb) atomicOr(c.err, eb);
 }
 
@@ -293,11 +335,18 @@ void step_carveout() {
     static std::once_flag once;
     std::call_once(once, [] {
         const int c = 75;  // as the per-solve staging kernels: three blocks per SM, L1 left for the gathers
-        cudaFuncSetAttribute(k_step_cls_k1<R1>, cudaFuncAttributePreferredSharedMemoryCarveout, c);
-        cudaFuncSetAttribute(k_step_cls_k3<R2>, cudaFuncAttributePreferredSharedMemoryCarveout, c);
-        cudaFuncSetAttribute(k_step_pipe_setup2<R2>, cudaFuncAttributePreferredSharedMemoryCarveout, c);
-        cudaFuncSetAttribute(k_step_spmv<true>, cudaFuncAttributePreferredSharedMemoryCarveout, c);
-        cudaFuncSetAttribute(k_step_spmv<false>, cudaFuncAttributePreferredSharedMemoryCarveout, c);
+        const auto set = [&](auto kern) {
+            cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, c);
+        };
+        set(k_step_cls_k1);
+        set(k_step_diag_k1);
+        set(k_step_cls_k3);
+        set(k_step_diag_k3);
+        set(k_step_pipe_setup2<R2>);
+        set(k_step_spmv<true, false>);
+        set(k_step_spmv<true, true>);
+        set(k_step_spmv<false, false>);
+        set(k_step_spmv<false, true>);
         cudaGetLastError();
     });
 }
@@ -305,7 +354,7 @@ void step_carveout() {
 }  // namespace
 
 void step_ctx_make(void *out, const CSRArgs &A, const SolverVecs &v, const double *b, const double *x0,
-                   const double *diag, SolverState *st, DotScratch *g, double *hist) {
+                   const double *diag, SolverState *st, DotScratch *g, double *hist, uint32_t *mask, int64_t *base) {
     Ctx c;
     memset(&c, 0, sizeof c);
     c.A = CSRView{A.n, A.nnz, A.rowptr, A.col, A.val};
@@ -321,15 +370,24 @@ void step_ctx_make(void *out, const CSRArgs &A, const SolverVecs &v, const doubl
     c.hist = hist;
     c.err = &g->err;
     c.spmv_mode = SPMV_MODE_SHORT;
+    c.D.mask = mask;
+    c.D.base = base;
     memcpy(out, &c, sizeof c);
 }
 
 size_t step_ctx_bytes() { return sizeof(Ctx); }
 
-cudaError_t step_admit(const void *ctxs, const StepTask *tasks, int ntasks, int variant, cudaStream_t s) {
+size_t step_ctx_diags_offset() { return offsetof(Ctx, D) + offsetof(DiagArgs, m); }
+
+bool step_wants_layout(const CSRArgs &A) {
+    return A.nnz > 0 && A.nnz <= STEP_DIAGS * A.n && ((uintptr_t)A.val & 15) == 0;
+}
+
+cudaError_t step_admit(void *ctxs, const StepTask *tasks, int ntasks, int variant, cudaStream_t s) {
     if (ntasks <= 0) return cudaSuccess;
     step_carveout();
-    const Ctx *c = static_cast<const Ctx *>(ctxs);
+    Ctx *c = static_cast<Ctx *>(ctxs);
+    k_step_sample<<<ntasks, 256, 0, s>>>(c, tasks);
     k_step_prepare<<<ntasks, 256, 0, s>>>(c, tasks);
     k_step_validate<<<(ntasks + 255) / 256, 256, 0, s>>>(c, tasks, ntasks);
     if (variant == RBS_CLASSIC) {
@@ -337,27 +395,36 @@ cudaError_t step_admit(const void *ctxs, const StepTask *tasks, int ntasks, int 
     } else {
         k_step_pipe_setup1<<<ntasks, 256, 0, s>>>(c, tasks);
         k_step_pipe_setup2<R2><<<ntasks, 256, 0, s>>>(c, tasks);
-        k_step_spmv<false><<<ntasks, 256, 0, s>>>(c, tasks);
+        k_step_spmv<false, false><<<ntasks, 256, 0, s>>>(c, tasks);
     }
     return cudaGetLastError();
 }
 
-cudaError_t step_iteration(const void *ctxs, const StepTask *tasks, int ntasks, int variant, cudaStream_t s) {
-    if (ntasks <= 0) return cudaSuccess;
-    step_carveout();
-    const Ctx *c = static_cast<const Ctx *>(ctxs);
+template <bool DIAG>
+static void iteration_t(const Ctx *c, const StepTask *tasks, int ntasks, int variant, cudaStream_t s) {
     if (variant == RBS_CLASSIC) {
-        k_step_cls_k1<R1><<<ntasks, 256, 0, s>>>(c, tasks);
+        if (DIAG) k_step_diag_k1<<<ntasks, 256, 0, s>>>(c, tasks);
+        else k_step_cls_k1<<<ntasks, 256, 0, s>>>(c, tasks);
         k_step_cls_k2<<<ntasks, 256, 0, s>>>(c, tasks);
-        k_step_cls_k3<R2><<<ntasks, 256, 0, s>>>(c, tasks);
+        if (DIAG) k_step_diag_k3<<<ntasks, 256, 0, s>>>(c, tasks);
+        else k_step_cls_k3<<<ntasks, 256, 0, s>>>(c, tasks);
         k_step_cls_k4<RowsR2><<<ntasks, 256, 0, s>>>(c, tasks);
         k_step_cls_k5<<<ntasks, 256, 0, s>>>(c, tasks);
     } else {
         k_step_pipe_p1<RowsR2><<<ntasks, 256, 0, s>>>(c, tasks);
-        k_step_spmv<true><<<ntasks, 256, 0, s>>>(c, tasks);
+        k_step_spmv<true, DIAG><<<ntasks, 256, 0, s>>>(c, tasks);
         k_step_pipe_p3<RowsR5><<<ntasks, 256, 0, s>>>(c, tasks);
-        k_step_spmv<false><<<ntasks, 256, 0, s>>>(c, tasks);
+        k_step_spmv<false, DIAG><<<ntasks, 256, 0, s>>>(c, tasks);
     }
+}
+
+cudaError_t step_iteration(const void *ctxs, const StepTask *tasks, int ntasks, int variant, bool diags,
+                           cudaStream_t s) {
+    if (ntasks <= 0) return cudaSuccess;
+    step_carveout();
+    const Ctx *c = static_cast<const Ctx *>(ctxs);
+    if (diags) iteration_t<true>(c, tasks, ntasks, variant, s);
+    else iteration_t<false>(c, tasks, ntasks, variant, s);
     return cudaGetLastError();
 }
 

@@ -183,14 +183,24 @@ struct StepTask {
 // diagonal, the system's own state and dot scratch (zero at rest), and its
 // device history records (nullable; state->hist_cap of them).
 size_t step_ctx_bytes();
+// mask, base (nullable): room for the system's layout by diagonals, one word per
+// row rounded up to 32 and one int64 per 32 rows.
 void step_ctx_make(void *out, const CSRArgs &A, const SolverVecs &v, const double *b, const double *x0,
-                   const double *diag, SolverState *st, DotScratch *g, double *hist);
+                   const double *diag, SolverState *st, DotScratch *g, double *hist, uint32_t *mask = nullptr,
+                   int64_t *base = nullptr);
+// Whether such room is worth giving: the steps know layouts of up to 7 diagonals.
+bool step_wants_layout(const CSRArgs &A);
+// Where in the device-side view the number of the system's diagonals stands after
+// its admission (int32; 0: not laid out).
+size_t step_ctx_diags_offset();
 // Admission of new systems (all of one variant): structure check and Jacobi,
 // then the set-up of Fig. 2 or Fig. 4; a system that fails its checks ends with
 // status RBS_EINVAL and its error bits in its scratch's err word.
-cudaError_t step_admit(const void *ctxs, const StepTask *tasks, int ntasks, int variant, cudaStream_t s);
-// One iteration of every listed system (all of one variant); stopped systems skip it.
-cudaError_t step_iteration(const void *ctxs, const StepTask *tasks, int ntasks, int variant, cudaStream_t s);
+cudaError_t step_admit(void *ctxs, const StepTask *tasks, int ntasks, int variant, cudaStream_t s);
+// One iteration of every listed system (all of one variant, and with `diags` all
+// laid out by their diagonals); stopped systems skip it.
+cudaError_t step_iteration(const void *ctxs, const StepTask *tasks, int ntasks, int variant, bool diags,
+                           cudaStream_t s);
 
 // occupancy-derived persistent grid for the kernels of one kind: which = 0 the
 // SpMV kernels (classic K1, pipelined S10/S18), 1 the vector kernels, 2 the
