@@ -96,6 +96,8 @@ _lib = None
 def load(path: str | None = None):
     """Load librbs.so (built by paper_2302_04180_gb300.build). Raises if absent."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -166,13 +168,30 @@ def _ptr(a):
     return a.data_ptr()
 
 
+_raw_stream = None  # torch's raw handle of a device's current stream, once torch is in use
+_float64 = None
+
+
+def _empty(n, like):
+    """n float64 values on the device of the tensor `like`."""
+    global _float64
+    if _float64 is None:
+        import torch
+        _float64 = torch.float64
+    return like.new_empty(n, dtype=_float64)
+
+
 def _stream(stream, *tensors):
     if stream is not None:
         return stream if isinstance(stream, int) else stream.cuda_stream
     for t in tensors:
         if t is not None and not isinstance(t, np.ndarray) and t.is_cuda:
-            import torch
-            return torch.cuda.current_stream(t.device).cuda_stream
+            # (torch.cuda.current_stream() builds a Stream object: 2 us of a 11 us call)
+            global _raw_stream
+            if _raw_stream is None:
+                import torch
+                _raw_stream = torch._C._cuda_getCurrentRawStream
+            return _raw_stream(t.get_device())
     return None
 
 
@@ -231,9 +250,7 @@ def rbs_exdot(x, y, out=None, stream=None):
         _check(load().rbs_exdot(_ptr(x), _ptr(y), n, res.ctypes.data, _stream(stream)))
         return float(res[0])
     if out is None:
-        import torch
-        dev = x.device if not isinstance(x, np.ndarray) else y.device
-        out = torch.empty(1, dtype=torch.float64, device=dev)
+        out = _empty(1, y if isinstance(x, np.ndarray) else x)
     _check(load().rbs_exdot(_ptr(x), _ptr(y), n, _ptr(out), _stream(stream, x, y, out)))
     return out
 
@@ -241,11 +258,10 @@ def rbs_exdot(x, y, out=None, stream=None):
 def rbs_exdot_multi(xs, ys, out=None, stream=None):
     k = len(xs)
     n = int(xs[0].shape[0])
-    xa = (C.c_void_p * k)(*[_ptr(t) for t in xs])
-    ya = (C.c_void_p * k)(*[_ptr(t) for t in ys])
+    xa = (C.c_void_p * k)(*map(_ptr, xs))
+    ya = (C.c_void_p * k)(*map(_ptr, ys))
     if out is None:
-        import torch
-        out = torch.empty(k, dtype=torch.float64, device=xs[0].device)
+        out = _empty(k, xs[0])
     _check(load().rbs_exdot_multi(k, xa, ya, n, _ptr(out), _stream(stream, xs[0], out)))
     return out
 
@@ -293,8 +309,7 @@ def rbs_round_limbs(limbs, flags, out=None, stream=None):
 
 def rbs_spmv_csr(A, x, y=None, stream=None):
     if y is None:
-        import torch
-        y = torch.empty(A.n, dtype=torch.float64, device=x.device)
+        y = _empty(A.n, x)
     csr = _csr(A)
     _check(load().rbs_spmv_csr(C.byref(csr), _ptr(x), _ptr(y), _stream(stream, x, y)))
     return y

@@ -135,7 +135,7 @@ struct Workspace {
     Buf h_tasks, h_states;  // pinned (cudaMallocHost)
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
-    std::string graph_key;
+    std::string graph_key, graph_seen;  // of exec; of the last solve that ran without one
     // batched solve: the per-batch launches captured once a system set and
     // schedule repeats (batch_seen: the previous call's key, not captured yet)
     cudaGraphExec_t batch_exec = nullptr;
@@ -355,11 +355,26 @@ struct EventTimer : KernelTimer {
 // condition cost 6 us a turn, an iteration after the stop a few empty launches
 // (32^3: 35.4 us an iteration with one, 31.0 with four, 30.5 with eight).
 constexpr int LOOP_UNROLL = 4;
-int graph_loop(Workspace *w, const SolverArgs &a, int variant, int maxit) {
-    const int unroll = maxit < LOOP_UNROLL ? maxit : LOOP_UNROLL;
+std::string graph_key(const SolverArgs &a, int variant, int unroll) {
     std::string key((const char *)&a, sizeof a);
     key.append((const char *)&variant, sizeof variant);
     key.append((const char *)&unroll, sizeof unroll);
+    return key;
+}
+// A solve of few iterations on arguments that were not the last one's either:
+// its iterations are enqueued one by one, since building the graph would cost
+// about 100 us and an iteration gains some 6 from it.
+constexpr int LOOP_DIRECT = 16;
+bool loop_direct(Workspace *w, const SolverArgs &a, int variant, int maxit) {
+    if (maxit > LOOP_DIRECT) return false;
+    std::string key = graph_key(a, variant, std::min(maxit, LOOP_UNROLL));
+    if ((w->exec && key == w->graph_key) || key == w->graph_seen) return false;
+    w->graph_seen = std::move(key);
+    return true;
+}
+int graph_loop(Workspace *w, const SolverArgs &a, int variant, int maxit) {
+    const int unroll = std::min(maxit, LOOP_UNROLL);
+    std::string key = graph_key(a, variant, unroll);
     if (!(w->exec && key == w->graph_key)) {
         std::lock_guard<std::mutex> cap(g_cap_mu);
         if (w->exec) cudaGraphExecDestroy(w->exec);
@@ -803,7 +818,9 @@ int rbs_solve_ex(const rbs_csr *A, const double *b, const double *x0, const doub
     CK(solver_setup(a, variant, w->stream, tm));
 
     const bool use_graph = !tm && o.loop_mode == RBS_LOOP_GRAPH && maxit > 0;
-    if (use_graph) {
+    if (use_graph && loop_direct(w, a, variant, maxit)) {
+        for (int i = 0; i < maxit; i++) CK(solver_iteration(a, variant, w->stream, nullptr));
+    } else if (use_graph) {
         if ((rc = graph_loop(w, a, variant, maxit))) return rc;
     }
     int chunk = o.check_every > 0 ? o.check_every : (p_check_every.load() > 0 ? (int)p_check_every.load() : 8);

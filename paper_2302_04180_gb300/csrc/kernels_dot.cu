@@ -1,9 +1,7 @@
 // Standalone kernels: exact dot (single and multi-output), long-accumulator
 // export and rounding, the allocation-free exact dot, the FPE-8 dot.
 #include <algorithm>
-#include <map>
 #include <mutex>
-#include <tuple>
 
 #include "kernels.cuh"
 #include "launch.h"
@@ -124,33 +122,18 @@ static auto with_window(int window, F &&f) {
     return f(k_exdot<16, false>);
 }
 
-// Cached per device and kernel variant: the query costs a few microseconds of
-// host time, which a short dot would otherwise pay on every call.
 int exdot_blocks_per_sm(int window, int block) {
-    static std::mutex mu;
-    static std::map<std::tuple<int, int, int>, int> cache;
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) {
-        cudaGetLastError();
-        dev = -1;
-    }
-    const auto key = std::make_tuple(dev, window, block);
-    {
-        std::lock_guard<std::mutex> lk(mu);
-        const auto it = cache.find(key);
-        if (it != cache.end()) return it->second;
-    }
-    const int nb = with_window(window, [&](auto kern) {
-        int v = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, kern, block, 0) != cudaSuccess || v < 1) {
-            cudaGetLastError();
-            v = 1;
-        }
-        return v;
+    static QueryCache<std::pair<int, int>> cache;
+    return cache.get({window, block}, [&] {
+        return with_window(window, [&](auto kern) {
+            int v = 0;
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, kern, block, 0) != cudaSuccess || v < 1) {
+                cudaGetLastError();
+                v = 1;
+            }
+            return v;
+        });
     });
-    std::lock_guard<std::mutex> lk(mu);
-    cache[key] = nb;
-    return nb;
 }
 
 cudaError_t launch_exdot(int k, const double *const *xs, const double *const *ys, int64_t n,

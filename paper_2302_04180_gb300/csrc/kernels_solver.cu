@@ -19,6 +19,7 @@
 //   P4  t = A what                                                  (S18)
 // Once the stop flag is set, every later kernel returns at once.
 #include <mutex>
+#include <tuple>
 #include <type_traits>
 
 #include "kernels.cuh"
@@ -456,10 +457,14 @@ static int blocks_per_sm_t(int variant, int which, int block, int spmv_mode) {
 }
 
 int solver_blocks_per_sm(int variant, int dot_mode, int which, int block, int carveout, int spmv_mode) {
-    apply_carveout(dot_mode, carveout);
     if (which == 0 && variant == RBS_PIPELINED) return spmv_blocks_per_sm(block, carveout, spmv_mode);
-    if (dot_mode == RBS_DOT_PLAIN) return blocks_per_sm_t<PlainR<1>, PlainR<2>, PlainR<2>, PlainR<5>>(variant, which, block, spmv_mode);
-    return blocks_per_sm_t<ExactR<1, SQ>, ExactR<2, SQ>, RowsR2, RowsR5>(variant, which, block, spmv_mode);
+    static QueryCache<std::tuple<int, int, int, int, int, int>> cache;
+    return cache.get({variant, dot_mode, which, block, carveout, spmv_mode}, [&] {
+        apply_carveout(dot_mode, carveout);
+        if (dot_mode == RBS_DOT_PLAIN)
+            return blocks_per_sm_t<PlainR<1>, PlainR<2>, PlainR<2>, PlainR<5>>(variant, which, block, spmv_mode);
+        return blocks_per_sm_t<ExactR<1, SQ>, ExactR<2, SQ>, RowsR2, RowsR5>(variant, which, block, spmv_mode);
+    });
 }
 
 }  // namespace rbs

@@ -1,6 +1,7 @@
 // Standalone SpMV kernels (short rows warp-staged, long rows register-staged,
 // one thread per row), Jacobi and the CSR structure check.
 #include <mutex>
+#include <tuple>
 
 #include "kernels.cuh"
 #include "launch.h"
@@ -75,20 +76,22 @@ static void spmv_carveout(int c) {
 // Resident blocks per SM of the SpMV kernel of `mode` at this block size (the
 // long-row kernel: at its own block of SPMV_REG_WARPS warps).
 int spmv_blocks_per_sm(int block, int carveout, int mode) {
-    spmv_carveout(carveout);
-    int nb = 0;
-    const cudaError_t e = mode == SPMV_MODE_DIAG7
-                              ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_spmv_diag<7>, block, 0)
-                          : mode == SPMV_MODE_DIAG32
-                              ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_spmv_diag<32>, block, 0)
-                          : mode == SPMV_MODE_LONG
-                              ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_spmv_reg<true>, SPMV_REG_WARPS * 32, 0)
-                              : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_spmv<true, SPMV_CAP_SHORT>, block, 0);
-    if (e != cudaSuccess || nb < 1) {
-        cudaGetLastError();
-        nb = 1;
-    }
-    return nb;
+    static QueryCache<std::tuple<int, int, int>> cache;
+    return cache.get({block, carveout, mode}, [&] {
+        spmv_carveout(carveout);
+        int nb = 0;
+        const cudaError_t e =
+            mode == SPMV_MODE_DIAG7    ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_spmv_diag<7>, block, 0)
+            : mode == SPMV_MODE_DIAG32 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_spmv_diag<32>, block, 0)
+            : mode == SPMV_MODE_LONG
+                ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_spmv_reg<true>, SPMV_REG_WARPS * 32, 0)
+                : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_spmv<true, SPMV_CAP_SHORT>, block, 0);
+        if (e != cudaSuccess || nb < 1) {
+            cudaGetLastError();
+            nb = 1;
+        }
+        return nb;
+    });
 }
 
 // The long-row kernel runs its own launch shape: blocks of SPMV_REG_WARPS

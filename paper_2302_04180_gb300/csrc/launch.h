@@ -5,6 +5,10 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <map>
+#include <mutex>
+#include <utility>
+
 #include "rbs.h"
 
 namespace rbs {
@@ -47,6 +51,29 @@ struct Cfg {
     int block = 256;
     int mode = 2;       // SpMV row schedule (SPMV_MODE_*)
     int carveout = -1;  // shared-memory carveout percent, -1 = driver default
+};
+
+// A launch-shape query's answer per device and key, asked once (the runtime's
+// occupancy queries take a microsecond or two each, which every short call would
+// pay). query() runs under the lock.
+template <class Key>
+class QueryCache {
+    std::mutex mu;
+    std::map<std::pair<int, Key>, int> known;
+
+public:
+    template <class F>
+    int get(const Key &key, F &&query) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess) {
+            cudaGetLastError();
+            dev = -1;
+        }
+        std::lock_guard<std::mutex> lk(mu);
+        const auto at = known.find({dev, key});
+        if (at != known.end()) return at->second;
+        return known[{dev, key}] = query();
+    }
 };
 
 // Set the calling thread's rbs_last_error() message and return `code`.
