@@ -176,7 +176,7 @@ static __device__ __noinline__ uint32_t special_flags(uint32_t xh, uint32_t xl, 
 
 // Exact accumulation of x*y into window W / block accumulator sacc. With
 // SQUARE the product is x*x: it cannot be negative, so no sign handling.
-template <int Q, bool SQUARE = false>
+template <int Q, bool SQUARE = false, bool COMMON = true>
 __device__ __forceinline__ void exact_add(Win<Q> &W, uint32_t &flags, unsigned long long *sacc, double x,
                                           double y) {
     const uint32_t xh = (uint32_t)__double2hiint(x), xl = (uint32_t)__double2loint(x);
@@ -211,9 +211,10 @@ __device__ __forceinline__ void exact_add(Win<Q> &W, uint32_t &flags, unsigned l
         // empty, or above the window: flush and re-anchor with the product at
         // offset Q-2 (or 0), leaving room for somewhat larger products. Lanes that
         // open their windows together take one anchor where their products are
-        // within two limbs, for the sake of warp_flush.
+        // within two limbs, for the sake of warp_flush (COMMON; the persistent batch
+        // kernel, full of windows, loses 2 % to the extra code and goes without).
         int top = L;
-        if (W.a < 0) {
+        if (COMMON && W.a < 0) {
             const int m = (int)__reduce_max_sync(__activemask(), (unsigned)L);
             if (m - L <= (Q >= 2 ? Q - 2 : 0)) top = m;
         }
@@ -287,20 +288,32 @@ __device__ __forceinline__ unsigned char *warp_scratch() {
 
 // Windows of one anchor (the usual case): every word summed over the warp in two
 // 16-bit halves, the top word's upper half signed, and one atomic per word.
-template <int Q>
-__device__ __forceinline__ void warp_sum_words(Win<Q> &W, unsigned long long *sacc, int lane, int anchor) {
+// (Words are zero in lanes without a window.)
+__device__ __forceinline__ void warp_sum(const uint32_t (&w)[8], unsigned long long *sacc, int anchor) {
     constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
     long long mine = 0;
 #pragma unroll
     for (int k = 0; k < 8; k++) {
-        const uint32_t w = W.w[k];  // zero in lanes without a window
-        const long long low = (long long)__reduce_add_sync(FULL, w & 0xffffu);
-        const long long high =
-            k < 7 ? (long long)__reduce_add_sync(FULL, w >> 16) : (long long)__reduce_add_sync(FULL, (int)w >> 16);
+        const long long low = (long long)__reduce_add_sync(FULL, w[k] & 0xffffu);
+        const long long high = k < 7 ? (long long)__reduce_add_sync(FULL, w[k] >> 16)
+                                     : (long long)__reduce_add_sync(FULL, (int)w[k] >> 16);
         if (lane == k) mine = low + high * 65536;
-        W.w[k] = 0u;
     }
     if (lane < 8 && mine && anchor + lane < NL) sacc_add(&sacc[anchor + lane], mine);
+}
+// The same as a call: inlined beside the windows it cost the persistent batch
+// kernel 10 %.
+static __device__ __noinline__ void warp_sum_call(unsigned long long *sacc, int anchor, uint32_t w0, uint32_t w1,
+                                                  uint32_t w2, uint32_t w3, uint32_t w4, uint32_t w5, uint32_t w6,
+                                                  uint32_t w7) {
+    const uint32_t w[8] = {w0, w1, w2, w3, w4, w5, w6, w7};
+    warp_sum(w, sacc, anchor);
+}
+template <int Q>
+__device__ __forceinline__ void win_clear(Win<Q> &W) {
+#pragma unroll
+    for (int k = 0; k < 8; k++) W.w[k] = 0u;
     W.a = WIN_EMPTY;
 }
 
@@ -318,7 +331,8 @@ __device__ __forceinline__ void warp_flush(Win<Q> &W, unsigned long long *sacc) 
         return;
     }
     if (lo == hi) {
-        warp_sum_words<Q>(W, sacc, lane, lo);
+        warp_sum_call(sacc, lo, W.w[0], W.w[1], W.w[2], W.w[3], W.w[4], W.w[5], W.w[6], W.w[7]);
+        win_clear<Q>(W);
         return;
     }
     __syncwarp();

@@ -58,6 +58,11 @@ __device__ __forceinline__ double spmv_row_l2(const CSRView &A, int64_t i, const
     return acc;
 }
 
+template <bool SQUARE>
+__device__ __forceinline__ void batch_add(Win<BQ> &w, uint32_t &flags, unsigned long long *sacc, double x, double y) {
+    exact_add<BQ, SQUARE, false>(w, flags, sacc, x, y);
+}
+
 struct ClusterRed {
     unsigned long long (*acc)[NL];  // this CTA's accumulators (shared)
     long long (*red)[NL];           // group sums (shared)
@@ -211,7 +216,7 @@ __device__ void solve_classic(const Grp &cl, const SysView &V, SolverState *st, 
         r0[i] = ri;
         p[i] = ri;
         ph[i] = __dmul_rn(ri, invd[i]);
-        exact_add<BQ, true>(w1[0], f1[0], R.acc[0], ri, ri);
+        batch_add<true>(w1[0], f1[0], R.acc[0], ri, ri);
     }
     group_reduce<1>(cl, w1, f1, R);
     if (threadIdx.x == 0) tail_cls_setup(st, R.vals);
@@ -219,7 +224,7 @@ __device__ void solve_classic(const Grp &cl, const SysView &V, SolverState *st, 
     for (int guard = 0; !st->done && guard <= st->maxit; guard++) {
         group_spmv(V, ph, r0, bad, [&](int64_t i, double si, double r0i) {  // K1
             s[i] = si;
-            exact_add<BQ>(w1[0], f1[0], R.acc[0], r0i, si);
+            batch_add<false>(w1[0], f1[0], R.acc[0], r0i, si);
         });
         group_reduce<1>(cl, w1, f1, R);
         if (threadIdx.x == 0) tail_cls_alpha(st, R.vals);
@@ -236,8 +241,8 @@ __device__ void solve_classic(const Grp &cl, const SysView &V, SolverState *st, 
         cl.sync();
         group_spmv(V, qh, q, bad, [&](int64_t i, double yi, double qi) {  // K3
             y[i] = yi;
-            exact_add<BQ>(w2[0], f2[0], R.acc[0], qi, yi);
-            exact_add<BQ, true>(w2[1], f2[1], R.acc[1], yi, yi);
+            batch_add<false>(w2[0], f2[0], R.acc[0], qi, yi);
+            batch_add<true>(w2[1], f2[1], R.acc[1], yi, yi);
         });
         group_reduce<2>(cl, w2, f2, R);
         if (threadIdx.x == 0) tail_cls_omega(st, R.vals);
@@ -249,8 +254,8 @@ __device__ void solve_classic(const Grp &cl, const SysView &V, SolverState *st, 
                 x[i] = fma(om, a.v[0], fma(al, a.v[1], a.v[2]));
                 const double ri = fma(nom, a.v[3], a.v[4]);
                 r[i] = ri;
-                exact_add<BQ>(w2[0], f2[0], R.acc[0], a.v[5], ri);
-                exact_add<BQ, true>(w2[1], f2[1], R.acc[1], ri, ri);
+                batch_add<false>(w2[0], f2[0], R.acc[0], a.v[5], ri);
+                batch_add<true>(w2[1], f2[1], R.acc[1], ri, ri);
             });
         group_reduce<2>(cl, w2, f2, R);
         if (threadIdx.x == 0) tail_cls_beta(st, R.vals, V.hist);
@@ -294,8 +299,8 @@ __device__ void solve_pipelined(const Grp &cl, const SysView &V, SolverState *st
     group_spmv(V, rh, r0, bad, [&](int64_t i, double wi, double r0i) {
         w[i] = wi;
         wh[i] = __dmul_rn(wi, invd[i]);
-        exact_add<BQ, true>(w2[0], f2[0], R.acc[0], r0i, r0i);
-        exact_add<BQ>(w2[1], f2[1], R.acc[1], r0i, wi);
+        batch_add<true>(w2[0], f2[0], R.acc[0], r0i, r0i);
+        batch_add<false>(w2[1], f2[1], R.acc[1], r0i, wi);
     });
     group_reduce<2>(cl, w2, f2, R);
     if (threadIdx.x == 0) tail_pipe_setup(st, R.vals);
@@ -354,8 +359,8 @@ __device__ void solve_pipelined(const Grp &cl, const SysView &V, SolverState *st
                 qh[i] = qhi;
                 y[i] = yi;
                 zh[i] = __dmul_rn(zi, a.v[5]);
-                exact_add<BQ>(w2[0], f2[0], R.acc[0], qi, yi);
-                exact_add<BQ, true>(w2[1], f2[1], R.acc[1], yi, yi);
+                batch_add<false>(w2[0], f2[0], R.acc[0], qi, yi);
+                batch_add<true>(w2[1], f2[1], R.acc[1], yi, yi);
             });
         group_reduce<2>(cl, w2, f2, R);  // also orders zhat for P2's gathers
         if (threadIdx.x == 0) tail_pipe_omega(st, R.vals);
@@ -380,11 +385,11 @@ __device__ void solve_pipelined(const Grp &cl, const SysView &V, SolverState *st
                 w[i] = wi;
                 wh[i] = __dmul_rn(wi, a.v[9]);
                 const double r0i = a.v[10];
-                exact_add<BQ>(w5[0], f5[0], R.acc[0], r0i, ri);
-                exact_add<BQ>(w5[1], f5[1], R.acc[1], r0i, wi);
-                exact_add<BQ>(w5[2], f5[2], R.acc[2], r0i, a.v[11]);
-                exact_add<BQ>(w5[3], f5[3], R.acc[3], r0i, a.v[12]);
-                exact_add<BQ, true>(w5[4], f5[4], R.acc[4], ri, ri);
+                batch_add<false>(w5[0], f5[0], R.acc[0], r0i, ri);
+                batch_add<false>(w5[1], f5[1], R.acc[1], r0i, wi);
+                batch_add<false>(w5[2], f5[2], R.acc[2], r0i, a.v[11]);
+                batch_add<false>(w5[3], f5[3], R.acc[3], r0i, a.v[12]);
+                batch_add<true>(w5[4], f5[4], R.acc[4], ri, ri);
             });
         group_reduce<5>(cl, w5, f5, R);  // also orders what for P4's gathers
         if (threadIdx.x == 0) tail_pipe_beta(st, R.vals, V.hist);

@@ -171,13 +171,16 @@ __device__ __noinline__ void small_exchange(int K, int b, uint32_t rank) {
 template <int Q>
 __device__ __forceinline__ void small_flush(Win<Q> &W, unsigned long long *acc) {
     constexpr unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
     const bool has = W.a >= 0;
     const int lo = (int)__reduce_min_sync(FULL, (unsigned)(has ? W.a : 0x7fffffff));
     const int hi = (int)__reduce_max_sync(FULL, (unsigned)(has ? W.a : 0));
     if (lo == 0x7fffffff) return;
-    if (lo == hi) warp_sum_words<Q>(W, acc, lane, lo);
-    else win_flush<Q>(W, acc);
+    if (lo == hi) {
+        warp_sum(W.w, acc, lo);
+        win_clear<Q>(W);
+    } else {
+        win_flush<Q>(W, acc);
+    }
 }
 
 // K dots over the cluster, into vals. b: the buffer, flipped here.
