@@ -543,22 +543,19 @@ stalled:
 // word, so the next group of eight is in flight while this one's chain runs,
 // and only the values are staged. What bounds the product then is the FP64 pipe
 // (7 points at 256^3: 117 million fmas, 186 us at two per SM and clock) as much
-// as HBM (K1: 84 bytes per row, 207 us). Measured at 256^3: K1 335 -> 249 us, K3
-// 383 -> 320; the product alone at 192^3 126 -> 98 (FP64 pipe 82 % of the active
-// cycles).
+// as HBM (K1: 84 bytes per row, 207 us). Measured at 256^3: K1 335 -> 235 us, K3
+// 383 -> 268 (with the dots' windows in shared memory); the product alone at 192^3
+// 126 -> 98 (FP64 pipe 82 % of the active cycles).
 //
-// Warps take chunks in tiles: a block runs SPMV_TILE groups of consecutive
-// chunks, one chunk per warp, before it moves on, so that rows that gather the
-// same x lines follow each other on one SM while the grid as a whole sweeps the
-// rows in order (a contiguous share per block would have each x line fetched
-// from HBM again for every plane offset).
+// Warps take chunks round robin over the grid. (Several groups of consecutive
+// chunks in a row per block, so that rows that gather the same x lines follow
+// each other on one SM, measured slower: K1 244 us with two or more, 235 so.)
 //
 // N: most diagonals, in groups of up to eight (7: one group, the next chunk's
 // gathers ahead of this one's chain; 32: four, of which the unused are skipped).
 // Each warp's two staging buffers take 32 N values. Every value span is one bulk
 // copy of whole 16-byte units; the last value of an odd nnz is stored by a
 // lane. Waits are bounded, with the timeout fallback of spmv_rows.
-constexpr int SPMV_TILE = 4;
 template <int N>
 struct DiagLayout {
     static constexpr int PER = N < 8 ? N : 8, G = N / PER;  // diagonals per group, groups
@@ -569,7 +566,6 @@ struct DiagLayout {
     static_assert(BUF % 16 == 0 && SCRATCH >= FLUSH_SCRATCH, "the flush reuses the staging buffers");
 };
 
-//
 // Rows [32 c_begin, n_end) of the chunks [c_begin, c_end), blocks 0 .. nblk - 1
 // (this one is blk) together; off(j): the j-th diagonal, m of them.
 template <int N, class Off, class F>
@@ -592,30 +588,7 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const uint32_t 
     }
     __syncwarp();
     const long long wait_limit = test_stall ? SPMV_TEST_WAIT_LIMIT : SPMV_WAIT_LIMIT;
-    // This warp's c_end in turn: whole rounds of tiles, then chunk by chunk, so
-    // that the last round is even over the blocks. `left`: steps to go in the
-    // tile; c >= c_end: none.
-    const int round = nblk * nw, tiled = c_begin + (c_end - c_begin) / (round * SPMV_TILE) * (round * SPMV_TILE);
-    struct Walk {
-        int c, left;
-    };
-    auto first = [&]() {
-        return tiled > c_begin ? Walk{c_begin + blk * (SPMV_TILE * nw) + wid, SPMV_TILE - 1}
-                               : Walk{c_begin + blk * nw + wid, 0};
-    };
-    auto next = [&](Walk &w) {
-        if (w.left > 0) {
-            w.left--;
-            w.c += nw;
-        } else if (w.c < tiled) {
-            // the next round's tile, or the first chunk after the rounds
-            w.c += (round - nw) * SPMV_TILE + nw;
-            w.left = SPMV_TILE - 1;
-            if (w.c >= tiled) w = Walk{tiled + blk * nw + wid, 0};
-        } else {
-            w.c += round;
-        }
-    };
+    const int round = nblk * nw;
     struct Head {
         long long base;  // the chunk's first nonzero
         uint32_t word;   // this lane's row: its diagonals (N = 7: and where its values start, at bit 8)
@@ -650,26 +623,23 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const uint32_t 
         for (int j = 0; j < PER; j++)
             if ((word >> (g * PER + j)) & 1u) xv[j] = __ldg(x + (row + off(g * PER + j)));
     };
-    Walk w0 = first(), w1 = w0;  // w0: the chunk being computed, w1: the one after
-    next(w1);
-    Head h0 = head(w0.c), h1 = head(w1.c);
+    int c0 = c_begin + blk * nw + wid, c1 = c0 + round;  // the chunk being computed, the one after
+    Head h0 = head(c0), h1 = head(c1);
     unsigned parity = 0u;  // bit b: phase of buffer b's barrier to wait for
     double xa[PER], xb[PER], z0 = 0.0, z1 = 0.0;
     int cur = 0;
-    if (w0.c < c_end) {
+    if (c0 < c_end) {
         stage(h0, 0);
-        gather(w0.c * 32 + lane, h0.word, 0, xa);
-        if (z && w0.c * 32 + lane < n) z0 = __ldg(z + w0.c * 32 + lane);
+        gather(c0 * 32 + lane, h0.word, 0, xa);
+        if (z && c0 * 32 + lane < n) z0 = __ldg(z + c0 * 32 + lane);
     }
     // One chunk: stage the next one's values, then this one's chain. xc, zc hold
     // its first gathers and companion; xn, zn get the next one's (G = 1). Returns
     // false when the wait for the values ran out.
     auto step = [&](int b, double (&xc)[PER], double (&xn)[PER], double &zc, double &zn) {
-        const int row = w0.c * 32 + lane, row1 = w1.c * 32 + lane;
-        if (w1.c < c_end) stage(h1, b ^ 1);
-        Walk w2 = w1;
-        next(w2);
-        const Head h2 = head(w2.c);
+        const int row = c0 * 32 + lane, row1 = c1 * 32 + lane;
+        if (c1 < c_end) stage(h1, b ^ 1);
+        const Head h2 = head(c1 + round);
         int at;  // this row's first value in the chunk
         if (N <= 8) {
             at = (int)(h0.word >> 8);
@@ -721,18 +691,18 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const uint32_t 
         }
         if (row < n) fn((int64_t)row, acc, zr);
         __syncwarp();  // buffer b is refilled in the next step
-        w0 = w1;
-        w1 = w2;
+        c0 = c1;
+        c1 += round;
         h0 = h1;
         h1 = h2;
         return true;
     };
     // two steps per turn (the buffers, and for one group the gathers, swap roles)
     bool ok = true;
-    while (w0.c < c_end) {
+    while (c0 < c_end) {
         cur = 0;
         if (!(ok = step(0, xa, xb, z0, z1))) break;
-        if (w0.c >= c_end) break;
+        if (c0 >= c_end) break;
         cur = 1;
         if (!(ok = G == 1 ? step(1, xb, xa, z1, z0) : step(1, xa, xb, z0, z1))) break;
     }
@@ -741,9 +711,9 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const uint32_t 
     // this and every later row from global memory, then wait (bounded) for the
     // copies in flight.
     err |= ERR_TIMEOUT;
-    const bool more = w1.c < c_end;
-    for (; w0.c < c_end; next(w0)) {
-        const int row = w0.c * 32 + lane;
+    const bool more = c1 < c_end;
+    for (; c0 < c_end; c0 += round) {
+        const int row = c0 * 32 + lane;
         if (row < n) {
             bool bad = false;
             const double acc = spmv_row(A, row, x, bad);
