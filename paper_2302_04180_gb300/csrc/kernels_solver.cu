@@ -373,14 +373,19 @@ static cudaError_t iter_t(const SolverArgs &a, int variant, cudaStream_t s, Kern
 
 // Shared-memory carveout (percent of the unified L1/shared storage, -1 = the
 // driver's choice) of the kernels that stage data per warp. The x gathers of
-// the SpMV live on L1 hits, so the split is a tuning knob, not a maximum.
+// the SpMV live on L1 hits, so the split is a tuning knob, not a maximum: the
+// kernels of short rows take no more than SPMV_SHORT_CARVEOUT of it, those of long
+// rows the driver's choice, which is what their resident blocks need (rows of 2 to
+// 39 random columns, 500000 rows: K1 86 us with all of it, 67 so; K3 93, 75.5; the
+// product alone 83, 69. The 27-point stencil is as fast with either).
 template <class R1, class R2, class V2, class V5>
 static void prefer_shared(int c) {
     for (int mode : {SPMV_MODE_SHORT, SPMV_MODE_LONG, SPMV_MODE_DIAG7, SPMV_MODE_DIAG32})
         with_cap(mode, [&](auto cap) {
             constexpr int CAP = decltype(cap)::value;
-            // the kernels of long rows need (nearly) all of it for their staging buffers
-            const int share = c < 0 || CAP == SPMV_CAP_SHORT || CAP == CAP_DIAG7 ? c : 100;
+            const int share = CAP == CAP_DIAG7 ? c
+                              : CAP != SPMV_CAP_SHORT ? -1
+                              : c > SPMV_SHORT_CARVEOUT ? SPMV_SHORT_CARVEOUT : c;
             cudaFuncSetAttribute(k_cls_k1<R1, CAP>, cudaFuncAttributePreferredSharedMemoryCarveout, share);
             cudaFuncSetAttribute(k_cls_k3<R2, CAP>, cudaFuncAttributePreferredSharedMemoryCarveout, share);
             cudaFuncSetAttribute(k_pipe_setup2<R2, CAP>, cudaFuncAttributePreferredSharedMemoryCarveout, share);

@@ -50,11 +50,6 @@ __global__ void __launch_bounds__(DiagLayout<N>::WARPS * 32, 3)
 
 static CSRView view(const CSRArgs &A) { return CSRView{A.n, A.nnz, A.rowptr, A.col, A.val}; }
 
-// Most percent of the L1/shared storage for k_spmv: what its three blocks per SM
-// take (48 KB each). More would only shrink the L1 that the x gathers live on:
-// 500000 ragged random rows 35.0 us at 75 %, 31.1 at this; Poisson 128^3 and the
-// 27-point stencil are as fast at either.
-constexpr int SPMV_CARVEOUT = 64;
 static void spmv_carveout(int c) {
     static std::mutex mu;
     static int applied[64];
@@ -66,14 +61,14 @@ static void spmv_carveout(int c) {
     }
     int dev = 0;
     if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 && applied[dev] != c) {
-        const int short_c = c > SPMV_CARVEOUT ? SPMV_CARVEOUT : c;
+        const int short_c = c > SPMV_SHORT_CARVEOUT ? SPMV_SHORT_CARVEOUT : c;
         cudaFuncSetAttribute(k_spmv<true, SPMV_CAP_SHORT>, cudaFuncAttributePreferredSharedMemoryCarveout, short_c);
         cudaFuncSetAttribute(k_spmv<false, SPMV_CAP_SHORT>, cudaFuncAttributePreferredSharedMemoryCarveout, short_c);
         cudaFuncSetAttribute(k_spmv_diag<7>, cudaFuncAttributePreferredSharedMemoryCarveout, c);
-        cudaFuncSetAttribute(k_spmv_diag<32>, cudaFuncAttributePreferredSharedMemoryCarveout, c < 0 ? c : 100);
-        // the long-row kernel needs all of it, whatever the knob says
-        cudaFuncSetAttribute(k_spmv_reg<true>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-        cudaFuncSetAttribute(k_spmv_reg<false>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        // the kernels of long rows: what their blocks need, whatever the knob says
+        cudaFuncSetAttribute(k_spmv_diag<32>, cudaFuncAttributePreferredSharedMemoryCarveout, -1);
+        cudaFuncSetAttribute(k_spmv_reg<true>, cudaFuncAttributePreferredSharedMemoryCarveout, -1);
+        cudaFuncSetAttribute(k_spmv_reg<false>, cudaFuncAttributePreferredSharedMemoryCarveout, -1);
         cudaGetLastError();
         applied[dev] = c;
     }

@@ -42,6 +42,11 @@ struct DiagArgs {
 // mode of its bounded wait (kernels.cuh).
 enum : int { SPMV_MODE_ROW = 1, SPMV_MODE_SHORT = 2, SPMV_MODE_LONG = 3, SPMV_MODE_DIAG7 = 4, SPMV_MODE_DIAG32 = 5,
              SPMV_MODE_MASK = 0xff, SPMV_TEST_STALL = 0x100 };
+// Most percent of the L1/shared storage for the kernels that stage short rows:
+// what their three blocks per SM take (48 to 50 KB each). More would only shrink
+// the L1 that the x gathers live on: 500000 ragged random rows 35.0 us at 75 %,
+// 31.1 at this (K1 36.7, 35.1); Poisson 128^3 is as fast at either.
+constexpr int SPMV_SHORT_CARVEOUT = 64;
 // Long rows run register-staged in blocks of SPMV_REG_WARPS warps: the
 // standalone SpMV, and the classic loop's fused K1/K3.
 constexpr int SPMV_REG_WARPS = 4;
