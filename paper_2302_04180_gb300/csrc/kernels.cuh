@@ -621,7 +621,7 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const uint32_t 
     auto gather = [&](int row, uint32_t word, int g, double (&xv)[PER]) {
 #pragma unroll
         for (int j = 0; j < PER; j++)
-            if ((word >> (g * PER + j)) & 1u) xv[j] = __ldg(x + (row + off(g * PER + j)));
+            if ((word >> (g * PER + j)) & 1u) xv[j] = __ldca(x + (row + off(g * PER + j)));
     };
     int c0 = c_begin + blk * nw + wid, c1 = c0 + round;  // the chunk being computed, the one after
     Head h0 = head(c0), h1 = head(c1);
@@ -631,7 +631,7 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const uint32_t 
     if (c0 < c_end) {
         stage(h0, 0);
         gather(c0 * 32 + lane, h0.word, 0, xa);
-        if (z && c0 * 32 + lane < n) z0 = __ldg(z + c0 * 32 + lane);
+        if (z && c0 * 32 + lane < n) z0 = __ldca(z + c0 * 32 + lane);
     }
     // One chunk: stage the next one's values, then this one's chain. xc, zc hold
     // its first gathers and companion; xn, zn get the next one's (G = 1). Returns
@@ -656,7 +656,7 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const uint32_t 
         const double *val = reinterpret_cast<const double *>(bufs + b * L::BUF) + ((int)(h0.base & 1) + at);
         auto next_gather = [&](double (&xv)[PER], double &zv) {
             gather(row1, h1.word, 0, xv);
-            if (z && row1 < n) zv = __ldg(z + row1);
+            if (z && row1 < n) zv = __ldca(z + row1);
         };
         if (G == 1) next_gather(xn, zn);
         {
@@ -716,7 +716,7 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const uint32_t 
         const int row = c0 * 32 + lane;
         if (row < n) {
             bool bad = false;
-            const double acc = spmv_row(A, row, x, bad);
+            const double acc = spmv_row<true>(A, row, x, bad);
             if (bad) err |= ERR_INDEX;
             fn((int64_t)row, acc, z ? z[row] : 0.0);
         }

@@ -108,10 +108,12 @@ __device__ __forceinline__ void fused_spmv(const Ctx &c, const double *x, const 
 // K1: s = A phat, <r0, s>
 template <class R, int CAP>
 __global__ void __launch_bounds__(FusedScratch<CAP>::THREADS, 3) k_cls_k1(Ctx c) {
+    typename FusedDot<R, CAP>::type red;
+    red.init();
+    chain_wait();
     StateCopy sc;
     sc.load(c.st);
-    typename FusedDot<R, CAP>::type red;
-    red.init();  // ends in a barrier
+    __syncthreads();
     if (sc.copy->done) return;
     unsigned eb = 0u;
     fused_spmv<CAP>(c, c.ph, c.r0, eb, [&](int64_t i, double si, double r0) {
@@ -128,6 +130,7 @@ __global__ void __launch_bounds__(FusedScratch<CAP>::THREADS, 3) k_cls_k1(Ctx c)
 // occupancy sizes the vector grid: left free, the compiler took 80 registers, three
 // blocks fit and the grid ran in 1.33 waves.
 __global__ void __launch_bounds__(256, 4) k_cls_k2(Ctx c) {
+    chain_wait();
     if (c.st->done) return;
     const double na = -c.st->alpha;
     for_pairs(c.n, [&](int64_t i, bool pair) {
@@ -147,10 +150,12 @@ __global__ void __launch_bounds__(256, 4) k_cls_k2(Ctx c) {
 // K3: y = A qhat, <q, y>, <y, y>
 template <class R, int CAP>
 __global__ void __launch_bounds__(FusedScratch<CAP>::THREADS, 3) k_cls_k3(Ctx c) {
+    typename FusedDot<R, CAP>::type red;
+    red.init();
+    chain_wait();
     StateCopy sc;
     sc.load(c.st);
-    typename FusedDot<R, CAP>::type red;
-    red.init();  // ends in a barrier
+    __syncthreads();
     if (sc.copy->done) return;
     unsigned eb = 0u;
     fused_spmv<CAP>(c, c.qh, c.q, eb, [&](int64_t i, double yi, double qi) {
@@ -167,10 +172,12 @@ __global__ void __launch_bounds__(FusedScratch<CAP>::THREADS, 3) k_cls_k3(Ctx c)
 // K4: x = fma(omega, qhat, fma(alpha, phat, x)), r = fma(-omega, y, q), <r0,r>, <r,r>
 template <class R>
 __global__ void __launch_bounds__(256, 4) k_cls_k4(Ctx c) {
+    R red;
+    red.init();
+    chain_wait();
     StateCopy sc;
     sc.load(c.st);
-    R red;
-    red.init();  // ends in a barrier
+    __syncthreads();
     if (sc.copy->done) return;
     cls_k4_pairs(c, red, sc.copy->alpha, sc.copy->omega, gtid(), c.n >> 1, gstride(),
                  (c.n & 1) && gtid() == 0 ? c.n - 1 : -1);
@@ -180,6 +187,7 @@ __global__ void __launch_bounds__(256, 4) k_cls_k4(Ctx c) {
 
 // K5: p = fma(beta, fma(-omega, s, p), r), phat = p * invd
 __global__ void __launch_bounds__(256) k_cls_k5(Ctx c) {
+    chain_wait();
     if (c.st->done) return;
     const double be = c.st->beta, nom = -c.st->omega;
     for_pairs(c.n, [&](int64_t i, bool pair) {
@@ -239,10 +247,12 @@ template <int K> struct P1Cfg<PlainR<K>> { static constexpr int blocks = 4, pair
 // not restrict-qualified, so later loads could not be issued early).
 template <class R>
 __global__ void __launch_bounds__(256, P1Cfg<R>::blocks) k_pipe_p1(Ctx c) {
+    R red;
+    red.init();
+    chain_wait();
     StateCopy sc;
     sc.load(c.st);
-    R red;
-    red.init();  // ends in a barrier
+    __syncthreads();
     if (sc.copy->done) return;
     const double al = sc.copy->alpha, nal = -al, be = sc.copy->beta, nom = -sc.copy->omega;
     const bool first = sc.copy->iter == 0;
@@ -266,10 +276,12 @@ template <int K> struct P3Cfg<PlainR<K>> { static constexpr int blocks = 3, pair
 // not restrict-qualified, so later loads could not be issued early).
 template <class R>
 __global__ void __launch_bounds__(256, P3Cfg<R>::blocks) k_pipe_p3(Ctx c) {
+    R red;
+    red.init();
+    chain_wait();
     StateCopy sc;
     sc.load(c.st);
-    R red;
-    red.init();  // ends in a barrier
+    __syncthreads();
     if (sc.copy->done) return;
     const double al = sc.copy->alpha, nal = -al, om = sc.copy->omega, nom = -om;
     if (P3Cfg<R>::pairs) {
@@ -329,8 +341,8 @@ static bool diag_mode(int mode) {
 }
 
 // y = A x without a dot (pipelined S10, S18 and set-up).
-static cudaError_t plain_spmv(const SolverArgs &a, const double *x, double *y, cudaStream_t s) {
-    if (diag_mode(a.spmv.mode)) return launch_spmv_diag(a.A, a.D, x, y, a.st, a.err, a.spmv, s);
+static cudaError_t plain_spmv(const SolverArgs &a, const double *x, double *y, cudaStream_t s, bool chain = false) {
+    if (diag_mode(a.spmv.mode)) return launch_spmv_diag(a.A, a.D, x, y, a.st, a.err, a.spmv, chain, s);
     return launch_spmv(a.A, x, y, a.st, a.err, a.spmv, s);
 }
 
@@ -352,21 +364,27 @@ static cudaError_t setup_t(const SolverArgs &a, int variant, cudaStream_t s, Ker
 template <class R1, class R2, class V2, class V5>
 static cudaError_t iter_t(const SolverArgs &a, int variant, cudaStream_t s, KernelTimer *tm) {
     Ctx c = make_ctx(a);
+    // general products are launched as usual: they read x through the read-only path
+    const bool diags = diag_mode(a.spmv.mode);
+    const auto go = [&](bool chain, auto kern, Cfg g) {
+        if (chain && !tm) launch_chained(kern, g.grid, g.block, s, c);
+        else kern<<<g.grid, g.block, 0, s>>>(c);
+    };
     if (variant == RBS_CLASSIC) {
         with_cap(a.spmv.mode, [&](auto cap) {
-            TIMED(PK_K1, (k_cls_k1<R1, decltype(cap)::value><<<a.spmv.grid, a.spmv.block, 0, s>>>(c)));
+            TIMED(PK_K1, (go(diags, k_cls_k1<R1, decltype(cap)::value>, a.spmv)));
         });
-        TIMED(PK_VEC, (k_cls_k2<<<a.vec.grid, a.vec.block, 0, s>>>(c)));
+        TIMED(PK_VEC, (go(true, k_cls_k2, a.vec)));
         with_cap(a.spmv.mode, [&](auto cap) {
-            TIMED(PK_K3, (k_cls_k3<R2, decltype(cap)::value><<<a.k3.grid, a.k3.block, 0, s>>>(c)));
+            TIMED(PK_K3, (go(diags, k_cls_k3<R2, decltype(cap)::value>, a.k3)));
         });
-        TIMED(PK_K4, (k_cls_k4<V2><<<a.vec.grid, a.vec.block, 0, s>>>(c)));
-        TIMED(PK_VEC, (k_cls_k5<<<a.vec.grid, a.vec.block, 0, s>>>(c)));
+        TIMED(PK_K4, (go(true, k_cls_k4<V2>, a.vec)));
+        TIMED(PK_VEC, (go(true, k_cls_k5, a.vec)));
     } else {
-        TIMED(PK_VEC_DOT, (k_pipe_p1<V2><<<a.vec.grid, a.vec.block, 0, s>>>(c)));
-        TIMED(PK_SPMV, (plain_spmv(a, a.v.zh, a.v.v, s)));
-        TIMED(PK_VEC_DOT, (k_pipe_p3<V5><<<a.p3.grid, a.p3.block, 0, s>>>(c)));
-        TIMED(PK_SPMV, (plain_spmv(a, a.v.wh, a.v.t, s)));
+        TIMED(PK_VEC_DOT, (go(true, k_pipe_p1<V2>, a.vec)));
+        TIMED(PK_SPMV, (plain_spmv(a, a.v.zh, a.v.v, s, !tm)));
+        TIMED(PK_VEC_DOT, (go(true, k_pipe_p3<V5>, a.p3)));
+        TIMED(PK_SPMV, (plain_spmv(a, a.v.wh, a.v.t, s, !tm)));
     }
     return cudaGetLastError();
 }

@@ -39,8 +39,9 @@ __global__ void __launch_bounds__(SPMV_REG_WARPS * 32, 3)
 // y = A x for a matrix laid out by its diagonals (a solver's product).
 template <int N>
 __global__ void __launch_bounds__(DiagLayout<N>::WARPS * 32, 3)
-    k_spmv_diag(CSRView A, const __grid_constant__ DiagArgs D, const double *__restrict__ x, double *__restrict__ y,
+    k_spmv_diag(CSRView A, const __grid_constant__ DiagArgs D, const double *x, double *y,
                 const SolverState *st, unsigned *err, int mode) {
+    chain_wait();
     if (st->done) return;
     unsigned eb = 0u;
     spmv_grid_diag<N>(A, D, x, nullptr, (mode & SPMV_TEST_STALL) != 0, eb,
@@ -140,11 +141,10 @@ cudaError_t launch_spmv(const CSRArgs &A, const double *x, double *y, const Solv
 }
 
 cudaError_t launch_spmv_diag(const CSRArgs &A, const DiagArgs &D, const double *x, double *y, const SolverState *st,
-                             unsigned *err, Cfg cfg, cudaStream_t s) {
-    if ((cfg.mode & SPMV_MODE_MASK) == SPMV_MODE_DIAG32)
-        k_spmv_diag<32><<<cfg.grid, cfg.block, 0, s>>>(view(A), D, x, y, st, err, cfg.mode);
-    else
-        k_spmv_diag<7><<<cfg.grid, cfg.block, 0, s>>>(view(A), D, x, y, st, err, cfg.mode);
+                             unsigned *err, Cfg cfg, bool chain, cudaStream_t s) {
+    const auto kern = (cfg.mode & SPMV_MODE_MASK) == SPMV_MODE_DIAG32 ? k_spmv_diag<32> : k_spmv_diag<7>;
+    if (chain) return launch_chained(kern, cfg.grid, cfg.block, s, view(A), D, x, y, st, err, cfg.mode);
+    kern<<<cfg.grid, cfg.block, 0, s>>>(view(A), D, x, y, st, err, cfg.mode);
     return cudaGetLastError();
 }
 

@@ -47,6 +47,25 @@ enum : int { SPMV_MODE_ROW = 1, SPMV_MODE_SHORT = 2, SPMV_MODE_LONG = 3, SPMV_MO
 // the L1 that the x gathers live on: 500000 ragged random rows 35.0 us at 75 %,
 // 31.1 at this (K1 36.7, 35.1); Poisson 128^3 is as fast at either.
 constexpr int SPMV_SHORT_CARVEOUT = 64;
+// Launch `kern`, which calls chain_wait() (common.cuh), so that it may be set up and
+// clear its shared memory while the kernel before it in the stream ends: 0.5 to 1 us
+// less per iteration of a solver (40^3 rows, 20 iterations: 768 -> 748 us; 64^3 1014
+// -> 996). The blocks start once the earlier kernel's have all left. Letting them in
+// earlier (griddepcontrol.launch_dependents) costs more than it hides: at the
+// kernel's start 40^3 865 us and 160^3 6 % more, before its flush between the two.
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kern)(P...), int grid, int block, cudaStream_t s, A &&...args) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
+}
 // Long rows run register-staged in blocks of SPMV_REG_WARPS warps: the
 // standalone SpMV, and the classic loop's fused K1/K3.
 constexpr int SPMV_REG_WARPS = 4;
@@ -107,7 +126,7 @@ cudaError_t launch_spmv(const CSRArgs &A, const double *x, double *y, const Solv
                         unsigned *err, Cfg cfg, cudaStream_t s);
 // The same product of a solver on a matrix laid out by its diagonals.
 cudaError_t launch_spmv_diag(const CSRArgs &A, const DiagArgs &D, const double *x, double *y, const SolverState *st,
-                             unsigned *err, Cfg cfg, cudaStream_t s);
+                             unsigned *err, Cfg cfg, bool chain, cudaStream_t s);
 cudaError_t launch_jacobi_invd(const CSRArgs &A, const double *diag, double *invd, unsigned *err,
                                Cfg cfg, cudaStream_t s);
 cudaError_t launch_jacobi_apply(int64_t n, const double *invd, const double *p, double *phat, Cfg cfg,
