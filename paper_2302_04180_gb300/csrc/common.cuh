@@ -37,11 +37,17 @@ struct SolverState {
     int32_t iter, maxit, done, status, converged, variant, hist_cap, loops;
 };
 
-// In a kernel of a chain (launch_chained, launch.h): returns once the kernel before
-// it is complete and its stores are visible; nothing in a kernel launched as usual.
-// Nothing that an earlier kernel writes is touched before it, or through the
-// read-only path at all (a load there may count as valid for the whole kernel).
-__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+// In a kernel launched by launch_chained (launch.h): returns once the work before
+// it is complete and its stores are visible, to asynchronous copies too; nothing in
+// a kernel launched as usual. Nothing that earlier work writes is touched before
+// it, or through the read-only path at all (a load there may count as valid for
+// the whole kernel).
+__device__ __forceinline__ void chain_wait() {
+    asm volatile(
+        "griddepcontrol.wait;\n\t"
+        "fence.proxy.async.global;\n" ::
+            : "memory");
+}
 
 __device__ __forceinline__ double qnan() { return __longlong_as_double(0x7ff8000000000000ll); }
 

@@ -34,7 +34,7 @@ __device__ __forceinline__ double spmv_row(const CSRView &A, int64_t i, const do
             bad = true;
             continue;
         }
-        acc = fma(A.val[k], L2X ? __ldcg(x + c) : __ldg(x + c), acc);
+        acc = fma(A.val[k], L2X ? __ldcg(x + c) : __ldca(x + c), acc);
     }
     return acc;
 }
@@ -302,9 +302,9 @@ __device__ __forceinline__ void spmv_rows(const CSRView &A, int64_t r_begin, int
                                 // a bad column is reported and its gather clamped
                                 // into range (the call fails; the value is moot)
                                 cmax = max(cmax, cidx);
-                                xv[j] = L2X ? __ldcg(x + min(cidx, ncol - 1u)) : __ldg(x + min(cidx, ncol - 1u));
+                                xv[j] = L2X ? __ldcg(x + min(cidx, ncol - 1u)) : __ldca(x + min(cidx, ncol - 1u));
                             } else {
-                                xv[j] = L2X ? __ldcg(x + cidx) : __ldg(x + cidx);
+                                xv[j] = L2X ? __ldcg(x + cidx) : __ldca(x + cidx);
                             }
                         }
                     }
@@ -452,9 +452,9 @@ __device__ __forceinline__ void spmv_rows_reg(const CSRView &A, int64_t r_begin,
                         const unsigned cidx = (unsigned)scol[k];
                         if (CHECKED) {
                             cmax = max(cmax, cidx);
-                            xv[j] = L2X ? __ldcg(x + min(cidx, ncol - 1u)) : __ldg(x + min(cidx, ncol - 1u));
+                            xv[j] = L2X ? __ldcg(x + min(cidx, ncol - 1u)) : __ldca(x + min(cidx, ncol - 1u));
                         } else {
-                            xv[j] = L2X ? __ldcg(x + cidx) : __ldg(x + cidx);
+                            xv[j] = L2X ? __ldcg(x + cidx) : __ldca(x + cidx);
                         }
                         vv[j] = sval[k];
                     }
@@ -472,7 +472,7 @@ __device__ __forceinline__ void spmv_rows_reg(const CSRView &A, int64_t r_begin,
                         const unsigned cidx = (unsigned)scol[k];
                         if (CHECKED) cmax = max(cmax, cidx);
                         const unsigned c = CHECKED ? min(cidx, ncol - 1u) : cidx;
-                        acc = fma(sval[k], L2X ? __ldcg(x + c) : __ldg(x + c), acc);
+                        acc = fma(sval[k], L2X ? __ldcg(x + c) : __ldca(x + c), acc);
                     }
                     if (CHECKED && len > 0 && cmax >= ncol) err |= ERR_INDEX;
                     if (z) zr = reinterpret_cast<const double *>(buf)[lane];
@@ -716,7 +716,7 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const uint32_t 
         const int row = c0 * 32 + lane;
         if (row < n) {
             bool bad = false;
-            const double acc = spmv_row<true>(A, row, x, bad);
+            const double acc = spmv_row(A, row, x, bad);
             if (bad) err |= ERR_INDEX;
             fn((int64_t)row, acc, z ? z[row] : 0.0);
         }

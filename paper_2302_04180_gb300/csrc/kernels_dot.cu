@@ -52,7 +52,9 @@ __global__ void __launch_bounds__(256, EXDOT_BLOCKS)
     using R = ExactRows<1, W, true>;
     R red;
     const int slot = EXPORT ? 0 : blockIdx.y;
-    const double *__restrict__ xp = a.x[slot], *__restrict__ yp = a.y[slot];
+    const double *xp = a.x[slot], *yp = a.y[slot];
+    red.init();
+    chain_wait();
     const int64_t st = gstride();
     if (((reinterpret_cast<uintptr_t>(xp) | reinterpret_cast<uintptr_t>(yp)) & 15) == 0) {
         constexpr int U = EXDOT_PAIRS;
@@ -79,7 +81,6 @@ __global__ void __launch_bounds__(256, EXDOT_BLOCKS)
             }
         };
         if (full > 0) load(xa, ya);
-        red.init();
         red.open({max(R::limb_of(x0[0].x, y0[0].x), R::limb_of(x0[0].y, y0[0].y))});
         add_pairs<1>(red, x0, y0);
         int64_t s = 0;
@@ -104,7 +105,6 @@ __global__ void __launch_bounds__(256, EXDOT_BLOCKS)
         if ((n & 1) && gtid() == 0) red.add(0, xp[n - 1], yp[n - 1]);
     } else {
         int64_t i = gtid();
-        red.init();
         red.open({i < n ? R::limb_of(xp[i], yp[i]) : -1});
         for (; i < n; i += st) red.add(0, xp[i], yp[i]);
     }
@@ -145,8 +145,8 @@ cudaError_t launch_exdot(int k, const double *const *xs, const double *const *ys
         a.y[j] = ys[j];
     }
     return with_window(window, [&](auto kern) {
-        kern<<<dim3((unsigned)cfg.grid, (unsigned)k), cfg.block, 0, s>>>(a, n, g, out, nullptr, nullptr);
-        return cudaGetLastError();
+        return launch_chained(kern, dim3((unsigned)cfg.grid, (unsigned)k), cfg.block, s, a, n, g, out,
+                              (long long *)nullptr, (int32_t *)nullptr);
     });
 }
 
@@ -155,8 +155,8 @@ cudaError_t launch_exdot_partial(const double *x, const double *y, int64_t n, Do
     DotArgs a{};
     a.x[0] = x;
     a.y[0] = y;
-    k_exdot<16, true><<<cfg.grid, cfg.block, 0, s>>>(a, n, g, nullptr, (long long *)limbs, flags);
-    return cudaGetLastError();
+    return launch_chained(k_exdot<16, true>, dim3((unsigned)cfg.grid), cfg.block, s, a, n, g, (double *)nullptr,
+                          (long long *)limbs, flags);
 }
 
 __global__ void k_round_limbs(const int64_t *limbs, const int32_t *flags, double *out) {

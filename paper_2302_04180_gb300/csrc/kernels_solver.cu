@@ -341,8 +341,8 @@ static bool diag_mode(int mode) {
 }
 
 // y = A x without a dot (pipelined S10, S18 and set-up).
-static cudaError_t plain_spmv(const SolverArgs &a, const double *x, double *y, cudaStream_t s, bool chain = false) {
-    if (diag_mode(a.spmv.mode)) return launch_spmv_diag(a.A, a.D, x, y, a.st, a.err, a.spmv, chain, s);
+static cudaError_t plain_spmv(const SolverArgs &a, const double *x, double *y, cudaStream_t s) {
+    if (diag_mode(a.spmv.mode)) return launch_spmv_diag(a.A, a.D, x, y, a.st, a.err, a.spmv, s);
     return launch_spmv(a.A, x, y, a.st, a.err, a.spmv, s);
 }
 
@@ -364,27 +364,22 @@ static cudaError_t setup_t(const SolverArgs &a, int variant, cudaStream_t s, Ker
 template <class R1, class R2, class V2, class V5>
 static cudaError_t iter_t(const SolverArgs &a, int variant, cudaStream_t s, KernelTimer *tm) {
     Ctx c = make_ctx(a);
-    // general products are launched as usual: they read x through the read-only path
-    const bool diags = diag_mode(a.spmv.mode);
-    const auto go = [&](bool chain, auto kern, Cfg g) {
-        if (chain && !tm) launch_chained(kern, g.grid, g.block, s, c);
-        else kern<<<g.grid, g.block, 0, s>>>(c);
-    };
+    const auto go = [&](auto kern, Cfg g) { launch_chained(kern, dim3((unsigned)g.grid), g.block, s, c); };
     if (variant == RBS_CLASSIC) {
         with_cap(a.spmv.mode, [&](auto cap) {
-            TIMED(PK_K1, (go(diags, k_cls_k1<R1, decltype(cap)::value>, a.spmv)));
+            TIMED(PK_K1, (go(k_cls_k1<R1, decltype(cap)::value>, a.spmv)));
         });
-        TIMED(PK_VEC, (go(true, k_cls_k2, a.vec)));
+        TIMED(PK_VEC, (go(k_cls_k2, a.vec)));
         with_cap(a.spmv.mode, [&](auto cap) {
-            TIMED(PK_K3, (go(diags, k_cls_k3<R2, decltype(cap)::value>, a.k3)));
+            TIMED(PK_K3, (go(k_cls_k3<R2, decltype(cap)::value>, a.k3)));
         });
-        TIMED(PK_K4, (go(true, k_cls_k4<V2>, a.vec)));
-        TIMED(PK_VEC, (go(true, k_cls_k5, a.vec)));
+        TIMED(PK_K4, (go(k_cls_k4<V2>, a.vec)));
+        TIMED(PK_VEC, (go(k_cls_k5, a.vec)));
     } else {
-        TIMED(PK_VEC_DOT, (go(true, k_pipe_p1<V2>, a.vec)));
-        TIMED(PK_SPMV, (plain_spmv(a, a.v.zh, a.v.v, s, !tm)));
-        TIMED(PK_VEC_DOT, (go(true, k_pipe_p3<V5>, a.p3)));
-        TIMED(PK_SPMV, (plain_spmv(a, a.v.wh, a.v.t, s, !tm)));
+        TIMED(PK_VEC_DOT, (go(k_pipe_p1<V2>, a.vec)));
+        TIMED(PK_SPMV, (plain_spmv(a, a.v.zh, a.v.v, s)));
+        TIMED(PK_VEC_DOT, (go(k_pipe_p3<V5>, a.p3)));
+        TIMED(PK_SPMV, (plain_spmv(a, a.v.wh, a.v.t, s)));
     }
     return cudaGetLastError();
 }

@@ -16,6 +16,7 @@ template <bool CHECKED, int CAP>
 __global__ void __launch_bounds__(256, 3)
     k_spmv(CSRView A, const double *__restrict__ x, double *__restrict__ y, const SolverState *st, unsigned *err,
            int mode) {
+    chain_wait();
     if (st && st->done) return;
     unsigned eb = 0u;
     spmv_each<CHECKED, CAP>(A, x, nullptr, mode, eb, [&](int64_t i, double v, double) { y[i] = v; });
@@ -28,6 +29,7 @@ template <bool CHECKED>
 __global__ void __launch_bounds__(SPMV_REG_WARPS * 32, 3)
     k_spmv_reg(CSRView A, const double *__restrict__ x, double *__restrict__ y, const SolverState *st,
                unsigned *err, int mode) {
+    chain_wait();
     if (st && st->done) return;
     unsigned eb = 0u;
     spmv_rows_reg<CHECKED, SPMV_CAP_LONG, false>(
@@ -130,22 +132,17 @@ cudaError_t launch_spmv(const CSRArgs &A, const double *x, double *y, const Solv
     spmv_carveout(cfg.carveout);
     if ((cfg.mode & SPMV_MODE_MASK) == SPMV_MODE_LONG) {
         const Cfg r = spmv_reg_cfg(A.n, cfg.carveout);
-        if (st) k_spmv_reg<false><<<r.grid, r.block, 0, s>>>(view(A), x, y, st, err, cfg.mode);
-        else k_spmv_reg<true><<<r.grid, r.block, 0, s>>>(view(A), x, y, st, err, cfg.mode);
-    } else if (st) {
-        k_spmv<false, SPMV_CAP_SHORT><<<cfg.grid, cfg.block, 0, s>>>(view(A), x, y, st, err, cfg.mode);
-    } else {
-        k_spmv<true, SPMV_CAP_SHORT><<<cfg.grid, cfg.block, 0, s>>>(view(A), x, y, st, err, cfg.mode);
+        return launch_chained(st ? k_spmv_reg<false> : k_spmv_reg<true>, dim3((unsigned)r.grid), r.block, s, view(A), x,
+                              y, st, err, cfg.mode);
     }
-    return cudaGetLastError();
+    return launch_chained(st ? k_spmv<false, SPMV_CAP_SHORT> : k_spmv<true, SPMV_CAP_SHORT>, dim3((unsigned)cfg.grid),
+                          cfg.block, s, view(A), x, y, st, err, cfg.mode);
 }
 
 cudaError_t launch_spmv_diag(const CSRArgs &A, const DiagArgs &D, const double *x, double *y, const SolverState *st,
-                             unsigned *err, Cfg cfg, bool chain, cudaStream_t s) {
+                             unsigned *err, Cfg cfg, cudaStream_t s) {
     const auto kern = (cfg.mode & SPMV_MODE_MASK) == SPMV_MODE_DIAG32 ? k_spmv_diag<32> : k_spmv_diag<7>;
-    if (chain) return launch_chained(kern, cfg.grid, cfg.block, s, view(A), D, x, y, st, err, cfg.mode);
-    kern<<<cfg.grid, cfg.block, 0, s>>>(view(A), D, x, y, st, err, cfg.mode);
-    return cudaGetLastError();
+    return launch_chained(kern, dim3((unsigned)cfg.grid), cfg.block, s, view(A), D, x, y, st, err, cfg.mode);
 }
 
 // invd_i = RN(1 / d_i) with d the given diagonal or the first stored (i, i)

@@ -48,18 +48,22 @@ enum : int { SPMV_MODE_ROW = 1, SPMV_MODE_SHORT = 2, SPMV_MODE_LONG = 3, SPMV_MO
 // 31.1 at this (K1 36.7, 35.1); Poisson 128^3 is as fast at either.
 constexpr int SPMV_SHORT_CARVEOUT = 64;
 // Launch `kern`, which calls chain_wait() (common.cuh), so that it may be set up and
-// clear its shared memory while the kernel before it in the stream ends: 0.5 to 1 us
-// less per iteration of a solver (40^3 rows, 20 iterations: 768 -> 748 us; 64^3 1014
-// -> 996). The blocks start once the earlier kernel's have all left. Letting them in
-// earlier (griddepcontrol.launch_dependents) costs more than it hides: at the
-// kernel's start 40^3 865 us and 160^3 6 % more, before its flush between the two.
+// clear its shared memory while the kernel before it in the stream, whosever it
+// is, ends. Without it the GPU idles 2 us between two kernels, as long as a dot of
+// a million elements takes from HBM: SpMV of Poisson 128^3 42.2 -> 39.8 us, of 500000
+// ragged rows 29.6 -> 27.5, dots of 2^24 55.4 -> 52.9, five of 2^21 32.9 -> 30.5,
+// and 0.5 to 1 us less per iteration of a solver (40^3 rows, 20 iterations: 768 ->
+// 748 us; 64^3 1014 -> 996). The blocks start once the earlier kernel's have all left.
+// Letting them in before (griddepcontrol.launch_dependents) costs more than it
+// hides: at the start of a solver's kernels 40^3 865 us and 160^3 6 % more, before
+// their flush between the two.
 template <class... P, class... A>
-cudaError_t launch_chained(void (*kern)(P...), int grid, int block, cudaStream_t s, A &&...args) {
+cudaError_t launch_chained(void (*kern)(P...), dim3 grid, int block, cudaStream_t s, A &&...args) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3((unsigned)grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)block);
     cfg.stream = s;
     cfg.attrs = &at;
@@ -126,7 +130,7 @@ cudaError_t launch_spmv(const CSRArgs &A, const double *x, double *y, const Solv
                         unsigned *err, Cfg cfg, cudaStream_t s);
 // The same product of a solver on a matrix laid out by its diagonals.
 cudaError_t launch_spmv_diag(const CSRArgs &A, const DiagArgs &D, const double *x, double *y, const SolverState *st,
-                             unsigned *err, Cfg cfg, bool chain, cudaStream_t s);
+                             unsigned *err, Cfg cfg, cudaStream_t s);
 cudaError_t launch_jacobi_invd(const CSRArgs &A, const double *diag, double *invd, unsigned *err,
                                Cfg cfg, cudaStream_t s);
 cudaError_t launch_jacobi_apply(int64_t n, const double *invd, const double *p, double *phat, Cfg cfg,
