@@ -157,12 +157,14 @@ __global__ void __launch_bounds__(256) k_step_cls_setup(const Ctx *ctxs, const S
 
 template <bool DIAG>
 __device__ __forceinline__ void step_k1(const Ctx *ctxs, const StepTask *tasks) {
+    StepDot<1, DIAG> red;
+    red.init();
+    chain_wait();
     const StepTask t = tasks[blockIdx.x];
     const Ctx c = ctxs[t.sys];
     StateCopy sc;
     sc.load(c.st);
-    StepDot<1, DIAG> red;
-    red.init();  // ends in a barrier
+    __syncthreads();
     if (sc.copy->done) return;
     unsigned eb = 0u;
     step_spmv<DIAG>(ctxs, c, t, c.ph, c.r0, eb, [&](int64_t i, double si, double r0) {
@@ -179,6 +181,7 @@ __global__ void __launch_bounds__(256, 3) k_step_cls_k1(const Ctx *ctxs, const S
 __global__ void __launch_bounds__(256, 3) k_step_diag_k1(const Ctx *ctxs, const StepTask *tasks) { step_k1<true>(ctxs, tasks); }
 
 __global__ void __launch_bounds__(256) k_step_cls_k2(const Ctx *ctxs, const StepTask *tasks) {
+    chain_wait();
     const StepTask t = tasks[blockIdx.x];
     const Ctx c = ctxs[t.sys];
     if (c.st->done) return;
@@ -199,12 +202,14 @@ __global__ void __launch_bounds__(256) k_step_cls_k2(const Ctx *ctxs, const Step
 
 template <bool DIAG>
 __device__ __forceinline__ void step_k3(const Ctx *ctxs, const StepTask *tasks) {
+    StepDot<2, DIAG> red;
+    red.init();
+    chain_wait();
     const StepTask t = tasks[blockIdx.x];
     const Ctx c = ctxs[t.sys];
     StateCopy sc;
     sc.load(c.st);
-    StepDot<2, DIAG> red;
-    red.init();  // ends in a barrier
+    __syncthreads();
     if (sc.copy->done) return;
     unsigned eb = 0u;
     step_spmv<DIAG>(ctxs, c, t, c.qh, c.q, eb, [&](int64_t i, double yi, double qi) {
@@ -223,12 +228,14 @@ __global__ void __launch_bounds__(256, 3) k_step_diag_k3(const Ctx *ctxs, const 
 
 template <class R>
 __global__ void __launch_bounds__(256, 4) k_step_cls_k4(const Ctx *ctxs, const StepTask *tasks) {
+    R red;
+    red.init();
+    chain_wait();
     const StepTask t = tasks[blockIdx.x];
     const Ctx c = ctxs[t.sys];
     StateCopy sc;
     sc.load(c.st);
-    R red;
-    red.init();  // ends in a barrier
+    __syncthreads();
     if (sc.copy->done) return;
     cls_k4_pairs(c, red, sc.copy->alpha, sc.copy->omega, (t.lo >> 1) + threadIdx.x, t.hi >> 1, blockDim.x, seg_odd(t));
     __shared__ double vals[R::K];
@@ -236,6 +243,7 @@ __global__ void __launch_bounds__(256, 4) k_step_cls_k4(const Ctx *ctxs, const S
 }
 
 __global__ void __launch_bounds__(256) k_step_cls_k5(const Ctx *ctxs, const StepTask *tasks) {
+    chain_wait();
     const StepTask t = tasks[blockIdx.x];
     const Ctx c = ctxs[t.sys];
     if (c.st->done) return;
@@ -290,6 +298,7 @@ __global__ void __launch_bounds__(256, 3) k_step_pipe_setup2(const Ctx *ctxs, co
 // y = A x without a dot: the pipelined S10 (v = A zhat) and S18 / set-up (t = A what)
 template <bool TO_V, bool DIAG>
 __global__ void __launch_bounds__(256, 3) k_step_spmv(const Ctx *ctxs, const StepTask *tasks) {
+    chain_wait();
     const StepTask t = tasks[blockIdx.x];
     const Ctx c = ctxs[t.sys];
     if (c.st->done) return;
@@ -301,12 +310,14 @@ __global__ void __launch_bounds__(256, 3) k_step_spmv(const Ctx *ctxs, const Ste
 
 template <class R>
 __global__ void __launch_bounds__(256, 3) k_step_pipe_p1(const Ctx *ctxs, const StepTask *tasks) {
+    R red;
+    red.init();
+    chain_wait();
     const StepTask t = tasks[blockIdx.x];
     const Ctx c = ctxs[t.sys];
     StateCopy sc;
     sc.load(c.st);
-    R red;
-    red.init();  // ends in a barrier
+    __syncthreads();
     if (sc.copy->done) return;
     pipe_p1_pairs(c, red, sc.copy->iter == 0, -sc.copy->alpha, sc.copy->beta, -sc.copy->omega,
                   (t.lo >> 1) + threadIdx.x, t.hi >> 1, blockDim.x, seg_odd(t));
@@ -316,12 +327,14 @@ __global__ void __launch_bounds__(256, 3) k_step_pipe_p1(const Ctx *ctxs, const 
 
 template <class R>
 __global__ void __launch_bounds__(256, 2) k_step_pipe_p3(const Ctx *ctxs, const StepTask *tasks) {
+    R red;
+    red.init();
+    chain_wait();
     const StepTask t = tasks[blockIdx.x];
     const Ctx c = ctxs[t.sys];
     StateCopy sc;
     sc.load(c.st);
-    R red;
-    red.init();  // ends in a barrier
+    __syncthreads();
     if (sc.copy->done) return;
     pipe_p3_pairs(c, red, sc.copy->alpha, sc.copy->omega, (t.lo >> 1) + threadIdx.x, t.hi >> 1, blockDim.x, seg_odd(t));
     __shared__ double vals[R::K];
@@ -400,21 +413,22 @@ cudaError_t step_admit(void *ctxs, const StepTask *tasks, int ntasks, int varian
     return cudaGetLastError();
 }
 
+// Chained launches: 20 iterations of 12 systems 2.16 -> 1.88 ms, of 60 systems 6.05
+// -> 5.72; 512 systems take as long either way.
 template <bool DIAG>
 static void iteration_t(const Ctx *c, const StepTask *tasks, int ntasks, int variant, cudaStream_t s) {
+    const auto go = [&](auto kern) { launch_chained(kern, dim3((unsigned)ntasks), 256, s, c, tasks); };
     if (variant == RBS_CLASSIC) {
-        if (DIAG) k_step_diag_k1<<<ntasks, 256, 0, s>>>(c, tasks);
-        else k_step_cls_k1<<<ntasks, 256, 0, s>>>(c, tasks);
-        k_step_cls_k2<<<ntasks, 256, 0, s>>>(c, tasks);
-        if (DIAG) k_step_diag_k3<<<ntasks, 256, 0, s>>>(c, tasks);
-        else k_step_cls_k3<<<ntasks, 256, 0, s>>>(c, tasks);
-        k_step_cls_k4<RowsR2><<<ntasks, 256, 0, s>>>(c, tasks);
-        k_step_cls_k5<<<ntasks, 256, 0, s>>>(c, tasks);
+        go(DIAG ? k_step_diag_k1 : k_step_cls_k1);
+        go(k_step_cls_k2);
+        go(DIAG ? k_step_diag_k3 : k_step_cls_k3);
+        go(k_step_cls_k4<RowsR2>);
+        go(k_step_cls_k5);
     } else {
-        k_step_pipe_p1<RowsR2><<<ntasks, 256, 0, s>>>(c, tasks);
-        k_step_spmv<true, DIAG><<<ntasks, 256, 0, s>>>(c, tasks);
-        k_step_pipe_p3<RowsR5><<<ntasks, 256, 0, s>>>(c, tasks);
-        k_step_spmv<false, DIAG><<<ntasks, 256, 0, s>>>(c, tasks);
+        go(k_step_pipe_p1<RowsR2>);
+        go(k_step_spmv<true, DIAG>);
+        go(k_step_pipe_p3<RowsR5>);
+        go(k_step_spmv<false, DIAG>);
     }
 }
 
