@@ -425,11 +425,13 @@ def _roofline(A, prof_tot):
     classic K1 (<r0,s>) and K3 (<q,y>, <y,y>) -- from the library's CUDA events
     over the timed solves. Only launches that ran are counted (the library
     leaves out those that returned at once on the stop flag). Algorithmic bytes
-    per launch: 12 nnz (col + val) + 8 (n+1) (rowptr) + 8 n (x, ideal reuse)
-    + 8 n (the companion vector of the dot) + 8 n (output) = 12 nnz + 32 n + 8.
+    per launch of a matrix of few diagonals: 8 nnz (val) + 4 n (row words) + n/4
+    (an int64 per 32 rows) + 8 n (x, ideal reuse) + 8 n (the companion vector of
+    the dot) + 8 n (output) = 8 nnz + 28.25 n; the CSR form's 12 nnz + 32 n + 8
+    (column indices, row pointers) is not read.
     K4 (x and r updates with <r0,r>, <r,r>) moves 64 n bytes per launch."""
     hbm, peak_kind = _peaks()
-    alg = 12 * A.nnz + 32 * A.n + 8
+    alg = 8 * A.nnz + 28 * A.n + 8 * ((A.n + 31) // 32)
     total_ms = max(sum(t[1] for t in prof_tot.values()), 1e-12)
 
     def stat(names, byt):

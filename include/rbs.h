@@ -371,9 +371,12 @@ int rbs_release(void);
  * "spmv.block" (short rows; long rows run in their own 4-warp blocks),
  * "spmv.mode" (0 auto: warp-staged rows, the long-row schedule when rows average
  * more than 8 nonzeros -- one staging buffer per warp, each row's values and x
- * entries moved to registers; 1 one thread per row; 2 short; 3 long rows),
- * "vec.grid", "vec.block", "solve.check_every", "smem.carveout" (percent of
- * L1/shared storage for the staging kernels; default 75, -1 = driver default);
+ * entries moved to registers; solves also lay matrices of up to 32 diagonals out
+ * without column indices and run small systems in one cluster; 1 one thread per
+ * row; 2 short; 3 long rows),
+ * "vec.grid", "vec.block", "solve.check_every", "smem.carveout" (most percent of
+ * L1/shared storage for the staging kernels, which take no more than their
+ * resident blocks need; default 75, -1 = driver default);
  * "test.stall_staging" (1: a test mode of the bounded device-side wait --
  * the staged SpMV announces its bulk copies without issuing them and gives up
  * after 64 polls, reads those rows from global memory instead, and the call

@@ -278,11 +278,11 @@ Cfg exdot_cfg(Workspace *w, int64_t n, int k, int window) {
     return persistent_cfg(w, n, exdot_blocks_per_sm(window, block), block, k);
 }
 
-// Shared-memory carveout of the staging kernels. Measured on GB300 (Poisson
-// 256^3): 60-75 % of the unified L1/shared storage is best -- enough shared
-// memory for three 256-thread blocks per SM while L1 keeps the SpMV's x
-// gathers; the maximum split costs about 5 % (25 % with a third staging
-// buffer per warp), a small one halves throughput.
+// Shared-memory carveout of the staging kernels, an upper bound: 60-75 % of the
+// unified L1/shared storage is best on Poisson 256^3 -- enough for three 256-thread
+// blocks per SM while L1 keeps the SpMV's x gathers; the maximum split costs about
+// 5 % there and 20 % on random columns, a small one halves throughput. (Kernels
+// that need less than the bound take less: SPMV_SHORT_CARVEOUT, prefer_shared.)
 int carveout_param() {
     const int64_t c = p_carveout.load();
     return (c >= 0 && c <= 100) ? (int)c : -1;

@@ -43,7 +43,7 @@ __device__ __forceinline__ void add_pairs(R &red, const double2 (&x)[U], const d
 // thread left two blocks per SM, and issue slots empty (2 million elements: 41
 // us against 30 now); an operand that several dots name comes from L2 for all
 // but the first of them, since their blocks walk the vectors together.
-// Bound by HBM once long (2^27: 331 us, 0.96 of the copy rate, cond 1; 378 with
+// Bound by HBM once long (2^27: 328 us, 0.965 of the copy rate, cond 1; 378 with
 // 64-bit digits) and by the windows' set-up, flush and cross-block sum when
 // short (2^24: 49 us, 39.5 of them HBM's; cond 1e48: 54 against 73).
 template <int W, bool EXPORT>
