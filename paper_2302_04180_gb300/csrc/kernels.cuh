@@ -544,7 +544,7 @@ stalled:
 // and only the values are staged. What bounds the product then is the FP64 pipe
 // (7 points at 256^3: 117 million fmas, 186 us at two per SM and clock) as much
 // as HBM (K1: 84 bytes per row, 207 us). Measured at 256^3: K1 335 -> 235 us, K3
-// 383 -> 268 (with the dots' windows in shared memory); the product alone at 192^3
+// 383 -> 252 (with the dots' windows in shared memory); the product alone at 192^3
 // 126 -> 98 (FP64 pipe 82 % of the active cycles).
 //
 // Warps take chunks round robin over the grid. (Several groups of consecutive

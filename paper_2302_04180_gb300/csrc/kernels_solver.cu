@@ -73,8 +73,9 @@ template <> struct FusedScratch<CAP_DIAG32> : FusedDiag<32> {};
 // The reducer R as K1, K3 and the pipelined set-up carry it: the kernels of few
 // diagonals, whose smaller staging leaves the shared memory, keep the exact
 // windows there (256^3, first hundred iterations: K3 320 -> 275 us, K1 249 -> 244,
-// 265 and 234 since; 283 with 10 words and 314 with 8, since products below the window go to
-// atomics while the vectors fall off steeply).
+// 252 and 234 since; 283 with 10 words and 314 with 8, since products below the window go to
+// atomics while the vectors fall off steeply; one branch for both of K3's products
+// 291).
 template <class R, int CAP>
 struct FusedDot {
     using type = R;
