@@ -547,9 +547,11 @@ stalled:
 // 383 -> 252 (with the dots' windows in shared memory); the product alone at 192^3
 // 126 -> 98 (FP64 pipe 82 % of the active cycles).
 //
-// Warps take chunks round robin over the grid. (Several groups of consecutive
-// chunks in a row per block, so that rows that gather the same x lines follow
-// each other on one SM, measured slower: K1 244 us with two or more, 235 so.)
+// Warps take chunks round robin over the grid, or in tiles: TILE groups of a
+// block's consecutive chunks, one per warp, before it moves on, so that rows that
+// gather the same x lines follow each other on one SM. Many diagonals gain from it
+// (27 points, 159^3: product 254 -> 242 us, K1 271 -> 259), seven lose registers and
+// time to the walk (256^3: K1 234 us without, 242 with tiles).
 //
 // N: most diagonals, in groups of up to eight (7: one group, the next chunk's
 // gathers ahead of this one's chain; 32: four, of which the unused are skipped).
@@ -561,6 +563,7 @@ struct DiagLayout {
     static constexpr int PER = N < 8 ? N : 8, G = N / PER;  // diagonals per group, groups
     static_assert(G == 1 || G % 2 == 0, "groups in pairs");
     static constexpr int WARPS = G == 1 ? MAX_WARPS : SPMV_REG_WARPS;
+    static constexpr int TILE = G == 1 ? 1 : 4;
     static constexpr int BUF = (32 * N + 2) * 8;
     static constexpr int SCRATCH = 2 * BUF;  // per warp
     static_assert(BUF % 16 == 0 && SCRATCH >= FLUSH_SCRATCH, "the flush reuses the staging buffers");
@@ -588,7 +591,21 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const uint32_t 
     }
     __syncwarp();
     const long long wait_limit = test_stall ? SPMV_TEST_WAIT_LIMIT : SPMV_WAIT_LIMIT;
+    // This warp's chunks in turn: whole rounds of tiles, then chunk by chunk, so
+    // that the last round is even over the blocks. `left`: steps to go in the
+    // tile; c >= c_end: none.
+    constexpr int TILE = L::TILE;
     const int round = nblk * nw;
+    const int tiled = TILE == 1 ? c_begin : c_begin + (c_end - c_begin) / (round * TILE) * (round * TILE);
+    struct Walk {
+        int c, left;
+    };
+    auto next = [&](Walk w) {
+        if (TILE == 1 || (w.left == 0 && w.c >= tiled)) return Walk{w.c + round, 0};
+        if (w.left > 0) return Walk{w.c + nw, w.left - 1};
+        w = Walk{w.c + (round - nw) * TILE + nw, TILE - 1};  // the next round's tile
+        return w.c < tiled ? w : Walk{tiled + blk * nw + wid, 0};
+    };
     struct Head {
         long long base;  // the chunk's first nonzero
         uint32_t word;   // this lane's row: its diagonals (N = 7: and where its values start, at bit 8)
@@ -623,23 +640,26 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const uint32_t 
         for (int j = 0; j < PER; j++)
             if ((word >> (g * PER + j)) & 1u) xv[j] = __ldca(x + (row + off(g * PER + j)));
     };
-    int c0 = c_begin + blk * nw + wid, c1 = c0 + round;  // the chunk being computed, the one after
-    Head h0 = head(c0), h1 = head(c1);
+    // the chunk being computed, the one after
+    Walk w0 = tiled > c_begin ? Walk{c_begin + blk * (TILE * nw) + wid, TILE - 1} : Walk{c_begin + blk * nw + wid, 0};
+    Walk w1 = next(w0);
+    Head h0 = head(w0.c), h1 = head(w1.c);
     unsigned parity = 0u;  // bit b: phase of buffer b's barrier to wait for
     double xa[PER], xb[PER], z0 = 0.0, z1 = 0.0;
     int cur = 0;
-    if (c0 < c_end) {
+    if (w0.c < c_end) {
         stage(h0, 0);
-        gather(c0 * 32 + lane, h0.word, 0, xa);
-        if (z && c0 * 32 + lane < n) z0 = __ldca(z + c0 * 32 + lane);
+        gather(w0.c * 32 + lane, h0.word, 0, xa);
+        if (z && w0.c * 32 + lane < n) z0 = __ldca(z + w0.c * 32 + lane);
     }
     // One chunk: stage the next one's values, then this one's chain. xc, zc hold
     // its first gathers and companion; xn, zn get the next one's (G = 1). Returns
     // false when the wait for the values ran out.
     auto step = [&](int b, double (&xc)[PER], double (&xn)[PER], double &zc, double &zn) {
-        const int row = c0 * 32 + lane, row1 = c1 * 32 + lane;
-        if (c1 < c_end) stage(h1, b ^ 1);
-        const Head h2 = head(c1 + round);
+        const int row = w0.c * 32 + lane, row1 = w1.c * 32 + lane;
+        if (w1.c < c_end) stage(h1, b ^ 1);
+        const Walk w2 = next(w1);
+        const Head h2 = head(w2.c);
         int at;  // this row's first value in the chunk
         if (N <= 8) {
             at = (int)(h0.word >> 8);
@@ -691,18 +711,18 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const uint32_t 
         }
         if (row < n) fn((int64_t)row, acc, zr);
         __syncwarp();  // buffer b is refilled in the next step
-        c0 = c1;
-        c1 += round;
+        w0 = w1;
+        w1 = w2;
         h0 = h1;
         h1 = h2;
         return true;
     };
     // two steps per turn (the buffers, and for one group the gathers, swap roles)
     bool ok = true;
-    while (c0 < c_end) {
+    while (w0.c < c_end) {
         cur = 0;
         if (!(ok = step(0, xa, xb, z0, z1))) break;
-        if (c0 >= c_end) break;
+        if (w0.c >= c_end) break;
         cur = 1;
         if (!(ok = G == 1 ? step(1, xb, xa, z1, z0) : step(1, xa, xb, z0, z1))) break;
     }
@@ -711,9 +731,9 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const uint32_t 
     // this and every later row from global memory, then wait (bounded) for the
     // copies in flight.
     err |= ERR_TIMEOUT;
-    const bool more = c1 < c_end;
-    for (; c0 < c_end; c0 += round) {
-        const int row = c0 * 32 + lane;
+    const bool more = w1.c < c_end;
+    for (; w0.c < c_end; w0 = next(w0)) {
+        const int row = w0.c * 32 + lane;
         if (row < n) {
             bool bad = false;
             const double acc = spmv_row(A, row, x, bad);
