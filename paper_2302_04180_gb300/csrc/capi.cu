@@ -958,9 +958,12 @@ int batch_stepped(Workspace *w, int32_t nsys, const rbs_system *systems, rbs_inf
     std::vector<int32_t> maxit((size_t)nsys, 0);
     size_t work_elems = 0, hist_recs = 0, layout_bytes = 0;
     // room for a system's layout by diagonals: one word per row, one int64 per 32
+    // (the knob is read once: another thread may change it during the call)
+    std::vector<size_t> layout((size_t)nsys, 0);
+    const bool layouts = p_spmv_mode.load() == 0;
     auto layout_of = [&](const rbs_system &S) -> size_t {
         const CSRArgs A{S.A.n, S.A.nnz, S.A.rowptr, S.A.col, S.A.val};
-        if (p_spmv_mode.load() != 0 || !step_wants_layout(A)) return 0;
+        if (!layouts || !step_wants_layout(A)) return 0;
         const size_t chunks = (size_t)(S.A.n + 31) / 32;
         return chunks * (32 * sizeof(uint32_t) + sizeof(int64_t));
     };
@@ -980,7 +983,7 @@ int batch_stepped(Workspace *w, int32_t nsys, const rbs_system *systems, rbs_inf
         maxit[(size_t)i] = proxy ? std::min(S.maxit, std::max(proxy_maxit[i], 1)) : S.maxit;
         const int64_t stride = (S.A.n + 31) / 32 * 32;
         work_elems += (size_t)stride * ((S.variant == RBS_PIPELINED ? 16 : 9) + (proxy ? 1 : 0));
-        layout_bytes += layout_of(S);
+        layout_bytes += layout[(size_t)i] = layout_of(S);
         const int cap = hists ? std::min(hists[i].cap, S.maxit) : 0;
         hist_recs += (size_t)(cap > 0 ? cap : 0);
     }
@@ -1038,10 +1041,10 @@ int batch_stepped(Workspace *w, int32_t nsys, const rbs_system *systems, rbs_inf
         CSRArgs A{S.A.n, S.A.nnz, S.A.rowptr, S.A.col, S.A.val};
         int64_t *base = nullptr;
         uint32_t *mask = nullptr;
-        if (const size_t bytes = layout_of(S)) {
+        if (layout[(size_t)i]) {
             base = (int64_t *)((char *)w->step_diag.p + loff);
             mask = (uint32_t *)(base + (S.A.n + 31) / 32);
-            loff += bytes;
+            loff += layout[(size_t)i];
         }
         step_ctx_make(hctx.data() + (size_t)i * cb, A, V, S.b, S.x0, S.jacobi_diag, dst + i, dscr + i,
                       hist_dev[(size_t)i], mask, base);

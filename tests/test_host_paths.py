@@ -1,0 +1,42 @@
+"""Host code of the library against a fake CUDA runtime (host_library.py): what it
+allocates, copies and launches where no GPU is needed to tell right from wrong."""
+import numpy as np
+import pytest
+
+from host_library import host_library
+from paper_2302_04180_gb300 import gen
+
+
+@pytest.fixture()
+def host():
+    with host_library() as h:
+        yield h
+        assert h.faults() == ""
+
+
+def _system(h, A, maxit, variant=0):
+    return {"A": h.csr(A), "b": h.device(np.ones(A.n)), "x": h.device(np.zeros(A.n)), "tol": 1e-8, "maxit": maxit,
+            "variant": variant}
+
+
+def test_stepped_batch_reads_the_schedule_knob_once(host):
+    """spmv.mode changed by another thread while a stepped batch is being laid out: the
+    systems' layouts by diagonals lie in the memory that was sized for them."""
+    A = gen.poisson3d(20)
+    systems = [_system(host, A, 3, v) for v in (0, 1)]
+    host.rbs.rbs_stream_status()  # the workspace exists
+    host.rbs.rbs_set_param("spmv.mode", 2)
+    stray = []
+
+    def change(call, what, n):
+        if call == "cudaMalloc":
+            host.rbs.rbs_set_param("spmv.mode", 0)
+        if call == "launch" and "k_step_prepare" in what:
+            stray.append(host.fake.fake_stray_pointers())
+    host.fail = change
+    try:
+        host.rbs.rbs_solve_batched(systems, schedule={"cluster": 0, "split": 0})
+    finally:
+        host.fail = None
+        host.rbs.rbs_set_param("spmv.mode", 0)
+    assert len(stray) == 2 and not any(stray)
