@@ -947,9 +947,9 @@ int batch_stepped(Workspace *w, int32_t nsys, const rbs_system *systems, rbs_inf
     // left (so that they still spread over every SM)
     const int64_t fixed_rows = sched.split > 0 ? (sched.split + 63) / 64 * 64 : 0;
     int64_t rows = fixed_rows ? fixed_rows : 8192;
+    const int64_t waves = 4LL * w->sms * 3;
     auto pick_rows = [&](int64_t active_rows) {
         if (fixed_rows) return fixed_rows;
-        const int64_t waves = 4LL * w->sms * 3;
         int64_t r = (active_rows + waves - 1) / waves;
         r = std::max<int64_t>(1024, std::min<int64_t>(65536, r));
         return (r + 63) / 64 * 64;
@@ -1070,7 +1070,10 @@ int batch_stepped(Workspace *w, int32_t nsys, const rbs_system *systems, rbs_inf
     tasks_of(cls, tasks);
     const size_t ncls = tasks.size();
     tasks_of(pipe, tasks);
-    CK(ensure(w->step_tasks, std::max<size_t>(tasks.size(), 1) * sizeof(StepTask)));
+    // A later list may be longer than this first one: fewer rows are cut into smaller
+    // blocks, and those are rounded to 64 rows. It has at most `waves` whole blocks
+    // and one more per system (blocks of the largest size: no more than now).
+    CK(ensure(w->step_tasks, std::max<size_t>(tasks.size(), (size_t)(waves + nsys)) * sizeof(StepTask)));
     StepTask *dtask = (StepTask *)w->step_tasks.p;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (ms) {

@@ -40,3 +40,16 @@ def test_stepped_batch_reads_the_schedule_knob_once(host):
         host.fail = None
         host.rbs.rbs_set_param("spmv.mode", 0)
     assert len(stray) == 2 and not any(stray)
+
+
+def _diagonal(n):
+    return gen.CSR(n, np.arange(n + 1, dtype=np.int64), np.arange(n, dtype=np.int32), np.ones(n))
+
+
+@pytest.mark.parametrize("sizes", [(1867776, 1088), (3735552, 70000, 900)])
+def test_stepped_batch_task_list_may_grow(host, sizes):
+    """Rows per block follow the rows still iterating, in steps of 64: once the small
+    system has run its iterations the large one may take more blocks than both did."""
+    systems = [_system(host, _diagonal(n), 20 if k == 0 else 3) for k, n in enumerate(sizes)]
+    got = host.rbs.rbs_solve_batched(systems, history=False, schedule={"cluster": 0, "split": 0})
+    assert len(got) == len(sizes) and host.faults() == ""
