@@ -19,8 +19,8 @@ struct DotArgs {
 // two at four in 346 (64 registers spill).
 constexpr int EXDOT_PAIRS = 2, EXDOT_BLOCKS = 3;
 
-// U pairs into the windows.
-template <int U, class R>
+// U pairs into the windows. WARP: every lane of the warp has them.
+template <int U, bool WARP, class R>
 __device__ __forceinline__ void add_pairs(R &red, const double2 (&x)[U], const double2 (&y)[U]) {
     double xv[2 * U], yv[2 * U];
 #pragma unroll
@@ -30,7 +30,7 @@ __device__ __forceinline__ void add_pairs(R &red, const double2 (&x)[U], const d
         yv[2 * u] = y[u].x;
         yv[2 * u + 1] = y[u].y;
     }
-    red.template add<2 * U>(0, xv, yv);
+    red.template add<2 * U, false, WARP>(0, xv, yv);
 }
 
 // Exact dots over the same length (Sec. 2 exdot; Sec. 4.1/4.2 merged
@@ -72,35 +72,37 @@ __global__ void __launch_bounds__(256, EXDOT_BLOCKS)
         // loop with the loads of each ahead of the adds of the other
         const int64_t full = n2 > st ? (n2 - st) / (U * st) : 0;
         double2 xa[U], ya[U], xb[U], yb[U];
+        const double2 *xq = x2 + j, *yq = y2 + j;
         auto load = [&](double2 (&xv)[U], double2 (&yv)[U]) {
 #pragma unroll
             for (int u = 0; u < U; u++) {
-                xv[u] = __ldcs(x2 + j);
-                yv[u] = __ldcs(y2 + j);
-                j += st;
+                xv[u] = __ldcs(xq);
+                yv[u] = __ldcs(yq);
+                xq += st;
+                yq += st;
             }
         };
         if (full > 0) load(xa, ya);
         red.open({max(R::limb_of(x0[0].x, y0[0].x), R::limb_of(x0[0].y, y0[0].y))});
-        add_pairs<1>(red, x0, y0);
+        add_pairs<1, false>(red, x0, y0);
         int64_t s = 0;
         for (; s + 2 < full; s += 2) {
             load(xb, yb);
-            add_pairs<U>(red, xa, ya);
+            add_pairs<U, true>(red, xa, ya);
             load(xa, ya);
-            add_pairs<U>(red, xb, yb);
+            add_pairs<U, true>(red, xb, yb);
         }
         if (s + 1 < full) {
             load(xb, yb);
-            add_pairs<U>(red, xa, ya);
-            add_pairs<U>(red, xb, yb);
+            add_pairs<U, true>(red, xa, ya);
+            add_pairs<U, true>(red, xb, yb);
         } else if (s < full) {
-            add_pairs<U>(red, xa, ya);
+            add_pairs<U, true>(red, xa, ya);
         }
-        for (; j < n2; j += st) {
+        for (j += full * (U * st); j < n2; j += st) {
             x0[0] = __ldcs(x2 + j);
             y0[0] = __ldcs(y2 + j);
-            add_pairs<1>(red, x0, y0);
+            add_pairs<1, false>(red, x0, y0);
         }
         if ((n & 1) && gtid() == 0) red.add(0, xp[n - 1], yp[n - 1]);
     } else {

@@ -97,7 +97,10 @@ struct ExactRows {
     static constexpr uint32_t ZERO = SPLIT ? 0u : 0x80000000u;  // a word that holds nothing
     static_assert(ROWS <= 255, "placements in bytes, the zero products' included");
     uint32_t *win;  // this thread's column: word j of sign s of dot k at win[(k * PER + s * W + j) * NT]
-    int a[K];       // anchor limbs, WIN_EMPTY when there is no window yet
+    // Anchor limbs. No window yet: NO_ANCHOR, with SPLIT the lowest window there is
+    // (whose products, below 2^-1764, are as good as none).
+    static constexpr int NO_ANCHOR = SPLIT ? 0 : WIN_EMPTY;
+    int a[K];
     unsigned long long (*sacc)[NL];
     uint32_t *sflags;
     int *amax;
@@ -112,7 +115,7 @@ struct ExactRows {
         sflags = s_flags;
         amax = s_amax;
 #pragma unroll
-        for (int k = 0; k < K; k++) a[k] = WIN_EMPTY;
+        for (int k = 0; k < K; k++) a[k] = NO_ANCHOR;
 #pragma unroll
         for (int j = 0; j < ROWS; j++) win[j * NT] = ZERO;
         if (threadIdx.x < K) s_amax[threadIdx.x] = -1;
@@ -162,24 +165,30 @@ struct ExactRows {
     // re-anchor). v: x and y of each in turn. Returns the thread's anchor.
     template <class... D>
     static __device__ __noinline__ int add_any(uint32_t *w, unsigned long long *sk, uint32_t *fl, int a, D... v) {
-        const double xy[] = {v...};
-#pragma unroll
+        // (SPLIT: one copy of the code, the products moving up in turn. Unrolled, the
+        // call took registers that the caller's loads in flight need: 2^27 325 us, 313 so)
+        constexpr int AHEAD = SPLIT ? 1 : 8;
+        double xy[] = {v...};
+#pragma unroll AHEAD
         for (int i = 0; i < (int)sizeof...(D); i += 2) {
+            const double x = xy[0], y = xy[1];
+#pragma unroll
+            for (int k = 2; k < (int)sizeof...(D); k++) xy[k - 2] = xy[k];
             uint32_t u[5], m, f = 0u;
             int L;
-            if (!prod_exact(xy[i], xy[i + 1], f, u, L, m)) {
-                if (f) atomicOr(fl, f);
+            if (!prod_exact(x, y, f, u, L, m)) {
+                if (f && (*(volatile uint32_t *)fl & f) != f) atomicOr(fl, f);
                 continue;
             }
             if (L < a) {
-                smem_deposit(sk, u, L, m);
+                if (SPLIT) smem_deposit_ahead(sk, u, L, m);
+                else smem_deposit(sk, u, L, m);
                 continue;
             }
             if (L - a > QMAX) {
                 int top = L;
-                if (a >= 0) {
-                    flush_column(w, sk, a);
-                } else {
+                if (SPLIT || a >= 0) flush_column(w, sk, a);
+                if (a <= 0) {
                     const int m = (int)__reduce_max_sync(__activemask(), (unsigned)L);
                     if (m - L <= ANCHOR) top = m;
                 }
@@ -211,22 +220,49 @@ struct ExactRows {
     // is normal and every product lands in the window (nearly always), straight
     // code. Otherwise zero products are sent to five words that nobody reads, and
     // any other kind sends all N through add_any(). N is 1, 2 or 4.
-    template <int N, bool SQ = false>
+    // WARP: all 32 lanes call it and take the branch together if one of them has to.
+    // Lanes that went out of line while the others ran the straight code cost the
+    // warp both: 2^24 products of which one in a hundred lies 2^400 below the rest
+    // 205 us, 102 so; exponents of -200 .. 200 331, 145.
+    template <int N, bool SQ = false, bool WARP = false>
     __device__ __forceinline__ void add(int k, const double (&x)[N], const double (&y)[N]) {
-        uint32_t xh[N], yh[N], e[N], q[N], odd = 0u, far = 0u;
+        uint32_t xh[N], yh[N], e[N], q[N];
         uint32_t *wk = win + k * PER * NT;
+        bool plain;  // every operand normal, every product in the window
+        if constexpr (SPLIT) {
+            // e: bit position above the window's lowest << 20, modulo 2^32, which holds
+            // every position: one subtraction for the placement, the shift and the test
+            uint32_t lowest = 0x7ff00000u, highest = 0u, far = 0u;
+            const uint32_t base = ((uint32_t)a[k] << 25) + (2u << 20);
 #pragma unroll
-        for (int i = 0; i < N; i++) {
-            xh[i] = (uint32_t)__double2hiint(x[i]);
-            yh[i] = (uint32_t)__double2hiint(y[i]);
-            const uint32_t ex = xh[i] & 0x7ff00000u, ey = yh[i] & 0x7ff00000u;
-            odd = max(max(odd, ex - 0x00100000u), ey - 0x00100000u);
-            e[i] = ex + ey - (2u << 20);  // bit position << 20; garbage for an odd operand
-            q[i] = (e[i] >> 25) - (uint32_t)a[k];
-            far = max(far, q[i]);
+            for (int i = 0; i < N; i++) {
+                xh[i] = (uint32_t)__double2hiint(x[i]);
+                yh[i] = (uint32_t)__double2hiint(y[i]);
+                const uint32_t ex = xh[i] & 0x7ff00000u, ey = yh[i] & 0x7ff00000u;
+                lowest = min(lowest, min(ex, ey));
+                highest = max(highest, max(ex, ey));
+                e[i] = ex + ey - base;
+                q[i] = e[i] >> 25;
+                far = max(far, e[i]);
+            }
+            plain = lowest != 0u && highest < 0x7ff00000u && far < (QMAX + 1u) << 25;
+        } else {
+            uint32_t odd = 0u, far = 0u;
+#pragma unroll
+            for (int i = 0; i < N; i++) {
+                xh[i] = (uint32_t)__double2hiint(x[i]);
+                yh[i] = (uint32_t)__double2hiint(y[i]);
+                const uint32_t ex = xh[i] & 0x7ff00000u, ey = yh[i] & 0x7ff00000u;
+                odd = max(max(odd, ex - 0x00100000u), ey - 0x00100000u);
+                e[i] = ex + ey - (2u << 20);  // bit position << 20; garbage for an odd operand
+                q[i] = (e[i] >> 25) - (uint32_t)a[k];
+                far = max(far, q[i]);
+            }
+            plain = odd < 0x7fe00000u && far <= (uint32_t)QMAX;
         }
         bool go = true;
-        if (!(odd < 0x7fe00000u && far <= (uint32_t)QMAX)) {
+        if (WARP ? __any_sync(0xffffffffu, !plain) : !plain) {
+            bool some = !WARP;  // a product that is not zero
 #pragma unroll
             for (int i = 0; i < N; i++) {
                 const uint32_t ex = xh[i] & 0x7ff00000u, ey = yh[i] & 0x7ff00000u;
@@ -236,9 +272,11 @@ struct ExactRows {
                     q[i] = (uint32_t)(ROWS - k * PER);
                     xh[i] = yh[i];
                 } else {
+                    some = true;
                     go = go && max(ex - 0x00100000u, ey - 0x00100000u) < 0x7fe00000u && q[i] <= (uint32_t)QMAX;
                 }
             }
+            if (WARP) go = !__any_sync(0xffffffffu, !go);
             if (!go) {
                 if constexpr (N == 1)
                     a[k] = add_any(wk, sacc[k], &sflags[k], a[k], x[0], y[0]);
@@ -246,6 +284,8 @@ struct ExactRows {
                     a[k] = add_any(wk, sacc[k], &sflags[k], a[k], x[0], y[0], x[1], y[1]);
                 else
                     a[k] = add_any(wk, sacc[k], &sflags[k], a[k], x[0], y[0], x[1], y[1], x[2], y[2], x[3], y[3]);
+            } else {
+                go = some;
             }
         }
         if (go) {
