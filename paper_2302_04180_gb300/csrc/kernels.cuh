@@ -4,6 +4,7 @@
 
 #include <cuda_pipeline.h>
 
+#include "diag_walk.h"
 #include "launch.h"
 #include "reduce.cuh"
 
@@ -591,21 +592,8 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const uint32_t 
     }
     __syncwarp();
     const long long wait_limit = test_stall ? SPMV_TEST_WAIT_LIMIT : SPMV_WAIT_LIMIT;
-    // This warp's chunks in turn: whole rounds of tiles, then chunk by chunk, so
-    // that the last round is even over the blocks. `left`: steps to go in the
-    // tile; c >= c_end: none.
-    constexpr int TILE = L::TILE;
-    const int round = nblk * nw;
-    const int tiled = TILE == 1 ? c_begin : c_begin + (c_end - c_begin) / (round * TILE) * (round * TILE);
-    struct Walk {
-        int c, left;
-    };
-    auto next = [&](Walk w) {
-        if (TILE == 1 || (w.left == 0 && w.c >= tiled)) return Walk{w.c + round, 0};
-        if (w.left > 0) return Walk{w.c + nw, w.left - 1};
-        w = Walk{w.c + (round - nw) * TILE + nw, TILE - 1};  // the next round's tile
-        return w.c < tiled ? w : Walk{tiled + blk * nw + wid, 0};
-    };
+    const DiagChunks<L::TILE> chunks{c_begin, c_end, blk, nblk, wid, nw};
+    using Walk = typename DiagChunks<L::TILE>::Walk;
     struct Head {
         long long base;  // the chunk's first nonzero
         uint32_t word;   // this lane's row: its diagonals (N = 7: and where its values start, at bit 8)
@@ -641,8 +629,7 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const uint32_t 
             if ((word >> (g * PER + j)) & 1u) xv[j] = __ldca(x + (row + off(g * PER + j)));
     };
     // the chunk being computed, the one after
-    Walk w0 = tiled > c_begin ? Walk{c_begin + blk * (TILE * nw) + wid, TILE - 1} : Walk{c_begin + blk * nw + wid, 0};
-    Walk w1 = next(w0);
+    Walk w0 = chunks.first(), w1 = chunks.next(w0);
     Head h0 = head(w0.c), h1 = head(w1.c);
     unsigned parity = 0u;  // bit b: phase of buffer b's barrier to wait for
     double xa[PER], xb[PER], z0 = 0.0, z1 = 0.0;
@@ -656,9 +643,9 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const uint32_t 
     // its first gathers and companion; xn, zn get the next one's (G = 1). Returns
     // false when the wait for the values ran out.
     auto step = [&](int b, double (&xc)[PER], double (&xn)[PER], double &zc, double &zn) {
-        const int row = w0.c * 32 + lane, row1 = w1.c * 32 + lane;
+        const int row = w0.c * 32 + lane, row1 = chunks.row(w1.c, n, lane);  // (w0.c < c_end)
         if (w1.c < c_end) stage(h1, b ^ 1);
-        const Walk w2 = next(w1);
+        const Walk w2 = chunks.next(w1);
         const Head h2 = head(w2.c);
         int at;  // this row's first value in the chunk
         if (N <= 8) {
@@ -732,7 +719,7 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const uint32_t 
     // copies in flight.
     err |= ERR_TIMEOUT;
     const bool more = w1.c < c_end;
-    for (; w0.c < c_end; w0 = next(w0)) {
+    for (; w0.c < c_end; w0 = chunks.next(w0)) {
         const int row = w0.c * 32 + lane;
         if (row < n) {
             bool bad = false;
