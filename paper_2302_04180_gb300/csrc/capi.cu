@@ -755,6 +755,11 @@ int rbs_solve_ex(const rbs_csr *A, const double *b, const double *x0, const doub
     const int carve = carveout_param();
     int smode = spmv_mode_for(n, nnz);
     const bool try_diags = p_spmv_mode.load() == 0 && nnz > 0 && nnz <= SPMV_DIAGS * n && ((uintptr_t)val & 15) == 0;
+    const auto check_and_invert = [&] {
+        const cudaError_t e = launch_csr_check(a.A, &w->g->err, grid_for(w, nnz > n ? nnz : n, 256, 8), w->stream);
+        return e != cudaSuccess ? e : launch_jacobi_invd(a.A, (const double *)ddiag, V.invd, &w->g->err,
+                                                         grid_for(w, n, 256, 8), w->stream);
+    };
     if (try_diags) {
         const int64_t chunks = (n + 31) / 32;
         const size_t mask_at = ((size_t)(chunks + 1) * 8 + sizeof(DiagArgs) + 255) / 256 * 256;
@@ -768,11 +773,15 @@ int rbs_solve_ex(const rbs_csr *A, const double *b, const double *x0, const doub
         a.D.mask = mask;
         a.D.base = base;
     } else {
-        CK(launch_csr_check(a.A, &w->g->err, grid_for(w, nnz > n ? nnz : n, 256, 8), w->stream));
-        CK(launch_jacobi_invd(a.A, (const double *)ddiag, V.invd, &w->g->err, grid_for(w, n, 256, 8), w->stream));
+        CK(check_and_invert());
     }
     unsigned err = 0;
     if ((rc = read_err(w, &err))) return rc;
+    if (err & ERR_LONG) {
+        CK(check_and_invert());
+        if ((rc = read_err(w, &err))) return rc;
+        err |= ERR_DIAGS;
+    }
     if (err & 1u) return fail(RBS_EINVAL, "invalid CSR structure");
     if (err & 2u) return fail(RBS_EINVAL, "zero, NaN or missing diagonal entry");
     if (try_diags && !(err & ERR_DIAGS)) {

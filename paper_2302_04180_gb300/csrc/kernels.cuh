@@ -796,16 +796,21 @@ __device__ __forceinline__ int sample_diags(const CSRView &A, int most, int32_t 
 // stored (i, i) entry, a zero, NaN or missing one sets bit 2 and inv = 0; word:
 // which of the m diagonals s_off (ascending, then 0x7fffffff) the row has, or
 // ERR_DIAGS if its columns do not ascend along them. Eight columns are loaded at a
-// time.
+// time. A row of more than `most` nonzeros only gets ERR_LONG.
 struct RowSetup {
     uint32_t word;
     unsigned err;
     double inv;
     int64_t first;  // rowptr[i]
 };
-__device__ __forceinline__ RowSetup check_row(const CSRView &A, int64_t i, const double *diag, const int *s_off, int m) {
+__device__ __forceinline__ RowSetup check_row(const CSRView &A, int64_t i, const double *diag, const int *s_off, int m,
+                                              int64_t most = INT64_MAX) {
     const int64_t b = A.rowptr[i], e = A.rowptr[i + 1];
     RowSetup o{0u, 0u, 0.0, b};
+    if (e - b > most) {
+        o.err = ERR_LONG;
+        return o;
+    }
     double d = 0.0;
     bool found = false, fits = m > 0;
     if (b < 0 || e < b || e > A.nnz) {

@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(256) k_prepare(CSRView A, const double *diag, 
     for (int64_t i = gtid(); i < padded; i += gstride()) {
         uint32_t word = 0u;
         if (i < A.n) {
-            const RowSetup r = check_row(A, i, diag, s_off, m);
+            const RowSetup r = check_row(A, i, diag, s_off, m, LONG_ROW);
             eb |= r.err;
             invd[i] = r.inv;
             if ((i & 31) == 0) base[i >> 5] = r.first;

@@ -141,6 +141,12 @@ cudaError_t launch_csr_check(const CSRArgs &A, unsigned *err, Cfg cfg, cudaStrea
 // they are too many; mask and base are written for them, and a row that does
 // not fit them sets ERR_DIAGS in err (it is no error of the matrix).
 constexpr unsigned ERR_DIAGS = 16u;
+// A row of more than LONG_ROW nonzeros sets ERR_LONG, is not looked into and has no
+// layout: launch_csr_check and launch_jacobi_invd then do the whole set-up, the
+// check with the nonzeros spread over the grid. (One thread took 13.8 ms for one
+// dense row of 200000, they take 0.09; 256 nonzeros take it 16 us.)
+constexpr unsigned ERR_LONG = 32u;
+constexpr int LONG_ROW = 256;
 cudaError_t launch_prepare(const CSRArgs &A, const double *diag, double *invd, DiagArgs *diags, uint32_t *mask,
                            int64_t *base, unsigned *err, Cfg cfg, cudaStream_t s);
 
