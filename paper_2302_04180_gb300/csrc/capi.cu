@@ -687,13 +687,19 @@ int rbs_solve_ex(const rbs_csr *A, const double *b, const double *x0, const doub
         }
         CSRArgs A1{n, nnz, (const int64_t *)rowptr, (const int32_t *)col, (const double *)val};
         CK(ensure(w->batch_out, sizeof(BatchOut)));
-        BatchOut *d_out = (BatchOut *)w->batch_out.p, O;
+        BatchOut *d_out = (BatchOut *)w->batch_out.p, O{};
+        O.err = SMALL_NO_ROOM;
         CK(cudaMemsetAsync(d_out, 0, sizeof(BatchOut), w->stream));
-        CK(launch_small(A1, (const double *)db, (const double *)dx0, (const double *)ddiag, dx, tol, maxit, variant,
-                        (double *)w->hist.p, hcap, d_out, w->stream));
-        CK(cudaMemcpyAsync(w->h_small, d_out, sizeof(BatchOut), cudaMemcpyDeviceToHost, w->stream));
-        CK(cudaStreamSynchronize(w->stream));
-        O = *w->h_small;
+        const cudaError_t launched =
+            launch_small(A1, (const double *)db, (const double *)dx0, (const double *)ddiag, dx, tol, maxit, variant,
+                         (double *)w->hist.p, hcap, d_out, w->stream);
+        if (launched == cudaSuccess) {
+            CK(cudaMemcpyAsync(w->h_small, d_out, sizeof(BatchOut), cudaMemcpyDeviceToHost, w->stream));
+            CK(cudaStreamSynchronize(w->stream));
+            O = *w->h_small;
+        } else {
+            cudaGetLastError();  // no cluster to be had: the launch-per-step kernels
+        }
         if (O.err & 1u) return fail(RBS_EINVAL, "invalid CSR structure");
         if (!(O.err & SMALL_NO_ROOM)) {
             if (O.err & 2u) return fail(RBS_EINVAL, "zero, NaN or missing diagonal entry");

@@ -53,3 +53,24 @@ def test_stepped_batch_task_list_may_grow(host, sizes):
     systems = [_system(host, _diagonal(n), 20 if k == 0 else 3) for k, n in enumerate(sizes)]
     got = host.rbs.rbs_solve_batched(systems, history=False, schedule={"cluster": 0, "split": 0})
     assert len(got) == len(sizes) and host.faults() == ""
+
+
+NO_MEMORY, CLUSTER_FAILED = 2, 912  # cudaErrorMemoryAllocation, cudaErrorClusterOutOfResources
+
+
+def _solve(host, A, **kw):
+    return host.rbs.rbs_solve(host.csr(A), host.device(np.ones(A.n)), tol=1e-8, maxit=20, x_out=host.device(np.zeros(A.n)), **kw)
+
+
+@pytest.mark.parametrize("variant", [0, 1])
+def test_small_solve_goes_on_when_its_launch_is_refused(host, variant):
+    """A refused cluster launch is no error of the solve: the launch-per-step loop runs it."""
+    A = gen.poisson3d(8)
+    host.fail = lambda call, what, n: CLUSTER_FAILED if call == "launch" and "k_small" in what else 0
+    _solve(host, A, variant=variant)
+    host.fail = None
+    names = " ".join(host.launched())
+    assert "k_small" in names and ("k_cls_k1" if variant == 0 else "k_pipe_p1") in names
+    host.events.clear()
+    _solve(host, A, variant=variant)  # nothing of the refusal is left
+    assert [n for n in host.launched() if "k_small" in n] and not [n for n in host.launched() if "k_prepare" in n]
