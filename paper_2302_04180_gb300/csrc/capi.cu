@@ -760,16 +760,19 @@ int rbs_solve_ex(const rbs_csr *A, const double *b, const double *x0, const doub
     // few diagonals are laid out by them in the same pass
     const int carve = carveout_param();
     int smode = spmv_mode_for(n, nnz);
-    const bool try_diags = p_spmv_mode.load() == 0 && nnz > 0 && nnz <= SPMV_DIAGS * n && ((uintptr_t)val & 15) == 0;
+    bool try_diags = p_spmv_mode.load() == 0 && nnz > 0 && nnz <= SPMV_DIAGS * n && ((uintptr_t)val & 15) == 0;
+    const int64_t chunks = (n + 31) / 32;
+    const size_t mask_at = ((size_t)(chunks + 1) * 8 + sizeof(DiagArgs) + 255) / 256 * 256;
+    if (try_diags && ensure(w->diag, mask_at + (size_t)chunks * 32 * 4) != cudaSuccess) {
+        cudaGetLastError();  // no room for it: the general rows
+        try_diags = false;
+    }
     const auto check_and_invert = [&] {
         const cudaError_t e = launch_csr_check(a.A, &w->g->err, grid_for(w, nnz > n ? nnz : n, 256, 8), w->stream);
         return e != cudaSuccess ? e : launch_jacobi_invd(a.A, (const double *)ddiag, V.invd, &w->g->err,
                                                          grid_for(w, n, 256, 8), w->stream);
     };
     if (try_diags) {
-        const int64_t chunks = (n + 31) / 32;
-        const size_t mask_at = ((size_t)(chunks + 1) * 8 + sizeof(DiagArgs) + 255) / 256 * 256;
-        CK(ensure(w->diag, mask_at + (size_t)chunks * 32 * 4));
         int64_t *base = (int64_t *)w->diag.p;
         DiagArgs *dd = (DiagArgs *)(base + chunks + 1);
         uint32_t *mask = (uint32_t *)((char *)w->diag.p + mask_at);

@@ -74,3 +74,28 @@ def test_small_solve_goes_on_when_its_launch_is_refused(host, variant):
     host.events.clear()
     _solve(host, A, variant=variant)  # nothing of the refusal is left
     assert [n for n in host.launched() if "k_small" in n] and not [n for n in host.launched() if "k_prepare" in n]
+
+
+def _sizes(host):
+    return {n for call, _, n in host.events if call == "cudaMalloc"}
+
+
+def test_solve_goes_on_without_room_for_the_layout(host):
+    """The diagonal layout is scratch that a solve can do without: when it does not fit,
+    the general rows run, and nothing of the refusal is left."""
+    A = gen.poisson3d(34)
+    host.rbs.rbs_set_param("spmv.mode", 2)
+    _solve(host, A)
+    host.rbs.rbs_set_param("spmv.mode", 0)
+    needed = _sizes(host)
+    host.rbs.rbs_release()
+    host.events.clear()
+    host.fail = lambda call, what, n: NO_MEMORY if call == "cudaMalloc" and n not in needed else 0
+    _solve(host, A)
+    assert _sizes(host) - needed, "nothing was refused"
+    k1 = [n for n in host.launched() if "k_cls_k1" in n]
+    assert k1 and all("Lin" not in n for n in k1), k1  # (a negative template argument is a diagonal kernel)
+    host.fail = None
+    host.events.clear()
+    _solve(host, A)
+    assert [n for n in host.launched() if "k_cls_k1" in n and "Lin7E" in n]
