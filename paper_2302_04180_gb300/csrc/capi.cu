@@ -1008,7 +1008,10 @@ int batch_stepped(Workspace *w, int32_t nsys, const rbs_system *systems, rbs_inf
     const size_t cb = step_ctx_bytes();
     CK(ensure(w->batch_work, work_elems * 8));
     CK(ensure(w->batch_hist, (hist_recs > 0 ? hist_recs : 1) * RBS_HIST_W * 8));
-    CK(ensure(w->step_diag, layout_bytes));
+    if (layout_bytes && ensure(w->step_diag, layout_bytes) != cudaSuccess) {
+        cudaGetLastError();  // no room for them: general rows
+        layout.assign((size_t)nsys, 0);
+    }
     CK(ensure(w->step_ctx, (size_t)nsys * cb));
     CK(ensure(w->step_state, (size_t)nsys * sizeof(SolverState)));
     CK(ensure(w->step_scr, (size_t)nsys * sizeof(DotScratch)));

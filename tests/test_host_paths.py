@@ -99,3 +99,24 @@ def test_solve_goes_on_without_room_for_the_layout(host):
     host.events.clear()
     _solve(host, A)
     assert [n for n in host.launched() if "k_cls_k1" in n and "Lin7E" in n]
+
+
+def test_stepped_batch_goes_on_without_room_for_the_layouts(host):
+    A = gen.poisson3d(20)
+    systems = [_system(host, A, 3, v) for v in (0, 1)]
+
+    def run():
+        host.events.clear()
+        host.rbs.rbs_solve_batched(systems, schedule={"cluster": 0, "split": 0})
+    host.rbs.rbs_set_param("spmv.mode", 2)
+    run()
+    host.rbs.rbs_set_param("spmv.mode", 0)
+    needed = _sizes(host)
+    host.rbs.rbs_release()
+    host.fail = lambda call, what, n: NO_MEMORY if call == "cudaMalloc" and n not in needed else 0
+    run()
+    assert _sizes(host) - needed, "nothing was refused"
+    assert [n for n in host.launched() if "k_step_cls_k1" in n] and host.fake.fake_stray_pointers() == 0
+    host.fail = None
+    run()
+    assert host.fake.fake_stray_pointers() == 0
