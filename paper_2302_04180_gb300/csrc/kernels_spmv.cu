@@ -141,6 +141,7 @@ cudaError_t launch_spmv(const CSRArgs &A, const double *x, double *y, const Solv
 
 cudaError_t launch_spmv_diag(const CSRArgs &A, const DiagArgs &D, const double *x, double *y, const SolverState *st,
                              unsigned *err, Cfg cfg, cudaStream_t s) {
+    spmv_carveout(cfg.carveout);
     const auto kern = (cfg.mode & SPMV_MODE_MASK) == SPMV_MODE_DIAG32 ? k_spmv_diag<32> : k_spmv_diag<7>;
     return launch_chained(kern, dim3((unsigned)cfg.grid), cfg.block, s, view(A), D, x, y, st, err, cfg.mode);
 }

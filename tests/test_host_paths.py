@@ -120,3 +120,23 @@ def test_stepped_batch_goes_on_without_room_for_the_layouts(host):
     host.fail = None
     run()
     assert host.fake.fake_stray_pointers() == 0
+
+
+def test_diagonal_product_runs_at_the_carveout_of_its_own_solve(host):
+    """smem.carveout changed and changed back between solves: the split that k_spmv_diag
+    runs at is the one its grid was sized for."""
+    A = gen.poisson3d(34)
+    before = host.rbs.rbs_get_param("smem.carveout")
+    try:
+        for c in (75, 0, 75, -1, 0):
+            host.rbs.rbs_set_param("smem.carveout", c)
+            _solve(host, A, variant=1)
+            seen = None
+            for call, what, n in host.events:
+                if call == "carveout" and "k_spmv_diagILi7E" in what:
+                    seen = n
+                if call == "launch" and "k_spmv_diagILi7E" in what:
+                    last = seen
+            assert last == c, (c, last)
+    finally:
+        host.rbs.rbs_set_param("smem.carveout", before)
