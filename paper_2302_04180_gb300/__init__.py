@@ -190,7 +190,9 @@ def _stream(stream, *tensors):
             global _raw_stream
             if _raw_stream is None:
                 import torch
-                _raw_stream = torch._C._cuda_getCurrentRawStream
+                # private to torch: the public way where a version has it not
+                _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (
+                    lambda index: torch.cuda.current_stream(index).cuda_stream)
             return _raw_stream(t.get_device())
     return None
 
