@@ -55,6 +55,7 @@ class DeviceArray:
         self.host, self.shape, self.dtype, self.nbytes = host, a.shape, a.dtype, a.nbytes
         self.p = C.c_void_p()
         assert host.fake.cudaMalloc(C.byref(self.p), C.c_size_t(a.nbytes)) == 0
+        host.fake.fake_data(self.p)
         C.memmove(self.p.value, a.ctypes.data, a.nbytes)
 
     def is_contiguous(self):
