@@ -253,7 +253,7 @@ def run_gpu(args):
     value = world * iters / (ms * 1e-3)
     clocks = clk.summary()
 
-    roofline = _roofline(A, prof_tot)
+    roofline = _roofline(A, prof_tot, diagonals=True)  # the 7-point stencil
 
     if not args.extras:
         line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world,
@@ -420,18 +420,19 @@ def _comparator(rbs, Ad, b, x, dev, reps=10):
     return out
 
 
-def _roofline(A, prof_tot):
+def _roofline(A, prof_tot, diagonals=False):
     """Roofline of the dominant kernel -- the SpMV with its exact-dot epilogue,
     classic K1 (<r0,s>) and K3 (<q,y>, <y,y>) -- from the library's CUDA events
     over the timed solves. Only launches that ran are counted (the library
     leaves out those that returned at once on the stop flag). Algorithmic bytes
-    per launch of a matrix of few diagonals: 8 nnz (val) + 4 n (row words) + n/4
-    (an int64 per 32 rows) + 8 n (x, ideal reuse) + 8 n (the companion vector of
-    the dot) + 8 n (output) = 8 nnz + 28.25 n; the CSR form's 12 nnz + 32 n + 8
-    (column indices, row pointers) is not read.
+    per launch: 12 nnz (col + val) + 8 (n+1) (rowptr) + 8 n (x, ideal reuse)
+    + 8 n (the companion vector of the dot) + 8 n (output) = 12 nnz + 32 n + 8.
+    diagonals: the matrix is one that solves lay out by its diagonals (stencils,
+    bands), where 4 n (row words) + n/4 (an int64 per 32 rows) take the place of the
+    column indices and row pointers: 8 nnz + 28.25 n.
     K4 (x and r updates with <r0,r>, <r,r>) moves 64 n bytes per launch."""
     hbm, peak_kind = _peaks()
-    alg = 8 * A.nnz + 28 * A.n + 8 * ((A.n + 31) // 32)
+    alg = 8 * A.nnz + 28 * A.n + 8 * ((A.n + 31) // 32) if diagonals else 12 * A.nnz + 32 * A.n + 8
     total_ms = max(sum(t[1] for t in prof_tot.values()), 1e-12)
 
     def stat(names, byt):
