@@ -1107,8 +1107,9 @@ int batch_stepped(Workspace *w, int32_t nsys, const rbs_system *systems, rbs_inf
     CK(cudaMemsetAsync(dscr, 0, (size_t)nsys * sizeof(DotScratch), w->stream));
     if (!tasks.empty())
         CK(cudaMemcpyAsync(dtask, tasks.data(), tasks.size() * sizeof(StepTask), cudaMemcpyHostToDevice, w->stream));
-    CK(step_admit(w->step_ctx.p, dtask, (int)ncls, RBS_CLASSIC, w->stream));
-    CK(step_admit(w->step_ctx.p, dtask + ncls, (int)(tasks.size() - ncls), RBS_PIPELINED, w->stream));
+    const bool room = std::any_of(layout.begin(), layout.end(), [](size_t bytes) { return bytes != 0; });
+    CK(step_admit(w->step_ctx.p, dtask, (int)ncls, RBS_CLASSIC, room, w->stream));
+    CK(step_admit(w->step_ctx.p, dtask + ncls, (int)(tasks.size() - ncls), RBS_PIPELINED, room, w->stream));
     CK(cudaMemcpyAsync(hst.data(), dst, (size_t)nsys * sizeof(SolverState), cudaMemcpyDeviceToHost, w->stream));
     std::vector<int32_t> diags((size_t)nsys, 0);
     CK(cudaMemcpy2DAsync(diags.data(), sizeof(int32_t), (const char *)w->step_ctx.p + step_ctx_diags_offset(), cb,

@@ -396,11 +396,11 @@ bool step_wants_layout(const CSRArgs &A) {
     return A.nnz > 0 && A.nnz <= STEP_DIAGS * A.n && ((uintptr_t)A.val & 15) == 0;
 }
 
-cudaError_t step_admit(void *ctxs, const StepTask *tasks, int ntasks, int variant, cudaStream_t s) {
+cudaError_t step_admit(void *ctxs, const StepTask *tasks, int ntasks, int variant, bool layouts, cudaStream_t s) {
     if (ntasks <= 0) return cudaSuccess;
     step_carveout();
     Ctx *c = static_cast<Ctx *>(ctxs);
-    k_step_sample<<<ntasks, 256, 0, s>>>(c, tasks);
+    if (layouts) k_step_sample<<<ntasks, 256, 0, s>>>(c, tasks);
     k_step_prepare<<<ntasks, 256, 0, s>>>(c, tasks);
     k_step_validate<<<(ntasks + 255) / 256, 256, 0, s>>>(c, tasks, ntasks);
     if (variant == RBS_CLASSIC) {

@@ -256,8 +256,9 @@ bool step_wants_layout(const CSRArgs &A);
 size_t step_ctx_diags_offset();
 // Admission of new systems (all of one variant): structure check and Jacobi,
 // then the set-up of Fig. 2 or Fig. 4; a system that fails its checks ends with
-// status RBS_EINVAL and its error bits in its scratch's err word.
-cudaError_t step_admit(void *ctxs, const StepTask *tasks, int ntasks, int variant, cudaStream_t s);
+// status RBS_EINVAL and its error bits in its scratch's err word. layouts: whether
+// any of them has room for a layout by diagonals.
+cudaError_t step_admit(void *ctxs, const StepTask *tasks, int ntasks, int variant, bool layouts, cudaStream_t s);
 // One iteration of every listed system (all of one variant, and with `diags` all
 // laid out by their diagonals); stopped systems skip it.
 cudaError_t step_iteration(const void *ctxs, const StepTask *tasks, int ntasks, int variant, bool diags,

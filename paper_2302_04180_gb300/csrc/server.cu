@@ -354,7 +354,7 @@ void Server::engine_loop() {
             for (int var = 0; var < 2 && ok; var++) {
                 cudaStream_t sv = var == RBS_CLASSIC ? st : side;
                 if (off[var + 1] > off[var])
-                    ok = step_admit(d_ctx, T + off[var], off[var + 1] - off[var], var, sv) == cudaSuccess;
+                    ok = step_admit(d_ctx, T + off[var], off[var + 1] - off[var], var, false, sv) == cudaSuccess;
                 if (ok && it_cnt[var] > 0)
                     ok = step_iteration(d_ctx, T + it_off[var], it_cnt[var], var, false, sv) == cudaSuccess;
             }

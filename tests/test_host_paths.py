@@ -140,3 +140,18 @@ def test_diagonal_product_runs_at_the_carveout_of_its_own_solve(host):
             assert last == c, (c, last)
     finally:
         host.rbs.rbs_set_param("smem.carveout", before)
+
+
+def test_server_admits_without_looking_for_layouts(host):
+    """A served system has no room for a layout by diagonals: its admission does not
+    launch the kernel that samples them; a stepped batch's does."""
+    A = gen.poisson3d(9)
+    srv = host.rbs.RbsServer(engines=1, max_active=4)
+    tickets = [srv.submit(_system(host, A, 3, v)) for v in (0, 1)]
+    for t in tickets:
+        assert srv.wait(t)["status"] == 0
+    srv.close()
+    assert [n for n in host.launched() if "k_step_prepare" in n]
+    assert not [n for n in host.launched() if "k_step_sample" in n]
+    host.rbs.rbs_solve_batched([_system(host, A, 2)], schedule={"cluster": 0, "split": 0})
+    assert [n for n in host.launched() if "k_step_sample" in n]
