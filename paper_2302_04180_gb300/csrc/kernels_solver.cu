@@ -442,11 +442,11 @@ cudaError_t solver_iteration(const SolverArgs &a, int variant, cudaStream_t s, K
     return iter_t<ExactR<1, SQ>, ExactR<2, SQ>, RowsR2, RowsR5>(a, variant, s, t);
 }
 
-// (a body holds one iteration or more, so maxit + 1 bodies are enough)
+// (a body holds one iteration or more, so maxit bodies are enough)
 __global__ void k_set_cond(cudaGraphConditionalHandle h, SolverState *st) {
     const int loops = st->loops + 1;
     st->loops = loops;
-    cudaGraphSetConditional(h, (!st->done && loops <= st->maxit + 1) ? 1u : 0u);
+    cudaGraphSetConditional(h, (!st->done && loops <= st->maxit) ? 1u : 0u);
 }
 
 cudaError_t launch_set_cond(cudaGraphConditionalHandle h, SolverState *st, cudaStream_t s) {

@@ -186,7 +186,7 @@ cudaError_t solver_setup(const SolverArgs &a, int variant, cudaStream_t s, Kerne
 cudaError_t solver_iteration(const SolverArgs &a, int variant, cudaStream_t s, KernelTimer *t);
 
 // Last node of the graph loop body: keeps the WHILE loop going while the stop
-// flag is clear, and at most maxit + 1 bodies in any case.
+// flag is clear, and at most maxit + 1 bodies in any case (maxit up to 2^31 - 1).
 cudaError_t launch_set_cond(cudaGraphConditionalHandle h, SolverState *st, cudaStream_t s);
 
 // ---- batched solver (kernels_batch.cu) ----
