@@ -415,30 +415,31 @@ cudaError_t step_admit(void *ctxs, const StepTask *tasks, int ntasks, int varian
 
 // Chained launches: 20 iterations of 12 systems 2.16 -> 1.88 ms, of 60 systems 6.05
 // -> 5.72; 512 systems take as long either way.
-template <bool DIAG>
-static void iteration_t(const Ctx *c, const StepTask *tasks, int ntasks, int variant, cudaStream_t s) {
-    const auto go = [&](auto kern) { launch_chained(kern, dim3((unsigned)ntasks), 256, s, c, tasks); };
-    if (variant == RBS_CLASSIC) {
-        go(DIAG ? k_step_diag_k1 : k_step_cls_k1);
-        go(k_step_cls_k2);
-        go(DIAG ? k_step_diag_k3 : k_step_cls_k3);
-        go(k_step_cls_k4<RowsR2>);
-        go(k_step_cls_k5);
-    } else {
-        go(k_step_pipe_p1<RowsR2>);
-        go(k_step_spmv<true, DIAG>);
-        go(k_step_pipe_p3<RowsR5>);
-        go(k_step_spmv<false, DIAG>);
-    }
-}
-
-cudaError_t step_iteration(const void *ctxs, const StepTask *tasks, int ntasks, int variant, bool diags,
-                           cudaStream_t s) {
-    if (ntasks <= 0) return cudaSuccess;
+cudaError_t step_iteration(const void *ctxs, const StepTask *tasks, int laid, int rest, int variant, cudaStream_t s) {
+    if (laid + rest <= 0) return cudaSuccess;
     step_carveout();
     const Ctx *c = static_cast<const Ctx *>(ctxs);
-    if (diags) iteration_t<true>(c, tasks, ntasks, variant, s);
-    else iteration_t<false>(c, tasks, ntasks, variant, s);
+    const auto go = [&](auto kern, const StepTask *t, int n) {
+        if (n > 0) launch_chained(kern, dim3((unsigned)n), 256, s, c, t);
+    };
+    // (a vector step is the same for both kinds: one launch)
+    const auto all = [&](auto kern) { go(kern, tasks, laid + rest); };
+    const auto product = [&](auto diag, auto general) {
+        go(diag, tasks, laid);
+        go(general, tasks + laid, rest);
+    };
+    if (variant == RBS_CLASSIC) {
+        product(k_step_diag_k1, k_step_cls_k1);
+        all(k_step_cls_k2);
+        product(k_step_diag_k3, k_step_cls_k3);
+        all(k_step_cls_k4<RowsR2>);
+        all(k_step_cls_k5);
+    } else {
+        all(k_step_pipe_p1<RowsR2>);
+        product(k_step_spmv<true, true>, k_step_spmv<true, false>);
+        all(k_step_pipe_p3<RowsR5>);
+        product(k_step_spmv<false, true>, k_step_spmv<false, false>);
+    }
     return cudaGetLastError();
 }
 

@@ -259,10 +259,10 @@ size_t step_ctx_diags_offset();
 // status RBS_EINVAL and its error bits in its scratch's err word. layouts: whether
 // any of them has room for a layout by diagonals.
 cudaError_t step_admit(void *ctxs, const StepTask *tasks, int ntasks, int variant, bool layouts, cudaStream_t s);
-// One iteration of every listed system (all of one variant, and with `diags` all
-// laid out by their diagonals); stopped systems skip it.
-cudaError_t step_iteration(const void *ctxs, const StepTask *tasks, int ntasks, int variant, bool diags,
-                           cudaStream_t s);
+// One iteration of every listed system, all of one variant: first the `laid` tasks
+// of systems laid out by their diagonals, whose products have launches of their
+// own, then `rest` tasks of others. Stopped systems skip it.
+cudaError_t step_iteration(const void *ctxs, const StepTask *tasks, int laid, int rest, int variant, cudaStream_t s);
 
 // occupancy-derived persistent grid for the kernels of one kind: which = 0 the
 // SpMV kernels (classic K1, pipelined S10/S18), 1 the vector kernels, 2 the

@@ -356,7 +356,7 @@ void Server::engine_loop() {
                 if (off[var + 1] > off[var])
                     ok = step_admit(d_ctx, T + off[var], off[var + 1] - off[var], var, false, sv) == cudaSuccess;
                 if (ok && it_cnt[var] > 0)
-                    ok = step_iteration(d_ctx, T + it_off[var], it_cnt[var], var, false, sv) == cudaSuccess;
+                    ok = step_iteration(d_ctx, T + it_off[var], 0, it_cnt[var], var, sv) == cudaSuccess;
             }
             if (pipe) {
                 ok = ok && cudaEventRecord(ev_join, side) == cudaSuccess &&
