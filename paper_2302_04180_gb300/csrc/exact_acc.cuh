@@ -10,10 +10,13 @@
 //    pos = e_x + e_y - 2, the accumulator's bit 0 weighing 2^-2148 (the lowest
 //    bit of a product of two subnormals). This is TwoProd's exact r + s, in
 //    integer form, with no underflow or overflow exception;
-//  * each thread adds its products into a 256-bit two's complement register
-//    window anchored at a 32-bit limb `a`; a product lands at limb offset
-//    q = (pos >> 5) - a in [0, Q) with a funnel shift and a log-shifter of
-//    word selects, then one 8-word add with carry;
+//  * each thread adds its products into a window of 32-bit words anchored at a
+//    limb `a`. Two forms: here a 256-bit two's complement window in registers
+//    (SpMV kernels on general rows, set-up, batches, small solves), where a
+//    product lands at limb offset q = (pos >> 5) - a in [0, Q) with a funnel shift
+//    and a log-shifter of word selects, then one 8-word add with carry; and rows
+//    in shared memory, picked by address (ExactRows, reduce.cuh: the standalone
+//    dots, the vector kernels, SpMV kernels on few diagonals);
 //  * products above the window flush it and re-anchor it; products below it
 //    are added straight into the block's shared-memory long accumulator
 //    (RBS_LIMBS signed 64-bit limbs, limb j weighing 2^(32 j - 2148), carry-save
@@ -84,38 +87,28 @@ __device__ __forceinline__ void shift5(uint32_t p0, uint32_t p1, uint32_t p2, ui
 // two's complement negation.
 template <int Q, bool SIGNED>
 __device__ __forceinline__ void win_place_add(Win<Q> &W, const uint32_t (&u)[5], int q, uint32_t m) {
+    static_assert(Q == 4, "two levels of selects");
     uint32_t x[5], v[8];
 #pragma unroll
     for (int k = 0; k < 5; k++) x[k] = SIGNED ? (u[k] ^ m) : u[k];
     const uint32_t f = SIGNED ? m : 0u;
-    if (Q == 1) {
-        v[0] = x[0]; v[1] = x[1]; v[2] = x[2]; v[3] = x[3]; v[4] = x[4];
-        v[5] = f; v[6] = f; v[7] = f;
-    } else {
-        const bool b1 = (q & 1) != 0;
-        uint32_t t[6];
-        t[0] = b1 ? f : x[0];
-        t[1] = b1 ? x[0] : x[1];
-        t[2] = b1 ? x[1] : x[2];
-        t[3] = b1 ? x[2] : x[3];
-        t[4] = b1 ? x[3] : x[4];
-        t[5] = b1 ? x[4] : f;
-        if (Q == 2) {
-#pragma unroll
-            for (int k = 0; k < 6; k++) v[k] = t[k];
-            v[6] = f; v[7] = f;
-        } else {
-            const bool b2 = (q & 2) != 0;
-            v[0] = b2 ? f : t[0];
-            v[1] = b2 ? f : t[1];
-            v[2] = b2 ? t[0] : t[2];
-            v[3] = b2 ? t[1] : t[3];
-            v[4] = b2 ? t[2] : t[4];
-            v[5] = b2 ? t[3] : t[5];
-            v[6] = b2 ? t[4] : f;
-            v[7] = b2 ? t[5] : f;
-        }
-    }
+    const bool b1 = (q & 1) != 0;
+    uint32_t t[6];
+    t[0] = b1 ? f : x[0];
+    t[1] = b1 ? x[0] : x[1];
+    t[2] = b1 ? x[1] : x[2];
+    t[3] = b1 ? x[2] : x[3];
+    t[4] = b1 ? x[3] : x[4];
+    t[5] = b1 ? x[4] : f;
+    const bool b2 = (q & 2) != 0;
+    v[0] = b2 ? f : t[0];
+    v[1] = b2 ? f : t[1];
+    v[2] = b2 ? t[0] : t[2];
+    v[3] = b2 ? t[1] : t[3];
+    v[4] = b2 ? t[2] : t[4];
+    v[5] = b2 ? t[3] : t[5];
+    v[6] = b2 ? t[4] : f;
+    v[7] = b2 ? t[5] : f;
     add8_carry(W.w, v, SIGNED ? (m & 1u) : 0u);
 }
 
@@ -229,17 +222,17 @@ __device__ __forceinline__ void exact_add(Win<Q> &W, uint32_t &flags, unsigned l
     }
     if (W.a < 0 || q >= Q) {
         // empty, or above the window: flush and re-anchor with the product at
-        // offset Q-2 (or 0), leaving room for somewhat larger products. Lanes that
+        // offset Q-2, leaving room for somewhat larger products. Lanes that
         // open their windows together take one anchor where their products are
         // within two limbs, for the sake of warp_flush (COMMON; the persistent batch
         // kernel, full of windows, loses 2 % to the extra code and goes without).
         int top = L;
         if (COMMON && W.a < 0) {
             const int m = (int)__reduce_max_sync(__activemask(), (unsigned)L);
-            if (m - L <= (Q >= 2 ? Q - 2 : 0)) top = m;
+            if (m - L <= Q - 2) top = m;
         }
         win_flush<Q>(W, sacc);
-        int a = top - (Q >= 2 ? Q - 2 : 0);
+        int a = top - (Q - 2);
         a = a < 0 ? 0 : a;
         W.a = a;
         win_place_add<Q, !SQUARE>(W, u, L - a, m);
@@ -617,15 +610,13 @@ __device__ __forceinline__ bool block_grid_finish(const uint32_t (&flags)[K], un
 template <int K, int Q, int SCRATCH = FLUSH_SCRATCH, int WARPS = MAX_WARPS>
 __device__ __forceinline__ bool exact_finish(Win<Q> (&win)[K], uint32_t (&flags)[K],
                                              unsigned long long (*sacc)[NL], uint32_t *sflags,
-                                             DotScratch *g, double *vals, bool export_limbs = false,
-                                             long long *limbs_out = nullptr, int32_t *flags_out = nullptr,
-                                             unsigned nblk = 0u, bool coop = true) {
+                                             DotScratch *g, double *vals, unsigned nblk = 0u, bool coop = true) {
 #pragma unroll
     for (int k = 0; k < K; k++) {
         if (coop) warp_flush<Q, SCRATCH, WARPS>(win[k], sacc[k]);
         else win_flush<Q>(win[k], sacc[k]);
     }
-    return block_grid_finish<K>(flags, sacc, sflags, g, vals, export_limbs, limbs_out, flags_out, nblk);
+    return block_grid_finish<K>(flags, sacc, sflags, g, vals, false, nullptr, nullptr, nblk);
 }
 
 }  // namespace rbs

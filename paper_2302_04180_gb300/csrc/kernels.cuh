@@ -72,9 +72,9 @@ constexpr unsigned ERR_TIMEOUT = 4u;
 // the flush reuses the same shared buffer.
 // Staging layout of one chunk buffer for spans of at most CAP nonzeros: the
 // z slice (32 doubles), then val (CAP + 2 for the 16-byte rounding), then col
-// (CAP + 8); two buffers per warp. CAP 224 holds 32 rows of a 7-point stencil
-// (three 256-thread blocks per SM); CAP 1024 holds 32 rows of up to 32
-// nonzeros, e.g. the 27-point stencil (one block per SM).
+// (CAP + 8). CAP 224 holds 32 rows of a 7-point stencil: two buffers per warp, three
+// 256-thread blocks per SM. CAP 1024 holds 32 rows of up to 32 nonzeros, e.g. the
+// 27-point stencil: one buffer per warp (spmv_rows_reg).
 template <int CAP>
 struct SpmvLayout {
     static constexpr int VAL_OFF = 32 * 8;

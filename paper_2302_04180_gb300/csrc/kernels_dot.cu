@@ -115,8 +115,8 @@ __global__ void __launch_bounds__(256, EXDOT_BLOCKS)
 }
 
 // Words per sign for the "exdot.window" knob: 16 unless it asks for a small
-// window (1 or 2). 12 placements hold the products of 2^-128 .. 2^128 and more
-// around a block's first ones without re-anchoring.
+// window (1 or 2). 12 placements hold the products from 2^-256 below to 2^96 above
+// the largest of a block's first ones without re-anchoring.
 template <class F>
 static auto with_window(int window, F &&f) {
     if (window == 1) return f(k_exdot<6, false>);

@@ -8,18 +8,18 @@
 
 namespace rbs {
 
-// y = A x (Sec. 4.1), warp-staged rows (mode 0) or one thread per row (mode
-// 1) in a grid-stride loop. CHECKED: every index is range-checked (the
+// y = A x (Sec. 4.1), warp-staged short rows or, in mode 1, one thread per row
+// in a grid-stride loop. CHECKED: every index is range-checked (the
 // standalone product); without it the solver has validated the structure at
 // set-up. With a solver state, the kernel is a no-op once the solver stopped.
-template <bool CHECKED, int CAP>
+template <bool CHECKED>
 __global__ void __launch_bounds__(256, 3)
     k_spmv(CSRView A, const double *__restrict__ x, double *__restrict__ y, const SolverState *st, unsigned *err,
            int mode) {
     chain_wait();
     if (st && st->done) return;
     unsigned eb = 0u;
-    spmv_each<CHECKED, CAP>(A, x, nullptr, mode, eb, [&](int64_t i, double v, double) { y[i] = v; });
+    spmv_each<CHECKED, SPMV_CAP_SHORT>(A, x, nullptr, mode, eb, [&](int64_t i, double v, double) { y[i] = v; });
     if (eb) atomicOr(err, eb);
 }
 
@@ -65,8 +65,8 @@ static void spmv_carveout(int c) {
     int dev = 0;
     if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 && applied[dev] != c) {
         const int short_c = c > SPMV_SHORT_CARVEOUT ? SPMV_SHORT_CARVEOUT : c;
-        cudaFuncSetAttribute(k_spmv<true, SPMV_CAP_SHORT>, cudaFuncAttributePreferredSharedMemoryCarveout, short_c);
-        cudaFuncSetAttribute(k_spmv<false, SPMV_CAP_SHORT>, cudaFuncAttributePreferredSharedMemoryCarveout, short_c);
+        cudaFuncSetAttribute(k_spmv<true>, cudaFuncAttributePreferredSharedMemoryCarveout, short_c);
+        cudaFuncSetAttribute(k_spmv<false>, cudaFuncAttributePreferredSharedMemoryCarveout, short_c);
         cudaFuncSetAttribute(k_spmv_diag<7>, cudaFuncAttributePreferredSharedMemoryCarveout, c);
         // the kernels of long rows: what their blocks need, whatever the knob says
         cudaFuncSetAttribute(k_spmv_diag<32>, cudaFuncAttributePreferredSharedMemoryCarveout, -1);
@@ -89,7 +89,7 @@ int spmv_blocks_per_sm(int block, int carveout, int mode) {
             : mode == SPMV_MODE_DIAG32 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_spmv_diag<32>, block, 0)
             : mode == SPMV_MODE_LONG
                 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_spmv_reg<true>, SPMV_REG_WARPS * 32, 0)
-                : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_spmv<true, SPMV_CAP_SHORT>, block, 0);
+                : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_spmv<true>, block, 0);
         if (e != cudaSuccess || nb < 1) {
             cudaGetLastError();
             nb = 1;
@@ -135,7 +135,7 @@ cudaError_t launch_spmv(const CSRArgs &A, const double *x, double *y, const Solv
         return launch_chained(st ? k_spmv_reg<false> : k_spmv_reg<true>, dim3((unsigned)r.grid), r.block, s, view(A), x,
                               y, st, err, cfg.mode);
     }
-    return launch_chained(st ? k_spmv<false, SPMV_CAP_SHORT> : k_spmv<true, SPMV_CAP_SHORT>, dim3((unsigned)cfg.grid),
+    return launch_chained(st ? k_spmv<false> : k_spmv<true>, dim3((unsigned)cfg.grid),
                           cfg.block, s, view(A), x, y, st, err, cfg.mode);
 }
 

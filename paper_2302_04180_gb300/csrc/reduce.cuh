@@ -43,8 +43,7 @@ struct ExactR {
     // coop = false after a timed-out staged copy (ERR_TIMEOUT): per-lane flushes
     template <int SCRATCH = FLUSH_SCRATCH, int WARPS = MAX_WARPS>
     __device__ __forceinline__ bool finish(DotScratch *g, double *vals, unsigned nblk = 0u, bool coop = true) {
-        return exact_finish<K, Q, SCRATCH, WARPS>(win, flags, sacc, sflags, g, vals, false, nullptr, nullptr, nblk,
-                                                  coop);
+        return exact_finish<K, Q, SCRATCH, WARPS>(win, flags, sacc, sflags, g, vals, nblk, coop);
     }
 };
 
