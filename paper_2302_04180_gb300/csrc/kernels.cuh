@@ -643,7 +643,8 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const uint32_t 
     // its first gathers and companion; xn, zn get the next one's (G = 1). Returns
     // false when the wait for the values ran out.
     auto step = [&](int b, double (&xc)[PER], double (&xn)[PER], double &zc, double &zn) {
-        const int row = w0.c * 32 + lane, row1 = chunks.row(w1.c, n, lane);  // (w0.c < c_end)
+        const int row = w0.c * 32 + lane;  // (w0.c < c_end)
+        const unsigned row1 = chunks.row(w1.c, lane);
         if (w1.c < c_end) stage(h1, b ^ 1);
         const Walk w2 = chunks.next(w1);
         const Head h2 = head(w2.c);
@@ -662,8 +663,8 @@ __device__ __forceinline__ void spmv_rows_diag(const CSRView &A, const uint32_t 
         }
         const double *val = reinterpret_cast<const double *>(bufs + b * L::BUF) + ((int)(h0.base & 1) + at);
         auto next_gather = [&](double (&xv)[PER], double &zv) {
-            gather(row1, h1.word, 0, xv);
-            if (z && row1 < n) zv = __ldca(z + row1);
+            gather((int)row1, h1.word, 0, xv);
+            if (z && row1 < (unsigned)n) zv = __ldca(z + row1);
         };
         if (G == 1) next_gather(xn, zn);
         {

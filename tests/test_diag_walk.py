@@ -1,7 +1,7 @@
 """Index arithmetic of the diagonal product (csrc/diag_walk.h), compiled for the CPU
 with overflow checks: every chunk of 32 rows is taken by exactly one warp, whatever
 the grid, tiles and number of chunks (whole rounds, none, and several of them), and
-a chunk past the end has no row, also where 32 times its number leaves 32 bits."""
+a chunk past the end has no row below n, also where 32 times its number leaves an int."""
 import os
 import subprocess
 
@@ -37,7 +37,7 @@ template <int T> static void edge(int64_t n, int begin, int nblk, int nw) {
             for (int past = 0; past < 3; past += w.c >= end, w = d.next(w))
                 for (int lane : {0, 31}) {
                     const int64_t want = (int64_t)w.c * 32 + lane;
-                    const int got = d.row(w.c, (int)n, lane);
+                    const unsigned got = d.row(w.c, lane);
                     fails += w.c < end ? got != want : got < n;
                 }
         }
