@@ -14,9 +14,8 @@ struct DotArgs {
 };
 
 // Pairs of each operand that a thread loads at once, and blocks per SM to keep
-// registers for. The loads in flight set the rate: two pairs at three blocks
-// (80 registers) stream 2^27 products in 331 us, one pair at four blocks in 334,
-// two at four in 346 (64 registers spill).
+// registers for. The loads in flight set the rate: two pairs at three blocks (80
+// registers; one pair at four blocks, or two at four, were up to 5 % slower).
 constexpr int EXDOT_PAIRS = 2, EXDOT_BLOCKS = 3;
 
 // U pairs into the windows. WARP: every lane of the warp has them.
@@ -41,11 +40,12 @@ __device__ __forceinline__ void add_pairs(R &red, const double2 (&x)[U], const d
 //
 // Several dots share the launch but not their blocks: five dots' windows in one
 // thread left two blocks per SM, and issue slots empty (2 million elements: 41
-// us against 30 now); an operand that several dots name comes from L2 for all
+// us against 29 now); an operand that several dots name comes from L2 for all
 // but the first of them, since their blocks walk the vectors together.
-// Bound by HBM once long (2^27: 328 us, 0.965 of the copy rate, cond 1; 378 with
-// 64-bit digits) and by the windows' set-up, flush and cross-block sum when
-// short (2^24: 49 us, 39.5 of them HBM's; cond 1e48: 54 against 73).
+// Bound by HBM once long (2^27, cond 1: 311 us, the copy rate; 378 with 64-bit
+// digits), with the integer pipe where signs and exponents mix (cond 1e16 to 1e48: 347
+// us), and by the windows' set-up, flush and cross-block sum when short (2^24: 44 us,
+// 39.5 of them HBM's; cond 1e48: 50 against 73).
 template <int W, bool EXPORT>
 __global__ void __launch_bounds__(256, EXDOT_BLOCKS)
     k_exdot(const __grid_constant__ DotArgs a, int64_t n, DotScratch *g, double *out, long long *limbs, int32_t *flags_out) {
@@ -71,8 +71,10 @@ __global__ void __launch_bounds__(256, EXDOT_BLOCKS)
         // copies of the code for the last steps (a short dot meets every copy cold:
         // with three more 2^20 took 8.1 us on the device, 7.8 so), and the pairs left
         // over at the end (taken first, values that rise along the vectors would all
-        // fall below their windows)
-        const int64_t full = n2 > st ? (n2 - st) / (U * st) : 0;
+        // fall below their windows). A thread has at most 2^20 products: counted in 32
+        // bits, whose registers the loads in flight can use (2^27, cond 1e16: 372 -> 365
+        // us; with the operands' exponents tested one by one 347).
+        const int full = n2 > st ? (int)((n2 - st) / (U * st)) : 0;
         double2 xa[U], ya[U], xb[U], yb[U];
         const double2 *xq = x2 + gtid() + st, *yq = y2 + gtid() + st;
         auto load = [&](double2 (&xv)[U], double2 (&yv)[U]) {
@@ -87,7 +89,7 @@ __global__ void __launch_bounds__(256, EXDOT_BLOCKS)
         if (full > 0) load(xa, ya);
         red.open({max(R::limb_of(x0[0].x, y0[0].x), R::limb_of(x0[0].y, y0[0].y))});
         add_pairs<1, false>(red, x0, y0);
-        for (int64_t s = 0; s < full; s += 2) {
+        for (int s = 0; s < full; s += 2) {
             if (s + 1 < full) load(xb, yb);
             add_pairs<U, true>(red, xa, ya);
             if (s + 1 >= full) break;

@@ -165,7 +165,7 @@ struct ExactRows {
     template <class... D>
     static __device__ __noinline__ int add_any(uint32_t *w, unsigned long long *sk, uint32_t *fl, int a, D... v) {
         // (SPLIT: one copy of the code, the products moving up in turn. Unrolled, the
-        // call took registers that the caller's loads in flight need: 2^27 325 us, 313 so)
+        // call took registers that the caller's loads in flight need)
         constexpr int AHEAD = SPLIT ? 1 : 8;
         double xy[] = {v...};
 #pragma unroll AHEAD
@@ -222,7 +222,7 @@ struct ExactRows {
     // WARP: all 32 lanes call it and take the branch together if one of them has to.
     // Lanes that went out of line while the others ran the straight code cost the
     // warp both: 2^24 products of which one in a hundred lies 2^400 below the rest
-    // 205 us, 102 so; exponents of -200 .. 200 331, 145.
+    // 205 us, 98 so; exponents of -200 .. 200 331, 146.
     template <int N, bool SQ = false, bool WARP = false>
     __device__ __forceinline__ void add(int k, const double (&x)[N], const double (&y)[N]) {
         uint32_t xh[N], yh[N], e[N], q[N];
@@ -231,20 +231,19 @@ struct ExactRows {
         if constexpr (SPLIT) {
             // e: bit position above the window's lowest << 20, modulo 2^32, which holds
             // every position: one subtraction for the placement, the shift and the test
-            uint32_t lowest = 0x7ff00000u, highest = 0u, far = 0u;
+            uint32_t odd = 0u, far = 0u;
             const uint32_t base = ((uint32_t)a[k] << 25) + (2u << 20);
 #pragma unroll
             for (int i = 0; i < N; i++) {
                 xh[i] = (uint32_t)__double2hiint(x[i]);
                 yh[i] = (uint32_t)__double2hiint(y[i]);
                 const uint32_t ex = xh[i] & 0x7ff00000u, ey = yh[i] & 0x7ff00000u;
-                lowest = min(lowest, min(ex, ey));
-                highest = max(highest, max(ex, ey));
+                odd = max(max(odd, ex - 0x00100000u), ey - 0x00100000u);
                 e[i] = ex + ey - base;
                 q[i] = e[i] >> 25;
                 far = max(far, e[i]);
             }
-            plain = lowest != 0u && highest < 0x7ff00000u && far < (QMAX + 1u) << 25;
+            plain = odd < 0x7fe00000u && far < (QMAX + 1u) << 25;
         } else {
             uint32_t odd = 0u, far = 0u;
 #pragma unroll
