@@ -70,8 +70,8 @@ struct ExactR {
 // window update used to be five 64-bit carry-save digits, whose loads and
 // stores alone took 0.63 of them; 32-bit words take 0.31, and one add each
 // instead of two. One branch per four products and two middle terms summed as
-// 64 bits bring a product to 62 instructions from 90 (2^24 products, cond 1e48:
-// 54 us from 73).
+// 64 bits bring a product to some 64 instructions from 90 (2^24 products, cond
+// 1e48: 50 us from 73).
 //
 // A window covers W - 4 placements. Where a kernel has every thread's first
 // products before it adds any, all threads of a block start with one anchor
