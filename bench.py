@@ -662,6 +662,7 @@ def _c1(rbs, gen, dev, reps=30):
     b = rbs.rbs_spmv_csr(Ad, torch.ones(A.n, dtype=torch.float64, device=dev))
     x = torch.empty(A.n, dtype=torch.float64, device=dev)
     out = {}
+    # (the default driver solves a system this small by one cluster in one launch)
     for name, loop in (("graph_loop", 0), ("host_loop", 1)):
         for _ in range(3):
             r = rbs.rbs_solve(Ad, b, tol=1e-8, maxit=1000, x_out=x, loop_mode=loop, history=False)

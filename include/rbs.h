@@ -158,8 +158,11 @@ int rbs_jacobi_apply(int64_t n, const double *invd, const double *p, double *pha
 #define RBS_DOT_PLAIN 1 /* comparator: binary64 dots with atomic accumulation,
                            run-to-run non-reproducible (the paper's "original") */
 
-#define RBS_LOOP_GRAPH 0 /* the loop runs on the device: one iteration is the body of a
-                            CUDA-graph conditional WHILE node (no host round trips) */
+#define RBS_LOOP_GRAPH 0 /* the loop runs on the device, no host round trips: up to four
+                            iterations are the body of a CUDA-graph conditional WHILE node
+                            (few iterations on arguments not seen before are enqueued
+                            without one); a system that fits the shared memory of one
+                            thread-block cluster is solved in one launch */
 #define RBS_LOOP_HOST 1  /* the host enqueues iterations in chunks and reads the stop flag */
 
 typedef struct {

@@ -144,7 +144,7 @@ constexpr unsigned ERR_DIAGS = 16u;
 // A row of more than LONG_ROW nonzeros sets ERR_LONG, is not looked into and has no
 // layout: launch_csr_check and launch_jacobi_invd then do the whole set-up, the
 // check with the nonzeros spread over the grid. (One thread took 13.8 ms for one
-// dense row of 200000, they take 0.09; 256 nonzeros take it 16 us.)
+// dense row of 200000, they take 0.09.)
 constexpr unsigned ERR_LONG = 32u;
 constexpr int LONG_ROW = 256;
 cudaError_t launch_prepare(const CSRArgs &A, const double *diag, double *invd, DiagArgs *diags, uint32_t *mask,

@@ -50,9 +50,9 @@ def test_same_bits_as_alone(rbs, dev, orc, sides):
 
 def test_few_rows_of_each_kind_share_their_launches(rbs, dev):
     """Four systems of 27000 rows on 7 diagonals, four of 20000 on none and four of 30000 on
-    19. Measured for 8 iterations: 0.95 ms (1.21 with the kinds apart); the first kind
-    alone 0.53, the others 0.85. The bound is half way between 0.95 and 1.21 over the
-    longer of the two alone."""
+    19. Measured for 8 iterations: 0.93 ms (1.22 with the kinds apart); the first kind
+    alone 0.54, the others 0.81. The bound is the geometric mean of 0.93 and 1.22 over
+    the longer of the two alone."""
     import time
     import torch
     laid = _systems(rbs, dev, [gen.poisson3d(30)] * 2, 8)
@@ -68,4 +68,4 @@ def test_few_rows_of_each_kind_share_their_launches(rbs, dev):
         return sorted(best)[8]
     one, other, both = ms(laid), ms(rest), ms(laid + rest)
     print(f"{one:.3f} {other:.3f} {both:.3f}")
-    assert both < 1.27 * max(one, other), (one, other, both)
+    assert both < 1.31 * max(one, other), (one, other, both)
